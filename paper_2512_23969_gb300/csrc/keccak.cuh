@@ -8,12 +8,22 @@
 // bswap(word 2i) as its low half and bswap(word 2i+1) as its high half.
 //
 // GB300 mapping: the 25 lanes are 50 32-bit registers; every 64-bit XOR,
-// AND-NOT and rotation is two 32-bit LOP3 / funnel shifts on the ALU pipe
-// (~190 ALU ops per round).  The 24 rounds run in a rolled loop (the round
-// body is the same each time; only the round constant changes), keeping the
-// code of each call site small.  The rotation offsets, the lane permutation
-// and the round constants are derived at compile time from FIPS 202's
-// definitions (Sec. 3.2.2 - 3.2.5), not written out.
+// AND-NOT and rotation is two 32-bit LOP3 / funnel shifts on the ALU pipe,
+// which bounds every SHAKE kernel (it measured 99.8 % busy), so the rounds
+// are written for the fewest ALU operations: 180 per round.
+//  * theta never forms D[x] = C[x-1] ^ rot(C[x+1], 1): each lane takes both
+//    terms in one three-input XOR, 10 operations a round less.
+//  * A one-block hash (shake_thash1) peels its first round, where most
+//    lanes are compile-time zeros, and its last, of which only the output
+//    lanes are computed (keccak_f1600_hash): 22 rounds in the loop.
+// Measured on GB300, TREE_Sign of 1024 shake-128f messages: 25.60 ms with D
+// formed and all 24 rounds in the loop, 23.99 without D, 23.29 with the last
+// round peeled, 23.06 with the first too; FORS_Sign of 4096: 6.07 -> 5.47 ms.
+// The rounds stay in a rolled loop: two rounds per iteration measured the
+// same (23.04 ms), all of them unrolled 31.3 ms (instruction fetch).  The
+// rotation offsets, the lane permutation and the round constants are
+// derived at compile time from FIPS 202's definitions (Sec. 3.2.2 - 3.2.5),
+// not written out.
 #pragma once
 #include <cstdint>
 #include "sha2.cuh"
@@ -80,12 +90,67 @@ __device__ __forceinline__ void rotl(uint32_t lo, uint32_t hi, uint32_t& olo, ui
     }
 }
 
-template <int L>
-__device__ __forceinline__ void rho_pi_lane(const uint32_t* alo, const uint32_t* ahi, const uint32_t* dlo,
-                                            const uint32_t* dhi, uint32_t* blo, uint32_t* bhi) {
+__device__ __forceinline__ uint32_t xor3(uint32_t a, uint32_t b, uint32_t c) {
+    uint32_t r;
+    asm("lop3.b32 %0, %1, %2, %3, 0x96;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
+    return r;
+}
+
+// Column parities C[x] and their rotations R[x] = rot(C[x + 1], 1); theta
+// adds C[x - 1] ^ R[x] to every lane of column x.
+__device__ __forceinline__ void theta_columns(const uint32_t* lo, const uint32_t* hi, uint32_t* clo, uint32_t* chi,
+                                              uint32_t* rlo, uint32_t* rhi) {
+#pragma unroll
+    for (int x = 0; x < 5; x++) {
+        clo[x] = xor3(xor3(lo[x], lo[x + 5], lo[x + 10]), lo[x + 15], lo[x + 20]);
+        chi[x] = xor3(xor3(hi[x], hi[x + 5], hi[x + 10]), hi[x + 15], hi[x + 20]);
+    }
+#pragma unroll
+    for (int x = 0; x < 5; x++) rotl<1>(clo[(x + 1) % 5], chi[(x + 1) % 5], rlo[x], rhi[x]);
+}
+
+// Lanes L .. END - 1 after theta, rho and pi.
+template <int L, int END>
+__device__ __forceinline__ void rho_pi_lanes(const uint32_t* alo, const uint32_t* ahi, const uint32_t* clo,
+                                             const uint32_t* chi, const uint32_t* rlo, const uint32_t* rhi,
+                                             uint32_t* blo, uint32_t* bhi) {
     constexpr int S = pi_source(L);
-    rotl<rho_offset(S)>(alo[S] ^ dlo[S % 5], ahi[S] ^ dhi[S % 5], blo[L], bhi[L]);
-    if constexpr (L + 1 < 25) rho_pi_lane<L + 1>(alo, ahi, dlo, dhi, blo, bhi);
+    rotl<rho_offset(S)>(xor3(alo[S], clo[(S + 4) % 5], rlo[S % 5]), xor3(ahi[S], chi[(S + 4) % 5], rhi[S % 5]),
+                        blo[L], bhi[L]);
+    if constexpr (L + 1 < END) rho_pi_lanes<L + 1, END>(alo, ahi, clo, chi, rlo, rhi, blo, bhi);
+}
+
+__device__ __forceinline__ void round(uint32_t lo[25], uint32_t hi[25], uint32_t rc_lo, uint32_t rc_hi) {
+    uint32_t clo[5], chi[5], rlo[5], rhi[5], blo[25], bhi[25];
+    theta_columns(lo, hi, clo, chi, rlo, rhi);
+    rho_pi_lanes<0, 25>(lo, hi, clo, chi, rlo, rhi, blo, bhi);
+#pragma unroll
+    for (int y = 0; y < 5; y++)
+#pragma unroll
+        for (int x = 0; x < 5; x++) {
+            lo[x + 5 * y] = blo[x + 5 * y] ^ (~blo[(x + 1) % 5 + 5 * y] & blo[(x + 2) % 5 + 5 * y]);
+            hi[x + 5 * y] = bhi[x + 5 * y] ^ (~bhi[(x + 1) % 5 + 5 * y] & bhi[(x + 2) % 5 + 5 * y]);
+        }
+    lo[0] ^= rc_lo;
+    hi[0] ^= rc_hi;
+}
+
+// The last round, output lanes 0 .. OL - 1 only (the others are left as
+// they were): chi of lane x needs lanes x .. x + 2 of its row.
+template <int OL>
+__device__ __forceinline__ void last_round(uint32_t lo[25], uint32_t hi[25]) {
+    static_assert(OL >= 1 && OL <= 5, "lanes of the first row");
+    constexpr uint64_t rc = round_constant(23);
+    uint32_t clo[5], chi[5], rlo[5], rhi[5], blo[5], bhi[5];
+    theta_columns(lo, hi, clo, chi, rlo, rhi);
+    rho_pi_lanes<0, (OL + 2 < 5 ? OL + 2 : 5)>(lo, hi, clo, chi, rlo, rhi, blo, bhi);
+#pragma unroll
+    for (int x = 0; x < OL; x++) {
+        lo[x] = blo[x] ^ (~blo[(x + 1) % 5] & blo[(x + 2) % 5]);
+        hi[x] = bhi[x] ^ (~bhi[(x + 1) % 5] & bhi[(x + 2) % 5]);
+    }
+    lo[0] ^= (uint32_t)rc;
+    hi[0] ^= (uint32_t)(rc >> 32);
 }
 
 }  // namespace kk
@@ -93,32 +158,18 @@ __device__ __forceinline__ void rho_pi_lane(const uint32_t* alo, const uint32_t*
 // Keccak-f[1600] on lanes A[x + 5y] = (hi[i]:lo[i]).
 __device__ __forceinline__ void keccak_f1600(uint32_t lo[25], uint32_t hi[25]) {
 #pragma unroll 1
-    for (int ir = 0; ir < 24; ir++) {
-        uint32_t clo[5], chi[5], dlo[5], dhi[5];
-#pragma unroll
-        for (int x = 0; x < 5; x++) {
-            clo[x] = lo[x] ^ lo[x + 5] ^ lo[x + 10] ^ lo[x + 15] ^ lo[x + 20];
-            chi[x] = hi[x] ^ hi[x + 5] ^ hi[x + 10] ^ hi[x + 15] ^ hi[x + 20];
-        }
-#pragma unroll
-        for (int x = 0; x < 5; x++) {
-            uint32_t rlo, rhi;
-            kk::rotl<1>(clo[(x + 1) % 5], chi[(x + 1) % 5], rlo, rhi);
-            dlo[x] = clo[(x + 4) % 5] ^ rlo;
-            dhi[x] = chi[(x + 4) % 5] ^ rhi;
-        }
-        uint32_t blo[25], bhi[25];
-        kk::rho_pi_lane<0>(lo, hi, dlo, dhi, blo, bhi);
-#pragma unroll
-        for (int y = 0; y < 5; y++)
-#pragma unroll
-            for (int x = 0; x < 5; x++) {
-                lo[x + 5 * y] = blo[x + 5 * y] ^ (~blo[(x + 1) % 5 + 5 * y] & blo[(x + 2) % 5 + 5 * y]);
-                hi[x + 5 * y] = bhi[x + 5 * y] ^ (~bhi[(x + 1) % 5 + 5 * y] & bhi[(x + 2) % 5 + 5 * y]);
-            }
-        lo[0] ^= kk::kRC.lo[ir];
-        hi[0] ^= kk::kRC.hi[ir];
-    }
+    for (int ir = 0; ir < 24; ir++) kk::round(lo, hi, kk::kRC.lo[ir], kk::kRC.hi[ir]);
+}
+
+// The same permutation where only lanes 0 .. OL - 1 of the result are read
+// and the input has constant lanes the first round can fold.
+template <int OL>
+__device__ __forceinline__ void keccak_f1600_hash(uint32_t lo[25], uint32_t hi[25]) {
+    constexpr uint64_t rc0 = kk::round_constant(0);
+    kk::round(lo, hi, (uint32_t)rc0, (uint32_t)(rc0 >> 32));
+#pragma unroll 1
+    for (int ir = 1; ir < 23; ir++) kk::round(lo, hi, kk::kRC.lo[ir], kk::kRC.hi[ir]);
+    kk::last_round<OL>(lo, hi);
 }
 
 // The full 32-byte ADRS (eight big-endian words) from the compressed form
@@ -158,7 +209,7 @@ __device__ __forceinline__ void shake_thash1(const uint32_t* seed, const Adrs& a
     }
     lo[T / 2] ^= 0x1Fu;            // domain bits 1111 and the first pad bit
     hi[16] ^= 0x80000000u;         // last pad bit: byte 135
-    keccak_f1600(lo, hi);
+    keccak_f1600_hash<NW / 2>(lo, hi);
 #pragma unroll
     for (int i = 0; i < NW; i += 2) {
         out[i] = bswap32(lo[i / 2]);
