@@ -40,9 +40,15 @@ struct TuneSlots {
 TuneSlots g_slots;
 auto& g_tune = g_slots.v;
 std::atomic<int> g_ck_default{2};
-// Default batch size below which TREE_Sign runs chain-parallel, per set.
-constexpr int kSplitDefault[kNumSets] = {8192, 2048, 4096, 0, 64, 64, 64, 8192, 2048, 4096, 64, 64, 64,
-                                         8192, 2048, 4096};
+// TREE_Sign's form without a tuned cache, per set, as the tuner measured it
+// on GB300: the batch size below which it runs chain-parallel, and above
+// that the cost model's coefficients (split_faster below).
+constexpr int kSplitDefault[kNumSets] = {2048, 1024, 64, 0, 16, 16, 0, 16384, 16384, 16384, 256, 256, 256,
+                                         16384, 16384, 16384};
+constexpr int kStepUsDefault[kNumSets] = {637, 958, 1262, 0, 655, 1015, 1300, 2379, 3510, 4615, 2414, 3534, 4635,
+                                          2379, 3606, 6405};
+constexpr int kSplitNsDefault[kNumSets] = {5741, 9833, 22514, 0, 116992, 197938, 167196, 20966, 30673, 62918,
+                                           425882, 626482, 473714, 11576, 17815, 54806};
 constexpr int kStrides[] = {0, 1, 2, 4, 8};
 // Default batch size below which the message stage runs a warp per message
 // (SHA-2 sets; the SHAKE sets always run a thread per message).
@@ -63,7 +69,9 @@ int tune_get(int pset, int knob) {
     case 4: return 1;
     case 5: return g_ck_default.load();
     case 8: return kMsgWarpDefault[pset];
-    default: return 0;                  // 6, 7: no cost model
+    case 6: return kStepUsDefault[pset];
+    case 7: return kSplitNsDefault[pset];
+    default: return 0;
     }
 }
 
@@ -85,7 +93,7 @@ int tune_options(int pset, int knob, int32_t* values, int max) {
     switch (knob) {
     case 0: for (int i = 0; i < o->n_fors_lpt; i++) buf[n++] = o->fors_lpt[i]; break;
     case 1: for (int i = 0; i < o->n_tree_minb; i++) buf[n++] = o->tree_minb[i]; break;
-    case 2: for (int v : {0, 256, 512, 1024, 2048, 4096, 8192}) buf[n++] = v; break;   // suggestions: any value works
+    case 2: for (int v : {0, 16, 64, 256, 512, 1024, 2048, 4096, 8192, 16384}) buf[n++] = v; break;   // suggestions: any value works
     case 3: for (int v : {7, 15}) if (o->tree_has(0, v, 1)) buf[n++] = v; break;
     case 4: for (int v : {1, 2}) if (o->tree_has(0, o->tree_pol_default, v)) buf[n++] = v; break;
     case 5: for (int v : kStrides) buf[n++] = v; break;
@@ -93,29 +101,43 @@ int tune_options(int pset, int knob, int32_t* values, int max) {
         if (is_shake(pset)) buf[n++] = 0;
         else for (int v : {0, 64, 256, 512, 1024, 4096}) buf[n++] = v;
         break;
-    default: buf[n++] = 0; break;       // 6, 7: measured coefficients, any value >= 0
+    default:                            // 6, 7: measured coefficients, any value >= 0
+        buf[n++] = 0;
+        if (const int d = knob == 6 ? kStepUsDefault[pset] : kSplitNsDefault[pset]) buf[n++] = d;
+        break;
     }
     for (int i = 0; i < n && i < max; i++)
         if (values) values[i] = buf[i];
     return n;
 }
 
+// The two forms of building XMSS trees.  A thread per leaf: the time is a
+// staircase -- one warp per SM sub-partition already keeps the ALU pipe
+// busy, so it takes about step_us x ceil(warps / sub-partitions).
+// Chain-parallel: it grows with the trees (split_ns per message's d trees).
+// True if the second is predicted faster.
+static bool split_faster(int pset, const SetShape& sh, uint64_t trees, uint64_t max_steps) {
+    const int step_us = tune_get(pset, 6), split_ns = tune_get(pset, 7);
+    if (step_us <= 0 || split_ns <= 0) return false;
+    const uint64_t warps = (trees * sh.leaves + 31) / 32, smsp = 4ull * (uint64_t)sm_count();
+    const uint64_t steps = (warps + smsp - 1) / smsp;
+    if (steps > max_steps) return false;
+    return (uint64_t)split_ns * trees / sh.d < (uint64_t)step_us * 1000ull * steps;
+}
+
 bool tree_split(int pset, uint32_t count) {
     const int below = tune_get(pset, 2);
     if (below > 0 && count < (uint32_t)below) return true;
-    // Above the threshold, the per-leaf form's time is a staircase: one
-    // warp per SM sub-partition already keeps the ALU pipe busy, so it
-    // takes about step_us x ceil(warps / sub-partitions), while the
-    // chain-parallel form's time grows with the batch (split_ns per
-    // message).  Within the first few steps, where a batch just past a step
-    // wastes most of its last one, take the form predicted faster.
-    const int step_us = tune_get(pset, 6), split_ns = tune_get(pset, 7);
+    // Above the threshold: within the first few steps, where a batch just
+    // past a step wastes most of its last one, take the form predicted faster.
     SetShape sh{};
-    if (step_us <= 0 || split_ns <= 0 || !set_shape(pset, &sh)) return false;
-    const uint64_t warps = ((uint64_t)count * sh.d * sh.leaves + 31) / 32, smsp = 4ull * (uint64_t)sm_count();
-    const uint64_t steps = (warps + smsp - 1) / smsp;
-    if (steps > 4) return false;
-    return (uint64_t)split_ns * count < (uint64_t)step_us * 1000ull * steps;
+    return set_shape(pset, &sh) && split_faster(pset, sh, (uint64_t)count * sh.d, 4);
+}
+
+// Key generation builds one tree per key.
+bool keygen_split(int pset, uint32_t count) {
+    SetShape sh{};
+    return set_shape(pset, &sh) && split_faster(pset, sh, count, 4);
 }
 
 bool msg_warp(int pset, uint32_t count) {
@@ -200,17 +222,10 @@ cudaError_t launch_fors_pk(const Batch& b, cudaStream_t s) {
 cudaError_t launch_tree(const Batch& b, cudaStream_t s) {
     const SetOps* o = set_ops(b.pset);
     if (!o) return cudaErrorInvalidValue;
-    if (b.cached) {                       // prebuilt upper layers of a keyset
-        cudaError_t e = o->tree_cached(b, s);
-        if (e != cudaSuccess) return e;
-    } else if (b.dedup_layer) {           // shared upper layers first
-        cudaError_t e = cudaMemsetAsync(b.table, 0, sizeof(unsigned long long) << b.cap_log2, s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(b.nuniq, 0, sizeof(uint32_t), s);
-        if (e == cudaSuccess) e = o->tree_dedup(b, s);
-        if (e != cudaSuccess) return e;
-    }
-    return b.split ? o->tree_split(b, s)
-                   : o->tree(b, tune_get(b.pset, 1), tune_get(b.pset, 3), tune_get(b.pset, 4), s);
+    cudaError_t e = b.split ? o->tree_split(b, s)
+                            : o->tree(b, tune_get(b.pset, 1), tune_get(b.pset, 3), tune_get(b.pset, 4), s);
+    if (e == cudaSuccess && b.dedup_layer) e = o->tree_shared(b, s);     // the shared layers' auth paths and roots
+    return e;
 }
 cudaError_t launch_wots(const Batch& b, cudaStream_t s) {
     const SetOps* o = set_ops(b.pset);
@@ -223,7 +238,7 @@ cudaError_t launch_verify(const Batch& b, cudaStream_t s) {
 cudaError_t launch_keygen(int pset, const uint8_t* seeds, uint32_t count, uint8_t* pk, uint8_t* sk,
                           cudaStream_t s) {
     const SetOps* o = set_ops(pset);
-    return o ? o->keygen(seeds, count, pk, sk, s) : cudaErrorInvalidValue;
+    return o ? o->keygen(seeds, count, pk, sk, keygen_split(pset, count), s) : cudaErrorInvalidValue;
 }
 
 }  // namespace hs

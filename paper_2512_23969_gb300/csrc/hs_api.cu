@@ -5,6 +5,7 @@
 // are independent given the digest, WOTS+_Sign consumes both).
 #include <cuda_runtime.h>
 #include <algorithm>
+#include <atomic>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -79,40 +80,40 @@ bool set_shape(int pset, SetShape* out) {
     return true;
 }
 
-// Tree sharing within a batch (process-wide switch, off by default).
-static bool g_share = false;
+// Tree sharing within a batch (process-wide switch).
+static std::atomic<bool> g_share{true};
+
+void drop_dedup(Batch& b) {
+    b.dedup_layer = 0;
+    b.cache_tpk = 0;
+    b.max_uniq = 0;
+}
 
 void plan_dedup(Batch& b) {
-    b.dedup_layer = 0;
-    b.cap_log2 = 0;
-    b.max_uniq = 0;
+    drop_dedup(b);
     SetInfo s{};
-    if (!g_share || !set_info(b.pset, &s) || b.num_keys > (1u << 20) || b.count == 0) return;
-    // Share layers from the top down while the number of distinct trees a
-    // layer can hold (keys x 2^bits of its tree index, at most one per
-    // message) is at most half the messages, and the tree index fits the
-    // 27 bits of the table key.
+    if (!g_share.load() || !set_info(b.pset, &s) || b.count == 0) return;
+    // Share layers from the top down while all the trees a layer can hold
+    // (keys x 2^bits of its tree index) are at most half the messages: at
+    // the line, half the trees are saved and nearly all of those built (86 %
+    // for random indices) are used, so none is built in vain to speak of;
+    // the next layer down holds 2^h' >= 8 times as many.
+    uint64_t tpk = 0;
     uint32_t L = (uint32_t)s.d;
-    uint64_t total = 0;
     for (int j = s.d - 1; j >= 1; j--) {
-        const int bits = s.tree_bits - j * s.hp > 0 ? s.tree_bits - j * s.hp : 0;
-        if (bits > 27) break;
-        const uint64_t u = std::min<uint64_t>(b.count, (uint64_t)b.num_keys << bits);
-        if (2 * u > b.count) break;
+        const int bits = (s.d - 1 - j) * s.hp;
+        if (bits > 31 || 2 * ((uint64_t)b.num_keys << bits) > b.count) break;
         L = (uint32_t)j;
-        total += u;
+        tpk += 1ull << bits;
     }
     if (L == (uint32_t)s.d) return;
-    const uint64_t entries = (uint64_t)b.count * (s.d - L);
-    uint32_t lg = 4;
-    while ((1ull << lg) < 2 * entries) lg++;
     b.dedup_layer = L;
-    b.cap_log2 = lg;
-    b.max_uniq = (uint32_t)total;
+    b.cache_tpk = (uint32_t)tpk;
+    b.max_uniq = (uint32_t)(tpk * b.num_keys);
 }
 
 // Every scratch region of a batch, in carve order (256-byte aligned each).
-static constexpr int kRegions = 18;
+static constexpr int kRegions = 14;
 static void scratch_layout(const Batch& b, const SetInfo& s, size_t sz[kRegions], int* n) {
     const size_t nw = (size_t)s.n / 4, cnt = b.count;
     int i = 0;
@@ -124,17 +125,11 @@ static void scratch_layout(const Batch& b, const SetInfo& s, size_t sz[kRegions]
     sz[i++] = cnt * nw * 4;                                          // pk_fors
     sz[i++] = cnt * s.d * nw * 4;                                    // roots
     sz[i++] = b.ck ? cnt * s.d * s.len * (16 / b.ck) * nw * 4 : 0;   // chk
+    const size_t own = b.dedup_layer ? b.dedup_layer : (size_t)s.d;  // layers built per message
+    const size_t mu = b.cached ? 0 : b.max_uniq;                     // trees built for several
     sz[i++] = b.verify ? cnt * s.len * nw * 4                        // ends (one layer when verifying)
-                       : (b.split ? cnt * s.d * s.leaves * s.len * nw * 4 : 0);
-    const bool sh = b.dedup_layer != 0 && !b.cached;                 // in-batch sharing
-    const size_t mj = b.dedup_layer ? cnt * (s.d - b.dedup_layer) : 0;
-    const size_t cap = sh ? ((size_t)1 << b.cap_log2) : 0;
-    sz[i++] = cap * sizeof(unsigned long long);                      // table
-    sz[i++] = sh ? mj * 4 : 0;                                       // mj_slot
-    sz[i++] = mj * 4;                                                // mj_id
-    sz[i++] = cap * 4;                                               // slot_id
-    sz[i++] = sh ? sizeof(uint32_t) : 0;                             // nuniq
-    const size_t mu = sh ? b.max_uniq : 0;
+                       : (b.split ? (cnt * own + mu) * s.leaves * s.len * nw * 4 : 0);
+    sz[i++] = b.dedup_layer ? cnt * (s.d - b.dedup_layer) * 4 : 0;   // mj_id
     sz[i++] = mu * sizeof(DedupDesc);                                // desc
     sz[i++] = mu * 2 * s.leaves * nw * 4 +                           // nodes_u, then chk_u
               (b.ck ? mu * s.leaves * s.len * (16 / b.ck) * nw * 4 : 0);
@@ -182,20 +177,15 @@ void carve_scratch(Batch& b, void* base) {
     b.roots = reinterpret_cast<uint32_t*>(r[6]);
     b.chk = b.ck ? reinterpret_cast<uint32_t*>(r[7]) : nullptr;
     b.ends = (b.split || b.verify) ? reinterpret_cast<uint32_t*>(r[8]) : nullptr;
-    b.leafv = s.leaves > 32 ? reinterpret_cast<uint32_t*>(r[16]) : nullptr;
-    b.vcnt = b.verify ? reinterpret_cast<uint32_t*>(r[17]) : nullptr;
+    b.leafv = s.leaves > 32 ? reinterpret_cast<uint32_t*>(r[12]) : nullptr;
+    b.vcnt = b.verify ? reinterpret_cast<uint32_t*>(r[13]) : nullptr;
     b.vsitem = b.verify ? b.vcnt + 16 * s.d : nullptr;
     b.vorder = b.verify ? b.vsitem + (size_t)b.count * s.len : nullptr;
-    const bool sh = b.dedup_layer != 0 && !b.cached;
-    b.table = sh ? reinterpret_cast<unsigned long long*>(r[9]) : nullptr;
-    b.mj_slot = sh ? reinterpret_cast<uint32_t*>(r[10]) : nullptr;
-    b.mj_id = b.dedup_layer ? reinterpret_cast<uint32_t*>(r[11]) : nullptr;
-    b.slot_id = sh ? reinterpret_cast<uint32_t*>(r[12]) : nullptr;
-    b.nuniq = sh ? reinterpret_cast<uint32_t*>(r[13]) : nullptr;
-    b.desc = sh ? reinterpret_cast<DedupDesc*>(r[14]) : nullptr;
+    b.mj_id = b.dedup_layer ? reinterpret_cast<uint32_t*>(r[9]) : nullptr;
     if (b.cached) return;             // nodes_u / chk_u belong to the keyset
-    b.nodes_u = sh ? reinterpret_cast<uint32_t*>(r[15]) : nullptr;
-    b.chk_u = (sh && b.ck) ? b.nodes_u + (size_t)b.max_uniq * 2 * s.leaves * (s.n / 4) : nullptr;
+    b.desc = b.max_uniq ? reinterpret_cast<DedupDesc*>(r[10]) : nullptr;
+    b.nodes_u = b.max_uniq ? reinterpret_cast<uint32_t*>(r[11]) : nullptr;
+    b.chk_u = (b.max_uniq && b.ck) ? b.nodes_u + (size_t)b.max_uniq * 2 * s.leaves * (s.n / 4) : nullptr;
 }
 
 // ----------------------------------------------------------- device state
@@ -346,7 +336,7 @@ HS_API hs_status hs_set_host_direct(int on) {
 }
 
 HS_API hs_status hs_set_tree_sharing(int on) {
-    g_share = on != 0;
+    g_share.store(on != 0);
     return HS_OK;
 }
 
@@ -502,14 +492,25 @@ static hs_status run_batch(const hs_keyset* ks, bool verify, hs_params p, const 
     } else if (!verify) {
         plan_dedup(b);
     }
-    if (ks) b.num_keys = 0;                       // no key blocks in scratch: they are resident
-    const size_t scratch = scratch_bytes(b);
-    b.num_keys = num_keys;
+    // scratch: no key blocks with a keyset, they are resident
+    auto need = [&] {
+        b.num_keys = ks ? 0 : num_keys;
+        const size_t n = scratch_bytes(b);
+        b.num_keys = num_keys;
+        return n;
+    };
+    size_t scratch = need();
     const size_t stage = (h_keys ? align256(key_bytes) : 0) + (h_idx ? align256((size_t)count * 4) : 0) +
                          (h_lens ? align256((size_t)count * 8) : 0) + (h_msgs ? align256(msg_total) : 0) +
                          (h_sig ? align256(sig_total) : 0) + (h_ok ? align256(count) : 0) + align256(plen);
     void* base = nullptr;
     e = cudaMallocFromPoolAsync(&base, scratch + stage, d->pool, s);
+    if (e == cudaErrorMemoryAllocation && b.max_uniq) {      // the shared trees are extra scratch: without them
+        cudaGetLastError();
+        drop_dedup(b);
+        scratch = need();
+        e = cudaMallocFromPoolAsync(&base, scratch + stage, d->pool, s);
+    }
     if (e != cudaSuccess) return cuda_fail(e, "cudaMallocFromPoolAsync(scratch)");
     carve_scratch(b, base);
     if (ks) {

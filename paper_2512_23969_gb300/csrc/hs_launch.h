@@ -10,7 +10,7 @@
 
 namespace hs {
 
-// A distinct XMSS tree of a batch (tree sharing, kern_dedup.cuh).
+// An XMSS tree built for several messages or as a key's root (kern_dedup.cuh).
 struct DedupDesc {
     uint64_t tree;
     uint32_t key;
@@ -43,25 +43,20 @@ struct Batch {
     uint32_t* chk;            // WOTS chain checkpoints: count * D * LEN * (16 / ck) * NW words
     uint32_t ck;              // checkpoint stride (1, 2, 4) or 0 = none
     bool split;               // TREE_Sign in its chain-parallel form (small batches)
-    uint32_t* ends;           // chain ends of the split form: count * D * 2^h' * LEN * NW words
+    uint32_t* ends;           // chain ends of the split form: LEN * NW words per leaf, own trees then shared
     uint32_t* leafv;          // wide trees (2^h' > 32): leaves, count * D * 2^h' * NW words
-    // tree sharing within the batch: layers dedup_layer .. D-1 are shared
-    // (dedup_layer == 0: off, every message builds all its layers)
+    // shared layers dedup_layer .. D-1 (dedup_layer == 0: none, every message
+    // builds all its layers): their trees are built once per (key, layer,
+    // tree), all max_uniq = num_keys * cache_tpk of them, with every node and
+    // the checkpoints of every leaf, and each message copies its auth paths
     uint32_t dedup_layer;
-    uint32_t cap_log2;        // hash table of 2^cap_log2 slots
-    uint32_t max_uniq;        // bound on the distinct trees
-    unsigned long long* table;
-    uint32_t* mj_slot;        // count * (D - L)
-    uint32_t* mj_id;          // count * (D - L)
-    uint32_t* slot_id;        // 2^cap_log2
-    uint32_t* nuniq;
+    uint32_t cache_tpk;       // shared trees per key
+    uint32_t max_uniq;        // shared trees built by this call (0 when cached)
+    uint32_t* mj_id;          // count * (D - L): the tree of each (message, shared layer)
     DedupDesc* desc;          // max_uniq
-    uint32_t* nodes_u;        // max_uniq * 2 * 2^h' * NW words
-    uint32_t* chk_u;          // max_uniq * 2^h' * LEN * (16 / ck) * NW words
-    // keyset cache: layers dedup_layer .. D-1 come prebuilt from nodes_u /
-    // chk_u (owned by the keyset), tree ids computed directly (no table)
-    bool cached;
-    uint32_t cache_tpk;       // cached trees per key
+    uint32_t* nodes_u;        // 2 * 2^h' * NW words per tree
+    uint32_t* chk_u;          // 2^h' * LEN * (16 / ck) * NW words per tree
+    bool cached;              // the trees come prebuilt from a keyset, which owns nodes_u / chk_u
     // FIPS 205 mode: FORS indices MSB first; prefix bytes hashed before
     // every message (0x00 || len(ctx) || ctx for pure signing; none = 0)
     bool fips;
@@ -86,9 +81,10 @@ uint32_t* device_status_word_if_ready();
 cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s);
 uint32_t chain_checkpoint_stride(int pset);
 
-// Tree sharing plan of a batch: fills dedup_layer, cap_log2 and max_uniq
-// (dedup_layer = 0 when sharing is off or not worth it).
+// Tree sharing plan of a batch: fills dedup_layer, cache_tpk and max_uniq
+// (all 0 when sharing is off or not worth it).
 void plan_dedup(Batch& b);
+void drop_dedup(Batch& b);    // back to every message's own trees
 size_t scratch_bytes(const Batch& b);
 
 // Scratch bytes for a batch (each region 256-byte aligned).
@@ -111,13 +107,12 @@ struct SetOps {
     cudaError_t (*tree)(const Batch&, int, int, int, cudaStream_t);
     bool (*tree_has)(int, int, int);
     cudaError_t (*tree_split)(const Batch&, cudaStream_t);
-    cudaError_t (*tree_dedup)(const Batch&, cudaStream_t);
-    cudaError_t (*tree_cached)(const Batch&, cudaStream_t);
+    cudaError_t (*tree_shared)(const Batch&, cudaStream_t);
     cudaError_t (*cache_build)(const KeyBlock*, uint32_t, uint32_t, uint32_t, DedupDesc*, uint32_t*, uint32_t*,
                                uint32_t, cudaStream_t);
     cudaError_t (*wots)(const Batch&, cudaStream_t);
     cudaError_t (*verify)(const Batch&, cudaStream_t);
-    cudaError_t (*keygen)(const uint8_t*, uint32_t, uint8_t*, uint8_t*, cudaStream_t);
+    cudaError_t (*keygen)(const uint8_t*, uint32_t, uint8_t*, uint8_t*, bool, cudaStream_t);
     const int* fors_lpt;
     int n_fors_lpt;
     int fors_lpt_default;
@@ -152,6 +147,7 @@ int tune_options(int pset, int knob, int32_t* values, int max);
 // Process-wide checkpoint stride: the value of every set whose knob 5 is unset.
 void set_default_checkpoint(uint32_t stride);
 bool tree_split(int pset, uint32_t count);
+bool keygen_split(int pset, uint32_t count);    // the same choice for key generation's trees
 // Whether a batch's message stage runs a warp per message (knob 8).
 bool msg_warp(int pset, uint32_t count);
 // SM count of the current device (cached per device).

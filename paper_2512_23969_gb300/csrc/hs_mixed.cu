@@ -212,17 +212,32 @@ HS_API hs_status hs_sign_mixed(const hs_sign_job* jobs, uint32_t njobs, int use_
     if (!status) return mx_fail(HS_ECUDA, "hs_sign_mixed: device state unavailable");
     std::lock_guard<std::mutex> lk(d->mu);
     void* base = nullptr;
-    cudaError_t e = cudaSuccess;
-    if (use_graph && total > d->gcap) {       // grow the graph's fixed scratch
-        if (d->gdone_valid) cudaEventSynchronize(d->gdone);
+    auto reserve = [&]() -> cudaError_t {
+        if (!use_graph) return pool_alloc(&base, total, s);
+        if (total <= d->gcap) return cudaSuccess;
+        if (d->gdone_valid) cudaEventSynchronize(d->gdone);   // grow the graph's fixed scratch
         cudaFree(d->gscratch);
         d->gscratch = nullptr;
         d->gcap = 0;
         d->last_bs.clear();                   // the old graph points into the old buffer
-        e = cudaMalloc(&d->gscratch, total);
-        if (e == cudaSuccess) d->gcap = total;
-    } else if (!use_graph) {
-        e = pool_alloc(&base, total, s);
+        const cudaError_t ea = cudaMalloc(&d->gscratch, total);
+        if (ea == cudaSuccess) d->gcap = total;
+        return ea;
+    };
+    cudaError_t e = reserve();
+    if (e == cudaErrorMemoryAllocation) {     // the shared trees are extra scratch: without them
+        bool any = false;
+        total = 0;
+        for (size_t j = 0; j < bs.size(); j++) {
+            any = any || bs[j].max_uniq != 0;
+            drop_dedup(bs[j]);
+            off[j] = total;
+            total += scratch_bytes(bs[j]);
+        }
+        if (any) {
+            cudaGetLastError();
+            e = reserve();
+        }
     }
     if (e != cudaSuccess) {
         cudaGetLastError();                  // consumed here: reported by the status below

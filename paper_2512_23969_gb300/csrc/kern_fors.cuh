@@ -19,6 +19,7 @@
 #include "hs_common.cuh"
 #include "hs_launch.h"
 #include "sha256_chain.cuh"
+#include "kern_tl.cuh"
 
 namespace hs {
 
@@ -238,30 +239,25 @@ __global__ void __launch_bounds__(256) fors_kernel(const KeyBlock* __restrict__ 
     }
 }
 
-// PK_FORS = T_k(FORS_ROOTS(layer 0, idx_tree, keypair idx_leaf), roots).
+// PK_FORS = T_k(FORS_ROOTS(layer 0, idx_tree, keypair idx_leaf), roots), 32
+// messages per block (kern_tl.cuh).
 template <class P>
-__global__ void fors_pk_kernel(const KeyBlock* __restrict__ keys, const MsgInfo* __restrict__ infos,
-                               uint32_t count, const uint32_t* __restrict__ fors_roots,
-                               uint32_t* __restrict__ pk_fors) {
-    const uint32_t m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= count) return;
-    const MsgInfo& info = infos[m];
-    if (info.key == KEY_INVALID) return;
-    const KeyBlock& kb = keys[info.key];
+__global__ void __launch_bounds__(TlShape<P>::THREADS) fors_pk_kernel(const KeyBlock* __restrict__ keys,
+                                                                      const MsgInfo* __restrict__ infos,
+                                                                      uint32_t count,
+                                                                      uint32_t* __restrict__ fors_roots,
+                                                                      uint32_t* __restrict__ pk_fors) {
     constexpr int NW = P::NW;
-    const uint32_t* r = fors_roots + (size_t)m * P::K * NW;
-    const Adrs a = make_adrs(0, info.idx_tree, T_FORS_ROOTS, info.idx_leaf, 0, 0);
+    __shared__ __align__(16) uint32_t smem[TlShape<P>::SMEM_WORDS];
+    const uint32_t m = blockIdx.x * 32 + (threadIdx.x & 31);
+    const uint32_t key = m < count ? infos[m].key : KEY_INVALID;
+    const bool active = key != KEY_INVALID;
+    const MsgInfo& info = infos[active ? m : 0];
+    const KeyBlock& kb = keys[active ? key : 0];
     uint32_t out[NW];
-    if constexpr (P::SHAKE) {
-        TStreamP<P> ts;
-        ts.init(kb.ms256, a);
-        for (int i = 0; i < P::K; i++) ts.template push_n<NW>(r + i * NW);
-        ts.template finish<NW>(P::K * P::N, out);
-    } else {
-        // robust: mask this message's roots in place (scratch, read once)
-        if constexpr (P::ROBUST) mask_mem<P::BIG, NW, P::K * NW>(kb.pk_seed, a, const_cast<uint32_t*>(r));
-        tl_from_mem<P::BIG, P::K * NW, NW>(P::BIG ? kb.ms512 : kb.ms256, a, r, out);
-    }
+    tl_group<P, P::K>(P::BIG ? kb.ms512 : kb.ms256, make_adrs(0, info.idx_tree, T_FORS_ROOTS, info.idx_leaf, 0, 0),
+                      fors_roots + (size_t)m * P::K * NW, active, kb.pk_seed, smem, out);
+    if (threadIdx.x >= 32 || !active) return;
 #pragma unroll
     for (int w = 0; w < NW; w++) pk_fors[(size_t)m * NW + w] = out[w];
 }

@@ -59,37 +59,49 @@ __global__ void __launch_bounds__(128, MINB) bleaf_kernel(const KeyBlock* __rest
 }
 
 // Chain-parallel form, second half: T_len over the len chain ends that
-// chains_kernel wrote for each leaf.
+// chains_kernel wrote for each leaf, 32 leaves per block (kern_tl.cuh); the
+// blocks behind the messages' own leaves take the trees of desc, whose
+// leaves go to nodes_u.
 template <class P>
-__global__ void __launch_bounds__(128) bleaf_from_ends_kernel(const KeyBlock* __restrict__ keys,
-                                                              const MsgInfo* __restrict__ infos, uint32_t count,
-                                                              const uint32_t* __restrict__ ends,
-                                                              uint32_t* __restrict__ leafv, uint32_t layers) {
+__global__ void __launch_bounds__(TlShape<P>::THREADS) bleaf_from_ends_kernel(const KeyBlock* __restrict__ keys,
+                                                                              const MsgInfo* __restrict__ infos,
+                                                                              uint32_t count,
+                                                                              uint32_t* __restrict__ ends,
+                                                                              uint32_t* __restrict__ leafv,
+                                                                              uint32_t layers,
+                                                                              const DedupDesc* __restrict__ desc,
+                                                                              uint32_t ndesc,
+                                                                              uint32_t* __restrict__ nodes_u) {
     constexpr int NW = P::NW, LV = P::LEAVES, LEN = P::LEN;
-    const uint64_t gid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    static_assert(LV % 32 == 0, "a block is 32 leaves of one tree");
+    __shared__ __align__(16) uint32_t smem[TlShape<P>::SMEM_WORDS];
+    const uint64_t gid = (uint64_t)blockIdx.x * 32 + (threadIdx.x & 31);
     const uint32_t per_msg = layers * LV;
-    const uint64_t m = gid / per_msg;
-    const uint32_t r = (uint32_t)(gid % per_msg);
-    const uint32_t j = r / LV;
-    const uint32_t l = r % LV;
-    if (m >= count) return;
-    const MsgInfo& info = infos[m];
-    if (info.key == KEY_INVALID) return;
-    const KeyBlock& kb = keys[info.key];
-    const uint64_t tree = layer_tree<P>(info.idx_tree, (int)j);
-    const uint32_t* e = ends + (size_t)gid * LEN * NW;
-    uint32_t node[NW];
-    if constexpr (P::SHAKE) {
-        TStreamP<P> ts;
-        ts.init(kb.ms256, make_adrs(j, tree, T_WOTS_PK, l, 0, 0));
-#pragma unroll 1
-        for (int i = 0; i < LEN; i++) ts.template push_n<NW>(e + i * NW);
-        ts.template finish<NW>(LEN * P::N, node);
+    const uint64_t own = (uint64_t)count * per_msg;
+    const uint32_t l = (uint32_t)(gid % LV);
+    uint32_t key, j;
+    uint64_t tree;
+    uint32_t* out;
+    if (gid < own) {                                // block-uniform, as are the exits below
+        const uint64_t m = gid / per_msg;
+        j = (uint32_t)(gid % per_msg) / LV;
+        key = infos[m].key;
+        if (key == KEY_INVALID) return;
+        tree = layer_tree<P>(infos[m].idx_tree, (int)j);
+        out = leafv + (((size_t)m * P::D + j) * LV + l) * NW;
     } else {
-        tl_from_mem<P::BIG, LEN * NW, NW>(P::BIG ? kb.ms512 : kb.ms256, make_adrs(j, tree, T_WOTS_PK, l, 0, 0), e,
-                                          node);
+        const uint64_t id = (gid - own) / LV;
+        if (id >= ndesc) return;
+        key = desc[id].key;
+        j = desc[id].layer;
+        tree = desc[id].tree;
+        out = nodes_u + ((size_t)id * 2 * LV + LV + l) * NW;
     }
-    uint32_t* out = leafv + (((size_t)m * P::D + j) * LV + l) * NW;
+    const KeyBlock& kb = keys[key];
+    uint32_t node[NW];
+    tl_group<P, LEN>(P::BIG ? kb.ms512 : kb.ms256, make_adrs(j, tree, T_WOTS_PK, l, 0, 0),
+                     ends + (size_t)gid * LEN * NW, true, kb.pk_seed, smem, node);
+    if (threadIdx.x >= 32) return;
 #pragma unroll
     for (int w = 0; w < NW; w++) out[w] = node[w];
 }
@@ -166,21 +178,20 @@ __global__ void __launch_bounds__(kMergeThreads) bmerkle_kernel(const KeyBlock* 
 }
 
 // ---------------------------------------------------------------- shared / cached trees
-// Distinct trees (tree sharing within a batch, keyset caches) for wide
+// Trees built for several messages (within a batch, keyset caches) for wide
 // trees: one thread per (tree, leaf) for the leaves, with the chain
 // checkpoints of every leaf, stored heap-ordered; then one block per tree
-// for the internal nodes.  nuniq (may be null) bounds the live trees.
+// for the internal nodes.
 template <class P, int POL>
 __global__ void __launch_bounds__(128) wtree_leaf_kernel(const KeyBlock* __restrict__ keys,
-                                                         const DedupDesc* __restrict__ desc,
-                                                         const uint32_t* __restrict__ nuniq, uint32_t max_uniq,
+                                                         const DedupDesc* __restrict__ desc, uint32_t ndesc,
                                                          uint32_t* __restrict__ nodes, uint32_t* __restrict__ chk_u,
                                                          uint32_t ck, uint32_t one) {
     constexpr int NW = P::NW, LV = P::LEAVES;
     const uint64_t gid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const uint64_t id = gid / LV;
     const uint32_t l = (uint32_t)(gid % LV);
-    if (id >= max_uniq || (nuniq && id >= *nuniq)) return;
+    if (id >= ndesc) return;
     const DedupDesc d = desc[id];
     const KeyBlock& kb = keys[d.key];
     uint32_t ms256[8], msT[P::BIG ? 16 : 8], skseed[NW];
@@ -202,12 +213,11 @@ __global__ void __launch_bounds__(128) wtree_leaf_kernel(const KeyBlock* __restr
 template <class P>
 __global__ void __launch_bounds__(kMergeThreads) wtree_merge_kernel(const KeyBlock* __restrict__ keys,
                                                                     const DedupDesc* __restrict__ desc,
-                                                                    const uint32_t* __restrict__ nuniq,
-                                                                    uint32_t max_uniq, uint32_t* __restrict__ nodes) {
+                                                                    uint32_t ndesc, uint32_t* __restrict__ nodes) {
     constexpr int NW = P::NW, LV = P::LEAVES;
     __shared__ uint32_t sh[LV * NW];
     const uint32_t id = blockIdx.x;
-    if (id >= max_uniq || (nuniq && id >= *nuniq)) return;      // block-uniform
+    if (id >= ndesc) return;                                    // block-uniform
     const DedupDesc d = desc[id];
     const KeyBlock& kb = keys[d.key];
     uint32_t ms256[8], msT[P::BIG ? 16 : 8];

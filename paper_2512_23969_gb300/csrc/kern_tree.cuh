@@ -23,6 +23,7 @@
 #include "hs_common.cuh"
 #include "hs_launch.h"
 #include "sha256_chain.cuh"
+#include "kern_tl.cuh"
 
 namespace hs {
 
@@ -206,6 +207,33 @@ __device__ __forceinline__ void merkle_finish(const uint32_t* ms256, const uint3
 }
 
 
+// The same levels of a tree built for several messages: every node stored
+// heap-ordered in tn (node (z, i) at (2^h' >> z) + i; root at 1).
+template <class P>
+__device__ __forceinline__ void heap_finish(const uint32_t* ms256, const uint32_t* msT, unsigned gmask,
+                                            uint32_t layer, uint64_t tree, uint32_t l, uint32_t* node,
+                                            uint32_t* __restrict__ tn, const uint32_t* pks) {
+    constexpr int NW = P::NW, HP = P::HP, LV = P::LEAVES;
+#pragma unroll
+    for (int w = 0; w < NW; w++) tn[(LV + l) * NW + w] = node[w];
+#pragma unroll
+    for (int z = 1; z <= HP; z++) {
+        const int step = 1 << (z - 1);
+        uint32_t other[NW];
+#pragma unroll
+        for (int w = 0; w < NW; w++) other[w] = __shfl_xor_sync(gmask, node[w], step);
+        if ((l & (2 * step - 1)) == 0) {
+            uint32_t lr[2 * NW];
+#pragma unroll
+            for (int w = 0; w < NW; w++) { lr[w] = node[w]; lr[NW + w] = other[w]; }
+            hashH_ms<P>(ms256, msT, make_adrs(layer, tree, T_TREE, 0, z, l >> z), lr, node, pks);
+#pragma unroll
+            for (int w = 0; w < NW; w++) tn[((LV >> z) + (l >> z)) * NW + w] = node[w];
+        }
+    }
+}
+
+
 template <class P, int POL, int MINB, int ILP = 1>
 __global__ void __launch_bounds__(128, MINB) tree_kernel(const KeyBlock* __restrict__ keys,
                                                    const MsgInfo* __restrict__ infos, uint32_t count,
@@ -252,38 +280,57 @@ __global__ void __launch_bounds__(128, MINB) tree_kernel(const KeyBlock* __restr
 // TREE_Sign, chain-parallel form for batches too small to fill the GPU with
 // one thread per leaf: first one thread per WOTS+ chain of every leaf of
 // every layer (d 2^h' len threads per message) writes its chain end to
-// scratch [m][j][l][i], then one thread per leaf absorbs its len chain ends
-// into T_len and the lane groups merge the Merkle levels as above.  Same
-// results; ~len times more parallelism per message.
+// scratch [m][j][l][i], then T_len absorbs each leaf's chain ends and the
+// lane groups merge the Merkle levels as above.  Same results; ~len times
+// more parallelism per message.  The trees built for several messages (desc,
+// ndesc of them, checkpoints of every leaf) follow the messages' own in both
+// launches, so they cost no serial step of their own.
 template <class P, int POL>
 __global__ void __launch_bounds__(128) chains_kernel(const KeyBlock* __restrict__ keys,
                                                      const MsgInfo* __restrict__ infos, uint32_t count,
                                                      uint32_t* __restrict__ ends, uint32_t* __restrict__ chk,
-                                                     uint32_t ck, uint32_t layers, uint32_t one) {
+                                                     uint32_t ck, uint32_t layers,
+                                                     const DedupDesc* __restrict__ desc, uint32_t ndesc,
+                                                     uint32_t* __restrict__ chk_u, uint32_t one) {
     constexpr int NW = P::NW, LV = P::LEAVES, LEN = P::LEN;
     const uint64_t gid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t per_msg = layers * LV * LEN;
-    const uint64_t m = gid / per_msg;
-    const uint32_t r = (uint32_t)(gid % per_msg);
-    const uint32_t j = r / (LV * LEN);
-    const uint32_t l = (r / LEN) % LV;
-    const uint32_t i = r % LEN;
-    if (m >= count) return;
-    const MsgInfo& info = infos[m];
-    if (info.key == KEY_INVALID) return;
-    const KeyBlock& kb = keys[info.key];
+    const uint64_t own = (uint64_t)count * per_msg;
+    const uint32_t per_chain = ck ? 16u >> (__ffs(ck) - 1) : 0u;      // ck: a power of two
+    const uint32_t ck_mask = ck ? ck - 1u : 0u, ck_shift = ck ? (uint32_t)(__ffs(ck) - 1) : 0u;
+    uint32_t key, j, l, i;
+    uint64_t tree;
+    uint32_t* mychk = nullptr;
+    if (gid < own) {
+        const uint64_t m = gid / per_msg;
+        const uint32_t r = (uint32_t)(gid % per_msg);
+        j = r / (LV * LEN);
+        l = (r / LEN) % LV;
+        i = r % LEN;
+        const MsgInfo& info = infos[m];
+        key = info.key;
+        if (key == KEY_INVALID) return;
+        tree = layer_tree<P>(info.idx_tree, (int)j);
+        if (ck != 0 && l == layer_leaf<P>(info.idx_tree, info.idx_leaf, (int)j))
+            mychk = chk + (((size_t)m * P::D + j) * (size_t)LEN + i) * per_chain * NW;
+    } else {
+        const uint64_t sid = gid - own, id = sid / (LV * LEN);
+        if (id >= ndesc) return;
+        const DedupDesc d = desc[id];
+        key = d.key;
+        j = d.layer;
+        tree = d.tree;
+        l = (uint32_t)((sid / LEN) % LV);
+        i = (uint32_t)(sid % LEN);
+        if (ck != 0) mychk = chk_u + (((size_t)id * LV + l) * (size_t)LEN + i) * per_chain * NW;
+    }
+    const KeyBlock& kb = keys[key];
     uint32_t ms256[8], x[NW];
 #pragma unroll
     for (int w = 0; w < 8; w++) ms256[w] = kb.ms256[w];
 #pragma unroll
     for (int w = 0; w < NW; w++) x[w] = kb.sk_seed[w];
-    const uint64_t tree = layer_tree<P>(info.idx_tree, (int)j);
-    const uint32_t sl = layer_leaf<P>(info.idx_tree, info.idx_leaf, (int)j);
     const Pipes<POL> pp(one);
-    uint32_t* mychk = nullptr;
-    const uint32_t per_chain = ck ? 16u >> (__ffs(ck) - 1) : 0u;      // ck: a power of two
-    const uint32_t ck_mask = ck ? ck - 1u : 0u, ck_shift = ck ? (uint32_t)(__ffs(ck) - 1) : 0u;
-    if (ck != 0 && l == sl) mychk = chk + (((size_t)m * P::D + j) * (size_t)LEN + i) * per_chain * NW;
     ChainCtx cx;
     MaskCtx<NW> mk;                              // robust sets: the chain's F masks
 #pragma unroll 1
@@ -321,46 +368,62 @@ __global__ void __launch_bounds__(128) chains_kernel(const KeyBlock* __restrict_
     for (int w = 0; w < NW; w++) e[w] = x[w];
 }
 
+// T_len and the Merkle levels over the chain ends, 32 leaves per block (whole
+// trees), T_len's schedules by the block's other warps (kern_tl.cuh); the
+// blocks behind the messages' own leaves take the trees of desc, whose nodes
+// go to nodes_u.
 template <class P>
-__global__ void __launch_bounds__(128) leaves_kernel(const KeyBlock* __restrict__ keys,
-                                                     const MsgInfo* __restrict__ infos, uint32_t count,
-                                                     const uint32_t* __restrict__ ends, uint8_t* __restrict__ sigs,
-                                                     uint32_t* __restrict__ roots, uint32_t layers) {
+__global__ void __launch_bounds__(TlShape<P>::THREADS) leaves_kernel(const KeyBlock* __restrict__ keys,
+                                                                     const MsgInfo* __restrict__ infos,
+                                                                     uint32_t count, uint32_t* __restrict__ ends,
+                                                                     uint8_t* __restrict__ sigs,
+                                                                     uint32_t* __restrict__ roots, uint32_t layers,
+                                                                     const DedupDesc* __restrict__ desc,
+                                                                     uint32_t ndesc, uint32_t* __restrict__ nodes_u) {
     constexpr int NW = P::NW, LV = P::LEAVES, LEN = P::LEN;
-    const uint32_t gid = blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ __align__(16) uint32_t smem[TlShape<P>::SMEM_WORDS];
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t per_msg = layers * LV;
-    const uint32_t m = gid / per_msg;
-    const uint32_t r = gid % per_msg;
-    const uint32_t j = r / LV;
-    const uint32_t l = r % LV;
-    if (m >= count) return;                         // whole trees exit together
-    const MsgInfo& info = infos[m];
-    if (info.key == KEY_INVALID) return;
+    const uint64_t own = (uint64_t)count * per_msg;
+    const uint32_t own_blocks = (uint32_t)((own + 31) / 32);
+    const bool shared = blockIdx.x >= own_blocks;    // block-uniform
+    uint32_t m = 0, id = 0, j = 0, key = KEY_INVALID;
+    uint64_t tree = 0, leaf;                         // leaf: its place in ends
+    if (!shared) {
+        leaf = (uint64_t)blockIdx.x * 32 + lane;
+        m = (uint32_t)(leaf / per_msg);
+        j = (uint32_t)(leaf % per_msg) / LV;
+        if (m < count) key = infos[m].key;
+        if (key != KEY_INVALID) tree = layer_tree<P>(infos[m].idx_tree, (int)j);
+    } else {
+        const uint64_t sid = (uint64_t)(blockIdx.x - own_blocks) * 32 + lane;
+        leaf = own + sid;
+        id = (uint32_t)(sid / LV);
+        if (id < ndesc) {
+            key = desc[id].key;
+            j = desc[id].layer;
+            tree = desc[id].tree;
+        }
+    }
+    const uint32_t l = lane % LV;                    // own leaves and shared ones both start at a tree
+    const bool active = key != KEY_INVALID;          // the same for a whole tree
+    const KeyBlock& kb = keys[active ? key : 0];
+    uint32_t node[NW];
+    tl_group<P, LEN>(P::BIG ? kb.ms512 : kb.ms256, make_adrs(j, tree, T_WOTS_PK, l, 0, 0), ends + leaf * LEN * NW,
+                     active, kb.pk_seed, smem, node);
+    if (threadIdx.x >= 32 || !active) return;
     const unsigned gmask = ((LV == 32) ? 0xFFFFFFFFu : ((1u << LV) - 1u)) << (lane & ~(uint32_t)(LV - 1));
-    const KeyBlock& kb = keys[info.key];
     uint32_t ms256[8], msT[P::BIG ? 16 : 8];
 #pragma unroll
     for (int w = 0; w < 8; w++) ms256[w] = kb.ms256[w];
 #pragma unroll
     for (int w = 0; w < (P::BIG ? 16 : 8); w++) msT[w] = P::BIG ? kb.ms512[w] : kb.ms256[w];
-    const uint64_t tree = layer_tree<P>(info.idx_tree, (int)j);
-    const uint32_t sl = layer_leaf<P>(info.idx_tree, info.idx_leaf, (int)j);
-    const uint32_t* e = ends + (size_t)gid * LEN * NW;
-    uint32_t node[NW];
-    if constexpr (P::SHAKE) {
-        TStreamP<P> ts;
-        ts.init(msT, make_adrs(j, tree, T_WOTS_PK, l, 0, 0));
-#pragma unroll 1
-        for (int i = 0; i < LEN; i++) ts.template push_n<NW>(e + i * NW);
-        ts.template finish<NW>(LEN * P::N, node);
+    if (shared) {
+        heap_finish<P>(ms256, msT, gmask, j, tree, l, node, nodes_u + (size_t)id * 2 * LV * NW, kb.pk_seed);
     } else {
-        const Adrs apk = make_adrs(j, tree, T_WOTS_PK, l, 0, 0);
-        // robust: mask this leaf's own chain ends in place (scratch, read once)
-        if constexpr (P::ROBUST) mask_mem<P::BIG, NW, LEN * NW>(kb.pk_seed, apk, const_cast<uint32_t*>(e));
-        tl_from_mem<P::BIG, LEN * NW, NW>(msT, apk, e, node);
+        const uint32_t sl = layer_leaf<P>(infos[m].idx_tree, infos[m].idx_leaf, (int)j);
+        merkle_finish<P>(ms256, msT, gmask, m, j, l, sl, tree, node, sigs, roots, kb.pk_seed);
     }
-    merkle_finish<P>(ms256, msT, gmask, m, j, l, sl, tree, node, sigs, roots, kb.pk_seed);
 }
 
 // Key generation: PK.root = root of tree 0 of the top layer d-1.  One lane

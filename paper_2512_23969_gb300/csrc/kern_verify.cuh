@@ -17,7 +17,7 @@
 // A chain needs w - 1 - digit steps (0 .. 15), so a warp of chains in
 // message order waits for its longest.  The chains of a layer are
 // therefore bucketed by their step count (the thread that produced msg_j
-// counts its message's digits and takes ranks with 16 atomics), scattered
+// counts its message's digits), scattered
 // longest first, and the chain kernel runs them in that order: the chains
 // of a warp then have the same length.
 #pragma once
@@ -25,6 +25,7 @@
 #include "hs_common.cuh"
 #include "hs_launch.h"
 #include "sha256_chain.cuh"
+#include "kern_tl.cuh"
 
 namespace hs {
 
@@ -71,84 +72,75 @@ __global__ void __launch_bounds__(128) vfors_kernel(const KeyBlock* __restrict__
     for (int w = 0; w < NW; w++) r[w] = node[w];
 }
 
-// The len base-w digits of an n-byte value (message nibbles, high first,
-// then the 3 checksum digits).
-template <class P>
-__device__ __forceinline__ uint32_t wots_digit(const uint32_t* msg, uint32_t i) {
-    constexpr int NW = P::NW;
-    if (i < (uint32_t)P::LEN1) return (msg[i >> 3] >> (28 - 4 * (i & 7))) & 15u;
-    uint32_t csum = 0;
-#pragma unroll
-    for (int w = 0; w < NW; w++)
-#pragma unroll
-        for (int b = 0; b < 8; b++) csum += 15u - ((msg[w] >> (28 - 4 * b)) & 15u);
-    return ((csum << 4) >> (12 - 4 * (i - P::LEN1))) & 15u;
-}
-
 constexpr uint32_t kRankBits = 28;        // sitem = steps << 28 | rank within the steps bucket
 
-// For message m's layer: each chain's step count, counted into the layer's
-// 16 buckets, with the chain's rank inside its bucket recorded in sitem.
-// Called by all 32 lanes of a warp, converged (inactive lanes count
-// nothing): per bucket the warp scans its lanes' counts with shuffles and
-// one lane adds the warp's total with a single atomic, so the 16 counters
-// see one atomic per warp instead of one per thread.  Messages with an
-// invalid key count as 0 steps.
+// The step counts of the chains of a block's messages (32 of them from m0 on:
+// digit sources and checksums in msg / csum, valid = false: 0 steps), counted
+// into the layer's 16 buckets, with each chain's rank inside its bucket
+// recorded in sitem.  The whole block works on the 32 * LEN chains: ranks in
+// the block from shared-memory counters, one global atomic per bucket and
+// block.  (A thread per message counting in registers, 16 selects per digit
+// and 80 shuffles, took about as long as T_len itself.)
 template <class P>
-__device__ __forceinline__ void count_steps(const uint32_t* msg, bool active, bool valid, uint64_t m,
+struct CountSmem {
+    uint32_t msg[32 * P::NW];
+    uint32_t csum[32];
+    uint32_t valid[32];
+    uint32_t hist[16], base[16];
+};
+template <class P>
+__device__ __forceinline__ void set_count_msg(CountSmem<P>& c, uint32_t lane, const uint32_t* msg, bool valid) {
+    uint32_t cs = 0;
+#pragma unroll
+    for (int w = 0; w < P::NW; w++) {
+        c.msg[lane * P::NW + w] = msg[w];
+#pragma unroll
+        for (int b = 0; b < 8; b++) cs += 15u - ((msg[w] >> (28 - 4 * b)) & 15u);
+    }
+    c.csum[lane] = cs << 4;
+    c.valid[lane] = valid ? 1u : 0u;
+    if (lane < 16) c.hist[lane] = 0;
+}
+// buf: 32 * LEN words of shared memory.  Every thread of the block calls it,
+// after a barrier behind set_count_msg.
+template <class P>
+__device__ __forceinline__ void count_block(CountSmem<P>& c, uint32_t* buf, uint32_t m0, uint32_t nmsg,
                                             uint32_t* __restrict__ cnt, uint32_t* __restrict__ sitem) {
     constexpr int LEN = P::LEN;
-    const uint32_t lane = threadIdx.x & 31;
-    uint32_t hist[16];
-#pragma unroll
-    for (int b = 0; b < 16; b++) hist[b] = 0;
-    if (active) {
-#pragma unroll 1
-        for (uint32_t i = 0; i < (uint32_t)LEN; i++) {
-            const uint32_t st = valid ? 15u - wots_digit<P>(msg, i) : 0u;
-#pragma unroll
-            for (int b = 0; b < 16; b++) hist[b] += (st == (uint32_t)b) ? 1u : 0u;
-        }
+    const uint32_t items = nmsg * LEN;
+    for (uint32_t it = threadIdx.x; it < items; it += blockDim.x) {
+        const uint32_t mm = it / LEN, i = it % LEN;
+        const uint32_t d = i < (uint32_t)P::LEN1 ? (c.msg[mm * P::NW + (i >> 3)] >> (28 - 4 * (i & 7))) & 15u
+                                                 : (c.csum[mm] >> (12 - 4 * (i - P::LEN1))) & 15u;
+        const uint32_t st = c.valid[mm] ? 15u - d : 0u;
+        buf[it] = (st << kRankBits) | atomicAdd(&c.hist[st], 1u);
     }
-    uint32_t base[16];
-#pragma unroll
-    for (int b = 0; b < 16; b++) {
-        uint32_t x = hist[b];                       // inclusive scan over the lanes
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, off);
-            if (lane >= (uint32_t)off) x += y;
-        }
-        const uint32_t total = __shfl_sync(0xFFFFFFFFu, x, 31);
-        uint32_t wbase = 0;
-        if (lane == 31 && total) wbase = atomicAdd(&cnt[b], total);
-        wbase = __shfl_sync(0xFFFFFFFFu, wbase, 31);
-        base[b] = wbase + x - hist[b];
-    }
-    if (!active) return;
-#pragma unroll 1
-    for (uint32_t i = 0; i < (uint32_t)LEN; i++) {
-        const uint32_t st = valid ? 15u - wots_digit<P>(msg, i) : 0u;
-        uint32_t r = 0;
-#pragma unroll
-        for (int b = 0; b < 16; b++)
-            if (st == (uint32_t)b) r = base[b]++;
-        sitem[m * LEN + i] = (st << kRankBits) | r;
+    __syncthreads();
+    if (threadIdx.x < 16) c.base[threadIdx.x] = c.hist[threadIdx.x] ? atomicAdd(&cnt[threadIdx.x], c.hist[threadIdx.x]) : 0u;
+    __syncthreads();
+    for (uint32_t it = threadIdx.x; it < items; it += blockDim.x) {
+        const uint32_t v = buf[it];
+        sitem[(size_t)m0 * LEN + it] = v + c.base[v >> kRankBits];
     }
 }
 
-// Layer 0: count from PK_FORS (every lane of every warp takes part).
+// Layer 0: count from PK_FORS, 32 messages per block.
 template <class P>
 __global__ void __launch_bounds__(128) vcount0_kernel(const MsgInfo* __restrict__ infos, uint32_t count,
                                                       const uint32_t* __restrict__ pk_fors, uint32_t* __restrict__ cnt,
                                                       uint32_t* __restrict__ sitem) {
-    const uint32_t m = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool active = m < count;
-    const bool valid = active && infos[m].key != KEY_INVALID;
-    uint32_t msg[P::NW];
+    __shared__ CountSmem<P> c;
+    __shared__ uint32_t buf[32 * P::LEN];
+    const uint32_t m0 = blockIdx.x * 32, m = m0 + threadIdx.x;
+    if (threadIdx.x < 32) {
+        const bool valid = m < count && infos[m].key != KEY_INVALID;
+        uint32_t msg[P::NW];
 #pragma unroll
-    for (int w = 0; w < P::NW; w++) msg[w] = active ? pk_fors[(size_t)m * P::NW + w] : 0u;
-    count_steps<P>(msg, active, valid, m, cnt, sitem);
+        for (int w = 0; w < P::NW; w++) msg[w] = valid ? pk_fors[(size_t)m * P::NW + w] : 0u;
+        set_count_msg<P>(c, threadIdx.x, msg, valid);
+    }
+    __syncthreads();
+    count_block<P>(c, buf, m0, min(32u, count - m0), cnt, sitem);
 }
 
 // Place every chain of the layer at its sorted position (longest first).
@@ -217,69 +209,62 @@ __global__ void __launch_bounds__(128) vchain_kernel(const KeyBlock* __restrict_
     for (int w = 0; w < NW; w++) e[w] = x[w];
 }
 
-// root_j of message m: T_len over its chain ends, h' climbs with the auth path.
+// Layer j of 32 messages per block: T_len over the chain ends (kern_tl.cuh),
+// then h' climbs with the auth path; root_j replaces msg_j in vroot and its
+// digits are counted for the next layer.
 template <class P>
-__device__ __forceinline__ void layer_root(const KeyBlock* __restrict__ keys, const MsgInfo& info,
-                                           const uint8_t* __restrict__ sigs, const uint32_t* __restrict__ ends,
-                                           uint32_t m, uint32_t j, uint32_t* node, uint32_t* __restrict__ vroot) {
+__global__ void __launch_bounds__(TlShape<P>::THREADS) vleaf_kernel(const KeyBlock* __restrict__ keys,
+                                                                    const MsgInfo* __restrict__ infos, uint32_t count,
+                                                                    const uint8_t* __restrict__ sigs,
+                                                                    uint32_t* __restrict__ ends,
+                                                                    uint32_t* __restrict__ vroot, uint32_t j,
+                                                                    uint32_t* __restrict__ cnt_next,
+                                                                    uint32_t* __restrict__ sitem) {
     constexpr int NW = P::NW, LEN = P::LEN, HP = P::HP;
-    const KeyBlock& kb = keys[info.key];
-    uint32_t ms256[8], msT[P::BIG ? 16 : 8];
-#pragma unroll
-    for (int w = 0; w < 8; w++) ms256[w] = kb.ms256[w];
-#pragma unroll
-    for (int w = 0; w < (P::BIG ? 16 : 8); w++) msT[w] = P::BIG ? kb.ms512[w] : kb.ms256[w];
+    constexpr int BUF = TlShape<P>::SMEM_WORDS > 32 * LEN ? TlShape<P>::SMEM_WORDS : 32 * LEN;
+    __shared__ __align__(16) uint32_t smem[BUF];
+    __shared__ CountSmem<P> c;
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t m0 = blockIdx.x * 32, m = m0 + lane;
+    const uint32_t key = m < count ? infos[m].key : KEY_INVALID;
+    const bool active = key != KEY_INVALID;
+    const MsgInfo& info = infos[active ? m : 0];
+    const KeyBlock& kb = keys[active ? key : 0];
     const uint64_t tree = layer_tree<P>(info.idx_tree, (int)j);
     const uint32_t kp = layer_leaf<P>(info.idx_tree, info.idx_leaf, (int)j);
-    const uint32_t* e = ends + (size_t)m * LEN * NW;
-    if constexpr (P::SHAKE) {
-        TStreamP<P> ts;
-        ts.init(msT, make_adrs(j, tree, T_WOTS_PK, kp, 0, 0));
-#pragma unroll 1
-        for (int i = 0; i < LEN; i++) ts.template push_n<NW>(e + i * NW);
-        ts.template finish<NW>(LEN * P::N, node);
-    } else {
-        const Adrs apk = make_adrs(j, tree, T_WOTS_PK, kp, 0, 0);
-        // robust: mask this message's chain ends of the layer in place (scratch, read once)
-        if constexpr (P::ROBUST) mask_mem<P::BIG, NW, LEN * NW>(kb.pk_seed, apk, const_cast<uint32_t*>(e));
-        tl_from_mem<P::BIG, LEN * NW, NW>(msT, apk, e, node);
-    }
-    const uint8_t* auth = sigs + (size_t)m * P::SIG_BYTES + P::N + P::FORS_BYTES + (size_t)j * P::LAYER_BYTES +
-                          (size_t)LEN * P::N;
-#pragma unroll 1
-    for (int z = 0; z < HP; z++) {
-        const uint32_t iz = kp >> z;
-        uint32_t au[NW], lr[2 * NW];
-        load_be<NW>(auth + (size_t)z * P::N, au);
-#pragma unroll
-        for (int w = 0; w < NW; w++) {
-            lr[w] = (iz & 1) ? au[w] : node[w];
-            lr[NW + w] = (iz & 1) ? node[w] : au[w];
-        }
-        hashH_ms<P>(ms256, msT, make_adrs(j, tree, T_TREE, 0, z + 1, iz >> 1), lr, node, kb.pk_seed);
-    }
-#pragma unroll
-    for (int w = 0; w < NW; w++) vroot[(size_t)m * NW + w] = node[w];
-}
-
-// Layer j of message m: T_len over the chain ends, then h' climbs with the
-// auth path; root_j replaces msg_j in vroot.
-template <class P>
-__global__ void __launch_bounds__(128) vleaf_kernel(const KeyBlock* __restrict__ keys,
-                                                    const MsgInfo* __restrict__ infos, uint32_t count,
-                                                    const uint8_t* __restrict__ sigs, const uint32_t* __restrict__ ends,
-                                                    uint32_t* __restrict__ vroot, uint32_t j,
-                                                    uint32_t* __restrict__ cnt_next, uint32_t* __restrict__ sitem) {
-    constexpr int NW = P::NW;
-    const uint32_t m = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool active = m < count;
-    const bool valid = active && infos[m].key != KEY_INVALID;
     uint32_t node[NW];
+    tl_group<P, LEN>(P::BIG ? kb.ms512 : kb.ms256, make_adrs(j, tree, T_WOTS_PK, kp, 0, 0),
+                     ends + (size_t)m * LEN * NW, active, kb.pk_seed, smem, node);
+    if (threadIdx.x < 32) {
+        if (active) {
+            uint32_t ms256[8], msT[P::BIG ? 16 : 8];
 #pragma unroll
-    for (int w = 0; w < NW; w++) node[w] = 0;
-    if (valid) layer_root<P>(keys, infos[m], sigs, ends, m, j, node, vroot);
-    __syncwarp();
-    if (cnt_next) count_steps<P>(node, active, valid, m, cnt_next, sitem);   // the next layer's chains
+            for (int w = 0; w < 8; w++) ms256[w] = kb.ms256[w];
+#pragma unroll
+            for (int w = 0; w < (P::BIG ? 16 : 8); w++) msT[w] = P::BIG ? kb.ms512[w] : kb.ms256[w];
+            const uint8_t* auth = sigs + (size_t)m * P::SIG_BYTES + P::N + P::FORS_BYTES + (size_t)j * P::LAYER_BYTES +
+                                  (size_t)LEN * P::N;
+#pragma unroll 1
+            for (int z = 0; z < HP; z++) {
+                const uint32_t iz = kp >> z;
+                uint32_t au[NW], lr[2 * NW];
+                load_be<NW>(auth + (size_t)z * P::N, au);
+#pragma unroll
+                for (int w = 0; w < NW; w++) {
+                    lr[w] = (iz & 1) ? au[w] : node[w];
+                    lr[NW + w] = (iz & 1) ? node[w] : au[w];
+                }
+                hashH_ms<P>(ms256, msT, make_adrs(j, tree, T_TREE, 0, z + 1, iz >> 1), lr, node, kb.pk_seed);
+            }
+#pragma unroll
+            for (int w = 0; w < NW; w++) vroot[(size_t)m * NW + w] = node[w];
+        }
+        if (cnt_next) set_count_msg<P>(c, lane, node, active);
+    }
+    if (cnt_next) {                                // the next layer's chains
+        __syncthreads();
+        count_block<P>(c, smem, m0, min(32u, count - m0), cnt_next, sitem);
+    }
 }
 
 // ok[m] = 1 iff the top root equals PK.root.

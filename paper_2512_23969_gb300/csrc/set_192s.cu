@@ -21,7 +21,7 @@ cudaError_t fors_variant(const Batch& b, int lpt, cudaStream_t s) {
 extern const SetOps kOps_192S = {
     SetImpl<P>::keyprep, SetImpl<P>::message, fors_variant, SetImpl<P>::fors_pk,
     TreeVariants<P, 0>::run, TreeVariants<P, 0>::has,
-    SetImpl<P>::tree_split, SetImpl<P>::tree_dedup, SetImpl<P>::tree_cached, SetImpl<P>::cache_build,
+    SetImpl<P>::tree_split, SetImpl<P>::tree_shared, SetImpl<P>::cache_build,
     SetImpl<P>::wots,       SetImpl<P>::verify,     SetImpl<P>::keygen,
     kForsLpt, 2, 32, kTreeMinb, 1, 0, tree_pol<P>()};
 

@@ -54,8 +54,7 @@ struct SetImpl {
         return cudaGetLastError();
     }
     static cudaError_t fors_pk(const Batch& b, cudaStream_t s) {
-        const uint32_t T = 128, G = (b.count + T - 1) / T;
-        fors_pk_kernel<P><<<G, T, 0, s>>>(b.keys, b.infos, b.count, b.fors_roots, b.pk_fors);
+        fors_pk_kernel<P><<<(b.count + 31) / 32, TlShape<P>::THREADS, 0, s>>>(b.keys, b.infos, b.count, b.fors_roots, b.pk_fors);
         return cudaGetLastError();
     }
     template <int MINB, int POL = tree_pol<P>(), int ILP = 1>
@@ -65,15 +64,24 @@ struct SetImpl {
         const uint32_t T = 128;
         const uint32_t G = (uint32_t)((threads + T - 1) / T);
         if (threads == 0) return cudaSuccess;
+        cudaError_t e = describe_shared(b, s);
+        if (e == cudaSuccess && b.max_uniq) e = build_trees(b.keys, b.desc, b.max_uniq, b.nodes_u, b.chk_u, b.ck, s);
+        if (e != cudaSuccess) return e;
         if constexpr (kWide) {
             bleaf_kernel<P, POL, MINB, ILP><<<G, T, 0, s>>>(b.keys, b.infos, b.count, b.leafv, b.chk, b.ck, L, 1u);
-            cudaError_t e = cudaGetLastError();
+            e = cudaGetLastError();
             return e == cudaSuccess ? merge(b, s) : e;
         } else {
             tree_kernel<P, POL, MINB, ILP><<<G, T, 0, s>>>(b.keys, b.infos, b.count, b.sigs, b.roots, b.chk, b.ck,
                                                         L, 1u);
             return cudaGetLastError();
         }
+    }
+    // The descriptions of the trees this call builds for several messages.
+    static cudaError_t describe_shared(const Batch& b, cudaStream_t s) {
+        if (b.max_uniq == 0) return cudaSuccess;
+        cache_desc_kernel<P><<<(b.max_uniq + 127) / 128, 128, 0, s>>>(b.num_keys, own_layers(b), b.cache_tpk, b.desc);
+        return cudaGetLastError();
     }
     // Wide trees: one block per (message, layer) merges the stored leaves.
     static cudaError_t merge(const Batch& b, cudaStream_t s) {
@@ -84,44 +92,26 @@ struct SetImpl {
                                                                      b.roots, L);
         return cudaGetLastError();
     }
-    // The distinct trees of the shared / cached layers, all nodes and the
-    // checkpoints of every leaf (desc: their (key, layer, tree)).
-    static cudaError_t build_trees(const KeyBlock* keys, const DedupDesc* desc, const uint32_t* nuniq,
-                                   uint32_t max_uniq, uint32_t* nodes, uint32_t* chk, uint32_t ck, cudaStream_t s) {
+    // The ndesc trees of desc, all nodes and the checkpoints of every leaf: a
+    // thread per leaf.
+    static cudaError_t build_trees(const KeyBlock* keys, const DedupDesc* desc, uint32_t ndesc, uint32_t* nodes,
+                                   uint32_t* chk, uint32_t ck, cudaStream_t s) {
         const uint32_t T = 128;
-        const uint64_t th = (uint64_t)max_uniq * P::LEAVES;
+        const uint64_t th = (uint64_t)ndesc * P::LEAVES;
         if (th == 0) return cudaSuccess;
+        const uint32_t G = (uint32_t)((th + T - 1) / T);
         if constexpr (kWide) {
-            wtree_leaf_kernel<P, tree_pol<P>()><<<(uint32_t)((th + T - 1) / T), T, 0, s>>>(keys, desc, nuniq, max_uniq,
-                                                                                      nodes, chk, ck, 1u);
+            wtree_leaf_kernel<P, tree_pol<P>()><<<G, T, 0, s>>>(keys, desc, ndesc, nodes, chk, ck, 1u);
             cudaError_t e = cudaGetLastError();
             if (e != cudaSuccess) return e;
-            wtree_merge_kernel<P><<<max_uniq, kMergeThreads, 0, s>>>(keys, desc, nuniq, max_uniq, nodes);
+            wtree_merge_kernel<P><<<ndesc, kMergeThreads, 0, s>>>(keys, desc, ndesc, nodes);
         } else {
-            utree_kernel<P, tree_pol<P>()><<<(uint32_t)((th + T - 1) / T), T, 0, s>>>(keys, desc, nuniq, max_uniq, nodes,
-                                                                                  chk, ck, 1u);
+            utree_kernel<P, tree_pol<P>()><<<G, T, 0, s>>>(keys, desc, ndesc, nodes, chk, ck, 1u);
         }
         return cudaGetLastError();
     }
-    static cudaError_t tree_dedup(const Batch& b, cudaStream_t s) {
-        const uint32_t T = 128, L = own_layers(b);
-        const uint64_t mj = (uint64_t)b.count * (P::D - L);
-        dedup_insert_kernel<P><<<(uint32_t)((mj + T - 1) / T), T, 0, s>>>(b.infos, b.count, L, b.table, b.cap_log2,
-                                                                          b.mj_slot, b.status);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        const uint32_t cap = 1u << b.cap_log2;
-        dedup_compact_kernel<<<(cap + T - 1) / T, T, 0, s>>>(b.table, cap, b.slot_id, b.desc, b.nuniq, b.max_uniq,
-                                                             b.status);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if ((e = build_trees(b.keys, b.desc, b.nuniq, b.max_uniq, b.nodes_u, b.chk_u, b.ck, s)) != cudaSuccess)
-            return e;
-        dedup_scatter_kernel<P><<<(uint32_t)((mj + T - 1) / T), T, 0, s>>>(b.infos, b.count, L, b.mj_slot, b.slot_id,
-                                                                           b.nodes_u, b.sigs, b.roots, b.mj_id);
-        return cudaGetLastError();
-    }
-    // Cached top layers (keyset): auth paths, roots and tree ids from the cache.
-    static cudaError_t tree_cached(const Batch& b, cudaStream_t s) {
+    // Shared or cached top layers: auth paths, roots and tree ids from their nodes.
+    static cudaError_t tree_shared(const Batch& b, cudaStream_t s) {
         const uint32_t T = 128, L = own_layers(b);
         const uint64_t mj = (uint64_t)b.count * (P::D - L);
         if (mj == 0) return cudaSuccess;
@@ -138,28 +128,43 @@ struct SetImpl {
         cache_desc_kernel<P><<<(uint32_t)((trees + T - 1) / T), T, 0, s>>>(num_keys, L, tpk, desc);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        return build_trees(keys, desc, nullptr, (uint32_t)trees, nodes, chk, ck, s);
+        return build_trees(keys, desc, (uint32_t)trees, nodes, chk, ck, s);
     }
-    static cudaError_t tree_split(const Batch& b, cudaStream_t s) {
+    // Chain-parallel form: the messages' own trees and the ndesc trees of
+    // desc in the same launches (either may be none).
+    static cudaError_t split_trees(const KeyBlock* keys, const MsgInfo* infos, uint32_t count, uint32_t L,
+                                   uint32_t* ends, uint32_t* chk, uint32_t ck, const DedupDesc* desc, uint32_t ndesc,
+                                   uint32_t* nodes_u, uint32_t* chk_u, uint32_t* leafv, uint8_t* sigs,
+                                   uint32_t* roots, cudaStream_t s) {
         const uint32_t T = 128;
-        const uint32_t L = own_layers(b);
-        const uint64_t chains = (uint64_t)b.count * L * P::LEAVES * P::LEN;
+        const uint64_t own = (uint64_t)count * L * P::LEAVES, shared = (uint64_t)ndesc * P::LEAVES;
+        const uint64_t chains = (own + shared) * P::LEN;
         if (chains == 0) return cudaSuccess;
-        chains_kernel<P, tree_pol<P>()><<<(uint32_t)((chains + T - 1) / T), T, 0, s>>>(b.keys, b.infos, b.count, b.ends,
-                                                                                  b.chk, b.ck, L, 1u);
+        chains_kernel<P, tree_pol<P>()><<<(uint32_t)((chains + T - 1) / T), T, 0, s>>>(
+            keys, infos, count, ends, chk, ck, L, desc, ndesc, chk_u, 1u);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        const uint64_t leaves = (uint64_t)b.count * L * P::LEAVES;
+        const uint32_t G = (uint32_t)((own + 31) / 32 + (shared + 31) / 32);
         if constexpr (kWide) {
-            bleaf_from_ends_kernel<P><<<(uint32_t)((leaves + T - 1) / T), T, 0, s>>>(b.keys, b.infos, b.count,
-                                                                                    b.ends, b.leafv, L);
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            return merge(b, s);
+            bleaf_from_ends_kernel<P><<<G, TlShape<P>::THREADS, 0, s>>>(keys, infos, count, ends, leafv, L, desc,
+                                                                        ndesc, nodes_u);
+            if ((e = cudaGetLastError()) != cudaSuccess || ndesc == 0) return e;
+            wtree_merge_kernel<P><<<ndesc, kMergeThreads, 0, s>>>(keys, desc, ndesc, nodes_u);
         } else {
-            leaves_kernel<P><<<(uint32_t)((leaves + T - 1) / T), T, 0, s>>>(b.keys, b.infos, b.count, b.ends,
-                                                                            b.sigs, b.roots, L);
-            return cudaGetLastError();
+            leaves_kernel<P><<<G, TlShape<P>::THREADS, 0, s>>>(keys, infos, count, ends, sigs, roots, L, desc, ndesc,
+                                                               nodes_u);
         }
+        return cudaGetLastError();
+    }
+    static cudaError_t tree_split(const Batch& b, cudaStream_t s) {
+        cudaError_t e = describe_shared(b, s);
+        if (e == cudaSuccess)
+            e = split_trees(b.keys, b.infos, b.count, own_layers(b), b.ends, b.chk, b.ck, b.desc, b.max_uniq,
+                            b.nodes_u, b.chk_u, b.leafv, b.sigs, b.roots, s);
+        if constexpr (kWide) {
+            if (e == cudaSuccess) e = merge(b, s);
+        }
+        return e;
     }
     static cudaError_t wots(const Batch& b, cudaStream_t s) {
         const uint64_t threads = (uint64_t)b.count * P::D * P::LEN;
@@ -186,9 +191,9 @@ struct SetImpl {
         }
         if (e == cudaSuccess) e = fors_pk(b, s);
         const uint64_t ct = (uint64_t)b.count * P::LEN;
-        const uint32_t G1 = (b.count + T - 1) / T;
+        const uint32_t G1 = (b.count + T - 1) / T, G32 = (b.count + 31) / 32;
         if (e == cudaSuccess) {
-            vcount0_kernel<P><<<G1, T, 0, s>>>(b.infos, b.count, b.pk_fors, b.vcnt, b.vsitem);
+            vcount0_kernel<P><<<G32, T, 0, s>>>(b.infos, b.count, b.pk_fors, b.vcnt, b.vsitem);
             e = cudaGetLastError();
         }
         for (uint32_t j = 0; j < (uint32_t)P::D && e == cudaSuccess; j++) {
@@ -198,7 +203,7 @@ struct SetImpl {
             vchain_kernel<P, kChainPol><<<(uint32_t)((ct + T - 1) / T), T, 0, s>>>(
                 b.keys, b.infos, b.count, b.sigs, b.vorder, b.vsitem, b.ends, j, 1u);
             if ((e = cudaGetLastError()) != cudaSuccess) break;
-            vleaf_kernel<P><<<G1, T, 0, s>>>(b.keys, b.infos, b.count, b.sigs, b.ends, b.roots, j,
+            vleaf_kernel<P><<<G32, TlShape<P>::THREADS, 0, s>>>(b.keys, b.infos, b.count, b.sigs, b.ends, b.roots, j,
                                              j + 1 < (uint32_t)P::D ? b.vcnt + 16 * (j + 1) : nullptr, b.vsitem);
             e = cudaGetLastError();
         }
@@ -206,34 +211,60 @@ struct SetImpl {
         vfinal_kernel<P><<<G1, T, 0, s>>>(b.keys, b.infos, b.count, b.roots, b.ok);
         return cudaGetLastError();
     }
-    static cudaError_t keygen(const uint8_t* seeds, uint32_t count, uint8_t* pk, uint8_t* sk, cudaStream_t s) {
+    // split: chain-parallel, one XMSS tree per key as the trees of desc.
+    static cudaError_t keygen(const uint8_t* seeds, uint32_t count, uint8_t* pk, uint8_t* sk, bool split,
+                              cudaStream_t s) {
         const uint64_t threads = (uint64_t)count * P::LEAVES;
         const uint32_t T = 128;
         const uint32_t G = (uint32_t)((threads + T - 1) / T);
-        if constexpr (kWide) {
-            // key blocks, top-tree leaves, then one block per key for the root
-            const size_t kb_bytes = ((size_t)count * sizeof(KeyBlock) + 255) & ~(size_t)255;
-            void* scratch = nullptr;
-            cudaError_t e = pool_alloc(&scratch, kb_bytes + threads * P::NW * 4, s);
-            if (e != cudaSuccess) return e;
-            KeyBlock* kbs = static_cast<KeyBlock*>(scratch);
-            uint32_t* leafv = reinterpret_cast<uint32_t*>(static_cast<char*>(scratch) + kb_bytes);
-            seed_keys_kernel<P><<<(count + T - 1) / T, T, 0, s>>>(seeds, count, kbs);
-            e = cudaGetLastError();
-            if (e == cudaSuccess) {
-                bkeygen_leaf_kernel<P, kChainPol><<<G, T, 0, s>>>(kbs, count, leafv, 1u);
-                e = cudaGetLastError();
-            }
-            if (e == cudaSuccess) {
-                bkeygen_root_kernel<P><<<count, kMergeThreads, 0, s>>>(kbs, seeds, count, leafv, pk, sk);
-                e = cudaGetLastError();
-            }
-            const cudaError_t f = cudaFreeAsync(scratch, s);
-            return e == cudaSuccess ? f : e;
-        } else {
-            keygen_kernel<P><<<G, T, 0, s>>>(seeds, count, pk, sk, 1u);
+        if (!kWide && !split) {
+            if constexpr (!kWide) keygen_kernel<P><<<G, T, 0, s>>>(seeds, count, pk, sk, 1u);
             return cudaGetLastError();
         }
+        auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
+        const size_t kb_bytes = al((size_t)count * sizeof(KeyBlock));
+        const size_t node_bytes = al((split ? 2 : 1) * threads * P::NW * 4);      // heap, or the leaves alone
+        const size_t desc_bytes = split ? al((size_t)count * sizeof(DedupDesc)) : 0;
+        const size_t end_bytes = split ? threads * P::LEN * P::NW * 4 : 0;
+        void* scratch = nullptr;
+        cudaError_t e = pool_alloc(&scratch, kb_bytes + node_bytes + desc_bytes + end_bytes, s);
+        if (e == cudaErrorMemoryAllocation && split) {       // the chain ends are extra scratch
+            cudaGetLastError();
+            return keygen(seeds, count, pk, sk, false, s);
+        }
+        if (e != cudaSuccess) return e;
+        KeyBlock* kbs = static_cast<KeyBlock*>(scratch);
+        char* at = static_cast<char*>(scratch) + kb_bytes;
+        uint32_t* nodes = reinterpret_cast<uint32_t*>(at);
+        seed_keys_kernel<P><<<(count + T - 1) / T, T, 0, s>>>(seeds, count, kbs);
+        e = cudaGetLastError();
+        if (split) {
+            DedupDesc* desc = reinterpret_cast<DedupDesc*>(at + node_bytes);
+            uint32_t* ends = reinterpret_cast<uint32_t*>(at + node_bytes + desc_bytes);
+            if (e == cudaSuccess) {
+                cache_desc_kernel<P><<<(count + T - 1) / T, T, 0, s>>>(count, (uint32_t)P::D - 1, 1u, desc);
+                e = cudaGetLastError();
+            }
+            if (e == cudaSuccess)
+                e = split_trees(kbs, nullptr, 0, 0, ends, nullptr, 0, desc, count, nodes, nullptr, nullptr, nullptr,
+                                nullptr, s);
+            if (e == cudaSuccess) {
+                const uint64_t bytes = (uint64_t)count * 4 * P::N;
+                keygen_out_kernel<P><<<(uint32_t)((bytes + T - 1) / T), T, 0, s>>>(seeds, count, nodes, pk, sk);
+                e = cudaGetLastError();
+            }
+        } else if constexpr (kWide) {       // top-tree leaves, then one block per key for the root
+            if (e == cudaSuccess) {
+                bkeygen_leaf_kernel<P, kChainPol><<<G, T, 0, s>>>(kbs, count, nodes, 1u);
+                e = cudaGetLastError();
+            }
+            if (e == cudaSuccess) {
+                bkeygen_root_kernel<P><<<count, kMergeThreads, 0, s>>>(kbs, seeds, count, nodes, pk, sk);
+                e = cudaGetLastError();
+            }
+        }
+        const cudaError_t f = cudaFreeAsync(scratch, s);
+        return e == cudaSuccess ? f : e;
     }
 };
 

@@ -564,5 +564,5 @@ def hs_set_host_direct(on=True):
 
 
 def hs_set_tree_sharing(on=True):
-    """Share repeated upper-layer XMSS trees within a batch (same bytes, less work)."""
+    """Build repeated upper-layer XMSS trees once per batch (default on; same bytes, less work)."""
     _check(load().hs_set_tree_sharing(1 if on else 0))
