@@ -219,13 +219,28 @@ cudaError_t launch_fors_pk(const Batch& b, cudaStream_t s) {
     const SetOps* o = set_ops(b.pset);
     return o ? o->fors_pk(b, s) : cudaErrorInvalidValue;
 }
-cudaError_t launch_tree(const Batch& b, cudaStream_t s) {
+static cudaError_t tree_beside(const Batch& b, BesideFn beside, cudaStream_t s) {
     const SetOps* o = set_ops(b.pset);
     if (!o) return cudaErrorInvalidValue;
-    cudaError_t e = b.split ? o->tree_split(b, s)
-                            : o->tree(b, tune_get(b.pset, 1), tune_get(b.pset, 3), tune_get(b.pset, 4), s);
+    cudaError_t e = b.split ? o->tree_split(b, beside, s)
+                            : o->tree(b, tune_get(b.pset, 1), tune_get(b.pset, 3), tune_get(b.pset, 4), beside, s);
     if (e == cudaSuccess && b.dedup_layer) e = o->tree_shared(b, s);     // the shared layers' auth paths and roots
     return e;
+}
+cudaError_t launch_tree(const Batch& b, cudaStream_t s) { return tree_beside(b, nullptr, s); }
+cudaError_t launch_sign_trees(const Batch& b, cudaStream_t s) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        cudaError_t e = launch_fors(b, s);
+        if (e == cudaSuccess) e = launch_fors_pk(b, s);
+        return e == cudaSuccess ? launch_tree(b, s) : e;
+    }
+    Batch c = b;
+    c.beside = true;
+    return tree_beside(c, [](const Batch& x, int stage, cudaStream_t st) {
+        return stage == 0 ? launch_fors(x, st) : launch_fors_pk(x, st);
+    }, s);
 }
 cudaError_t launch_wots(const Batch& b, cudaStream_t s) {
     const SetOps* o = set_ops(b.pset);

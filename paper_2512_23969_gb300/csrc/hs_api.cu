@@ -559,12 +559,16 @@ static hs_status run_batch(const hs_keyset* ks, bool verify, hs_params p, const 
     if (e == cudaSuccess) e = launch_message(b, verify, s);
     if (prof) prof_mark(3, s);
     if (!verify) {
-        if (e == cudaSuccess) e = launch_fors(b, s);
-        if (prof) prof_mark(4, s);
-        if (e == cudaSuccess) e = launch_fors_pk(b, s);
-        if (prof) prof_mark(5, s);
-        if (e == cudaSuccess) e = launch_tree(b, s);
-        if (prof) prof_mark(6, s);
+        if (prof) {                                  // a stage at a time, each between its events
+            if (e == cudaSuccess) e = launch_fors(b, s);
+            prof_mark(4, s);
+            if (e == cudaSuccess) e = launch_fors_pk(b, s);
+            prof_mark(5, s);
+            if (e == cudaSuccess) e = launch_tree(b, s);
+            prof_mark(6, s);
+        } else if (e == cudaSuccess) {
+            e = launch_sign_trees(b, s);
+        }
         if (e == cudaSuccess) e = launch_wots(b, s);
         if (prof) prof_mark(7, s);
     } else {

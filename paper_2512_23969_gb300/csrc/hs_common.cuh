@@ -21,6 +21,16 @@
 
 namespace hs {
 
+// Programmatic dependent launch.  A kernel that calls allow_next lets the
+// next launch of its stream start beside it, if that launch asks for it
+// (launch_beside) and once all of this grid's blocks have started.  The
+// grid that started beside it is complete only after it is: one extra block
+// of that grid does nothing but wait for it (wait_previous), so whatever
+// follows on the stream still comes after both.
+__device__ __forceinline__ void allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+constexpr uint32_t kNoGuard = 0xFFFFFFFFu;     // no such block: an ordinary launch
+
 // Fill the words of one message block after the midstate: ADRSc, payload of
 // PW words, 0x80 pad byte; zero the rest (length added by the caller).
 template <int BW, int PW>

@@ -66,7 +66,14 @@ struct Batch {
     // message stage: a warp per message (SHA-2 sets, small batches; the
     // form is fixed with the batch, like 'split')
     bool msg_warp;
+    // FORS launches: start beside the previous launch of the stream instead
+    // of behind it (sign_trees)
+    bool beside;
 };
+
+// Called by the TREE_Sign launchers behind their first launch (stage 0) and
+// their last (stage 1): FORS_Sign and T_k run beside them.  May be null.
+typedef cudaError_t (*BesideFn)(const Batch&, int stage, cudaStream_t);
 
 // Record the text hs_last_error() returns on the calling thread.
 void set_last_error(const char* msg);
@@ -104,9 +111,9 @@ struct SetOps {
     cudaError_t (*fors_pk)(const Batch&, cudaStream_t);
     // TREE_Sign per leaf: (min blocks, addition policy, chains per thread);
     // tree_has says which combinations are compiled
-    cudaError_t (*tree)(const Batch&, int, int, int, cudaStream_t);
+    cudaError_t (*tree)(const Batch&, int, int, int, BesideFn, cudaStream_t);
     bool (*tree_has)(int, int, int);
-    cudaError_t (*tree_split)(const Batch&, cudaStream_t);
+    cudaError_t (*tree_split)(const Batch&, BesideFn, cudaStream_t);
     cudaError_t (*tree_shared)(const Batch&, cudaStream_t);
     cudaError_t (*cache_build)(const KeyBlock*, uint32_t, uint32_t, uint32_t, DedupDesc*, uint32_t*, uint32_t*,
                                uint32_t, cudaStream_t);
@@ -158,11 +165,21 @@ int sm_count();
 int fors_lanes(int pset, uint32_t count);
 
 cudaError_t launch_keyprep(const Batch& b, bool from_pk, cudaStream_t s);
+// The message stage's warp form sums the lengths before its message itself
+// up to this many messages (1024 read 8 KB a warp at most; measured 7 us less
+// per call than the prefix sum's launch); above, and in the thread form, the
+// offsets come from a prefix sum.
+constexpr uint32_t kSumLens = 4096;
+inline bool needs_offsets(const Batch& b) { return !b.msg_warp || b.count > kSumLens; }
 cudaError_t launch_offsets(const Batch& b, cudaStream_t s);
 cudaError_t launch_message(const Batch& b, bool verify, cudaStream_t s);
 cudaError_t launch_fors(const Batch& b, cudaStream_t s);
 cudaError_t launch_fors_pk(const Batch& b, cudaStream_t s);
 cudaError_t launch_tree(const Batch& b, cudaStream_t s);
+// FORS_Sign, T_k and TREE_Sign of a batch on one stream, the FORS stages
+// beside TREE_Sign (independent given the digest) unless the stream is being
+// captured.
+cudaError_t launch_sign_trees(const Batch& b, cudaStream_t s);
 cudaError_t launch_wots(const Batch& b, cudaStream_t s);
 cudaError_t launch_verify(const Batch& b, cudaStream_t s);
 cudaError_t launch_keygen(int pset, const uint8_t* seeds, uint32_t count, uint8_t* pk, uint8_t* sk,

@@ -313,9 +313,7 @@ bool admit(ServerImpl& sv, Slot& slot) {
     if (e == cudaSuccess) e = cudaMemcpyAsync(d, h, o_sigs, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = launch_offsets(b, s);
     if (e == cudaSuccess) e = launch_message(b, false, s);
-    if (e == cudaSuccess) e = launch_fors(b, s);
-    if (e == cudaSuccess) e = launch_fors_pk(b, s);
-    if (e == cudaSuccess) e = launch_tree(b, s);
+    if (e == cudaSuccess) e = launch_sign_trees(b, s);
     if (e == cudaSuccess) e = launch_wots(b, s);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(h + o_sigs, d + o_sigs, count * (size_t)sig_bytes_of(p), cudaMemcpyDeviceToHost, s);

@@ -27,6 +27,7 @@ __global__ void offsets_kernel(const uint64_t* __restrict__ lens, uint32_t count
 }
 
 cudaError_t launch_offsets(const Batch& b, cudaStream_t s) {
+    if (!needs_offsets(b)) return cudaSuccess;
     offsets_kernel<<<1, 1024, 0, s>>>(b.lens, b.count, b.offsets);
     return cudaGetLastError();
 }

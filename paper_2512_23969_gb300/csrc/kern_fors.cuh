@@ -90,11 +90,68 @@ struct SibStack<R, RI, NW, false> {
     }
 };
 
+// A FORS leaf: sk = PRF(FORS_PRF(g)), then F(FORS_TREE(height 0, g), sk),
+// both through one call site of the compression.
+// With a chain context: PRF and F of every leaf of a message share address
+// words 0..4 (layer, tree, type, key pair, height 0 and the top half of the
+// leaf index, which is 0 while k * 2^a <= 2^16), so rounds 0..4 of each (and
+// round 5 up to its message word) are computed once per thread and a leaf
+// hash runs rounds 6..63 -- the same compression as the chain steps of
+// TREE_Sign, bit for bit.  The two contexts are read at a run-time index
+// (local memory): 60 registers instead of 79 for a register select, and as
+// fast or faster (FORS 128f 6.39 -> 6.19 ms, 256f 45.2 -> 43.6 ms per 16384 /
+// 8192 signatures).
+template <class P, int POL>
+struct ForsLeaf {
+    static constexpr int NW = P::NW;
+    static constexpr bool kCtx = !P::SHAKE && ((uint64_t)P::K << P::A) <= 65536u;
+    ChainCtx cxs[kCtx ? 2 : 1];
+    MaskCtx<NW> mk;                                // robust sets: the leaf F masks
+    __device__ __forceinline__ ForsLeaf(const KeyBlock& kb, const uint32_t* ms256, uint64_t tree, uint32_t kp,
+                                        const Pipes<POL>& pp) {
+        if constexpr (kCtx) {
+            chain_ctx<POL>(ms256, make_adrs(0, tree, T_FORS_PRF, kp, 0, 0), cxs[0], pp);
+            chain_ctx<POL>(ms256, make_adrs(0, tree, T_FORS_TREE, kp, 0, 0), cxs[1], pp);
+            if constexpr (P::ROBUST) mask_ctx<POL, NW>(kb.pk_seed, make_adrs(0, tree, T_FORS_TREE, kp, 0, 0), mk, pp);
+        }
+    }
+    // node = leaf g; the secret goes to sk_out if it is not null
+    __device__ __forceinline__ void hash(const KeyBlock& kb, const uint32_t* ms256, const uint32_t* skseed,
+                                         uint64_t tree, uint32_t kp, uint32_t g, uint32_t* node, uint8_t* sk_out,
+                                         const Pipes<POL>& pp) const {
+#pragma unroll
+        for (int w = 0; w < NW; w++) node[w] = skseed[w];
+#pragma unroll 1
+        for (int s = 0; s < 2; s++) {
+            if constexpr (kCtx && P::ROBUST) {
+                // the leaf F (s = 1) hashes sk masked with its own address; PRF does not
+                uint32_t xm[NW];
+#pragma unroll
+                for (int w = 0; w < NW; w++) xm[w] = node[w];
+                if (s == 1) {
+                    uint32_t m[NW];
+                    mask_step<POL, NW>(mk, g, m, pp);
+#pragma unroll
+                    for (int w = 0; w < NW; w++) xm[w] ^= m[w];
+                }
+                chain_step<POL, NW>(cxs[s], ms256, g, xm, node, pp);
+            } else if constexpr (kCtx) {
+                chain_step<POL, NW>(cxs[s], ms256, g, node, node, pp);
+            } else {
+                hashF_p<P, POL>(ms256, make_adrs(0, tree, s == 0 ? T_FORS_PRF : T_FORS_TREE, kp, 0, g), node, node, pp,
+                                s == 0 ? nullptr : kb.pk_seed);
+            }
+            if (s == 0 && sk_out != nullptr) store_be<NW>(sk_out, node);
+        }
+    }
+};
+
 template <class P, int POL, int LPT>
 __global__ void __launch_bounds__(256) fors_kernel(const KeyBlock* __restrict__ keys,
                                                    const MsgInfo* __restrict__ infos, uint32_t count,
                                                    uint8_t* __restrict__ sigs, uint32_t* __restrict__ fors_roots,
-                                                   uint32_t one) {
+                                                   uint32_t one, uint32_t guard) {
+    if (blockIdx.x == guard) { wait_previous(); return; }
     constexpr int NW = P::NW, A = P::A, K = P::K;
     constexpr int R = A - Log2<LPT>::v;           // height built inside one lane
     constexpr int RI = R < 7 ? R : 7;             // inner treehash height
@@ -128,24 +185,7 @@ __global__ void __launch_bounds__(256) fors_kernel(const KeyBlock* __restrict__ 
     uint8_t* sf = sigs + (size_t)m * P::SIG_BYTES + P::N + (size_t)i * (A + 1) * P::N;
 
     const Pipes<POL> pp(one);
-    // Leaf hashes with a chain context: PRF and F of every leaf of this
-    // message share address words 0..4 (layer, tree, type, key pair, height
-    // 0 and the top half of the leaf index, which is 0 while k * 2^a <=
-    // 2^16), so rounds 0..4 of each (and round 5 up to its message word)
-    // are computed once here and a leaf hash runs rounds 6..63 -- the same
-    // compression as the chain steps of TREE_Sign, bit for bit.  The two
-    // contexts are read at a run-time
-    // index (local memory): 60 registers instead of 79 for a register
-    // select, and as fast or faster (FORS 128f 6.39 -> 6.19 ms, 256f 45.2
-    // -> 43.6 ms per 16384 / 8192 signatures).
-    constexpr bool kCtx = !P::SHAKE && ((uint64_t)K << A) <= 65536u;
-    ChainCtx cxs[kCtx ? 2 : 1];
-    MaskCtx<NW> mk;                                // robust sets: the leaf F masks
-    if constexpr (kCtx) {
-        chain_ctx<POL>(ms256, make_adrs(0, tree, T_FORS_PRF, kp, 0, 0), cxs[0], pp);
-        chain_ctx<POL>(ms256, make_adrs(0, tree, T_FORS_TREE, kp, 0, 0), cxs[1], pp);
-        if constexpr (P::ROBUST) mask_ctx<POL, NW>(kb.pk_seed, make_adrs(0, tree, T_FORS_TREE, kp, 0, 0), mk, pp);
-    }
+    const ForsLeaf<P, POL> leaf(kb, ms256, tree, kp, pp);
     SibStack<R, RI, NW, (R <= 7)> stk;                 // left siblings, levels 0..R-1
     uint32_t node[NW];
     const uint32_t base = L << R;                  // first leaf of this lane (within tree)
@@ -155,32 +195,7 @@ __global__ void __launch_bounds__(256) fors_kernel(const KeyBlock* __restrict__ 
         for (uint32_t p = 0; p < (1u << RI); p++) {
             const uint32_t t = base + (ob << RI) + p;  // leaf index within tree
             const uint32_t g = (i << A) + t;           // global leaf index
-            // leaf g: sk = PRF(FORS_PRF(g)), then F(FORS_TREE(height 0, g), sk);
-            // both through one call site of the compression
-#pragma unroll
-            for (int w = 0; w < NW; w++) node[w] = skseed[w];
-#pragma unroll 1
-            for (int s = 0; s < 2; s++) {
-                if constexpr (kCtx && P::ROBUST) {
-                    // the leaf F (s = 1) hashes sk masked with its own address; PRF does not
-                    uint32_t xm[NW];
-#pragma unroll
-                    for (int w = 0; w < NW; w++) xm[w] = node[w];
-                    if (s == 1) {
-                        uint32_t m[NW];
-                        mask_step<POL, NW>(mk, g, m, pp);
-#pragma unroll
-                        for (int w = 0; w < NW; w++) xm[w] ^= m[w];
-                    }
-                    chain_step<POL, NW>(cxs[s], ms256, g, xm, node, pp);
-                } else if constexpr (kCtx) {
-                    chain_step<POL, NW>(cxs[s], ms256, g, node, node, pp);
-                } else {
-                    hashF_p<P, POL>(ms256, make_adrs(0, tree, s == 0 ? T_FORS_PRF : T_FORS_TREE, kp, 0, g), node,
-                                    node, pp, s == 0 ? nullptr : kb.pk_seed);
-                }
-                if (s == 0 && t == gs) store_be<NW>(sf, node);
-            }
+            leaf.hash(kb, ms256, skseed, tree, kp, g, node, t == gs ? sf : nullptr, pp);
             if (t == (gs ^ 1u)) store_be<NW>(sf + P::N, node);
             // merge with stacked left siblings while this node is a right child
             uint32_t z = 0, idx = t;
@@ -239,6 +254,80 @@ __global__ void __launch_bounds__(256) fors_kernel(const KeyBlock* __restrict__ 
     }
 }
 
+// FORS_Sign for batches too small to fill the GPU with lane groups: a thread
+// per leaf, T trees to a block (of T 2^a threads), the levels merged in
+// shared memory.  A lane group of 32 is as many warp instructions, but each
+// lane builds 2^a / 32 leaves and their subtree in series; here a tree takes
+// two leaf hashes and a node hashes of latency.
+template <class P, int POL, int T>
+__global__ void __launch_bounds__(T << P::A) fors_wide_kernel(const KeyBlock* __restrict__ keys,
+                                                              const MsgInfo* __restrict__ infos, uint32_t count,
+                                                              uint8_t* __restrict__ sigs,
+                                                              uint32_t* __restrict__ fors_roots, uint32_t one,
+                                                              uint32_t guard) {
+    if (blockIdx.x == guard) { wait_previous(); return; }
+    constexpr int NW = P::NW, A = P::A, K = P::K;
+    __shared__ uint32_t sh[(T << A) * NW];
+    const uint32_t t = threadIdx.x;
+    // this thread's tree at level z: T << (A - z) nodes of the block's trees, in tree order
+    auto hash_tree = [&](uint32_t local) { return (uint64_t)blockIdx.x * T + local; };
+    {
+        const uint64_t g = hash_tree(t >> A);
+        const uint32_t m = (uint32_t)(g / K), i = (uint32_t)(g % K), l = t & ((1u << A) - 1u);
+        const uint32_t key = m < count ? infos[m].key : KEY_INVALID;
+        if (key != KEY_INVALID) {
+            const KeyBlock& kb = keys[key];
+            const uint64_t tree = infos[m].idx_tree;
+            const uint32_t kp = infos[m].idx_leaf, gs = infos[m].fors_idx[i];
+            uint8_t* sf = sigs + (size_t)m * P::SIG_BYTES + P::N + (size_t)i * (A + 1) * P::N;
+            uint32_t ms256[8], skseed[NW], node[NW];
+#pragma unroll
+            for (int w = 0; w < 8; w++) ms256[w] = kb.ms256[w];
+#pragma unroll
+            for (int w = 0; w < NW; w++) skseed[w] = kb.sk_seed[w];
+            const Pipes<POL> pp(one);
+            const ForsLeaf<P, POL> leaf(kb, ms256, tree, kp, pp);
+            leaf.hash(kb, ms256, skseed, tree, kp, (i << A) + l, node, l == gs ? sf : nullptr, pp);
+            if (l == (gs ^ 1u)) store_be<NW>(sf + P::N, node);
+#pragma unroll
+            for (int w = 0; w < NW; w++) sh[t * NW + w] = node[w];
+        }
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int z = 1; z <= A; z++) {
+        const bool mine = t < ((uint32_t)T << (A - z));
+        uint32_t node[NW];
+        if (mine) {
+            const uint64_t g = hash_tree(t >> (A - z));
+            const uint32_t m = (uint32_t)(g / K), i = (uint32_t)(g % K), l = t & ((1u << (A - z)) - 1u);
+            const uint32_t key = m < count ? infos[m].key : KEY_INVALID;
+            if (key != KEY_INVALID) {
+                const KeyBlock& kb = keys[key];
+                uint32_t lr[2 * NW];
+#pragma unroll
+                for (int w = 0; w < 2 * NW; w++) lr[w] = sh[2 * t * NW + w];
+                hashH_p<P, POL>(kb.ms256, kb.ms512,
+                                make_adrs(0, infos[m].idx_tree, T_FORS_TREE, infos[m].idx_leaf, z, (i << (A - z)) + l),
+                                lr, node, Pipes<POL>(one), kb.pk_seed);
+                const uint32_t gs = infos[m].fors_idx[i];
+                if (z < A && l == ((gs >> z) ^ 1u))
+                    store_be<NW>(sigs + (size_t)m * P::SIG_BYTES + P::N + ((size_t)i * (A + 1) + 1 + z) * P::N, node);
+                if (z == A) {
+#pragma unroll
+                    for (int w = 0; w < NW; w++) fors_roots[(size_t)g * NW + w] = node[w];
+                }
+            }
+        }
+        __syncthreads();
+        if (mine) {
+#pragma unroll
+            for (int w = 0; w < NW; w++) sh[t * NW + w] = node[w];
+        }
+        __syncthreads();
+    }
+}
+
 // PK_FORS = T_k(FORS_ROOTS(layer 0, idx_tree, keypair idx_leaf), roots), 32
 // messages per block (kern_tl.cuh).
 template <class P>
@@ -246,7 +335,9 @@ __global__ void __launch_bounds__(TlShape<P>::THREADS) fors_pk_kernel(const KeyB
                                                                       const MsgInfo* __restrict__ infos,
                                                                       uint32_t count,
                                                                       uint32_t* __restrict__ fors_roots,
-                                                                      uint32_t* __restrict__ pk_fors) {
+                                                                      uint32_t* __restrict__ pk_fors,
+                                                                      uint32_t guard) {
+    if (blockIdx.x == guard) { wait_previous(); return; }
     constexpr int NW = P::NW;
     __shared__ __align__(16) uint32_t smem[TlShape<P>::SMEM_WORDS];
     const uint32_t m = blockIdx.x * 32 + (threadIdx.x & 31);

@@ -322,43 +322,57 @@ struct ByteSha {
 // ------------------------------------------------------------- keyprep
 // KeyBlock from a key buffer: sign keys are SK.seed||SK.prf||PK.seed||PK.root
 // (4n); verify keys are PK.seed||PK.root (2n).  The midstates are the SHA-2
-// state after the first block BlockPad(PK.seed).
+// state after the first block BlockPad(PK.seed).  At n = 24 / 32 two threads
+// share a key, one per midstate: with few keys the launch is one thread's
+// latency.
 template <class P>
 __global__ void keyprep_kernel(const uint8_t* __restrict__ in, uint32_t num_keys, int from_pk,
                                KeyBlock* __restrict__ out) {
-    const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
+    constexpr int NW = P::NW, TPK = P::BIG ? 2 : 1;
+    const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, k = t / TPK;
     if (k >= num_keys) return;
-    KeyBlock kb;
-    for (int i = 0; i < 64; i++) reinterpret_cast<uint32_t*>(&kb)[i] = 0;
-    constexpr int NW = P::NW;
-    if (from_pk) {
-        const uint8_t* p = in + (size_t)k * 2 * P::N;
-        load_be_unaligned<NW>(p, kb.pk_seed);
-        load_be_unaligned<NW>(p + P::N, kb.pk_root);
+    KeyBlock& kb = out[k];
+    const uint8_t* pk = in + (from_pk ? (size_t)k * 2 * P::N : (size_t)k * 4 * P::N + 2 * P::N);
+    uint32_t seed[8];
+#pragma unroll
+    for (int i = 0; i < 8; i++) seed[i] = 0;
+    load_be_unaligned<NW>(pk, seed);
+    if (t % TPK == 0) {
+        uint32_t v[8];
+#pragma unroll
+        for (int i = 0; i < 8; i++) { kb.pk_seed[i] = seed[i]; kb.pad[i] = 0; v[i] = 0; }
+        load_be_unaligned<NW>(pk + P::N, v);
+#pragma unroll
+        for (int i = 0; i < 8; i++) { kb.pk_root[i] = v[i]; v[i] = 0; }
+        if (!from_pk) load_be_unaligned<NW>(pk - 2 * P::N, v);
+#pragma unroll
+        for (int i = 0; i < 8; i++) { kb.sk_seed[i] = v[i]; v[i] = 0; }
+        if (!from_pk) load_be_unaligned<NW>(pk - P::N, v);
+#pragma unroll
+        for (int i = 0; i < 8; i++) { kb.sk_prf[i] = v[i]; v[i] = seed[i]; }
+        if constexpr (!P::SHAKE) {    // the SHAKE hashes take PK.seed itself
+            uint32_t W[16];
+#pragma unroll
+            for (int i = 0; i < 16; i++) W[i] = (i < NW) ? seed[i] : 0u;
+            sha256_iv(v);
+            sha256_compress_rolled(v, W);
+        }
+#pragma unroll
+        for (int i = 0; i < 8; i++) kb.ms256[i] = v[i];
+        if constexpr (!P::BIG) {
+#pragma unroll
+            for (int i = 0; i < 16; i++) kb.ms512[i] = 0;
+        }
     } else {
-        const uint8_t* p = in + (size_t)k * 4 * P::N;
-        load_be_unaligned<NW>(p, kb.sk_seed);
-        load_be_unaligned<NW>(p + P::N, kb.sk_prf);
-        load_be_unaligned<NW>(p + 2 * P::N, kb.pk_seed);
-        load_be_unaligned<NW>(p + 3 * P::N, kb.pk_root);
-    }
-    if constexpr (P::SHAKE) {         // the SHAKE hashes take PK.seed itself
-        for (int i = 0; i < 8; i++) kb.ms256[i] = (i < NW) ? kb.pk_seed[i] : 0u;
-    } else {
-        uint32_t W[16];
-        for (int i = 0; i < 16; i++) W[i] = (i < NW) ? kb.pk_seed[i] : 0u;
-        sha256_iv(kb.ms256);
-        sha256_compress_rolled(kb.ms256, W);
-    }
-    if constexpr (P::BIG) {
         uint32_t blk[32];
-        for (int i = 0; i < 32; i++) blk[i] = (i < NW) ? kb.pk_seed[i] : 0u;
+#pragma unroll
+        for (int i = 0; i < 32; i++) blk[i] = (i < NW) ? seed[i] : 0u;
         uint64_t s[8];
         sha512_iv(s);
         sha512_compress_w32(s, blk);
+#pragma unroll
         for (int i = 0; i < 8; i++) { kb.ms512[2 * i] = (uint32_t)(s[i] >> 32); kb.ms512[2 * i + 1] = (uint32_t)s[i]; }
     }
-    out[k] = kb;
 }
 
 // ------------------------------------------------------------- message stage
@@ -538,9 +552,9 @@ struct MsgWarp {
 template <class P>
 __device__ __forceinline__ void message_warp(MsgWarp<P>& sm, uint32_t m, const KeyBlock* __restrict__ keys,
                                              uint32_t num_keys, const uint32_t* __restrict__ key_idx,
-                                             const uint8_t* __restrict__ msgs, const uint64_t* __restrict__ off,
-                                             uint8_t* __restrict__ sigs, MsgInfo* __restrict__ infos,
-                                             uint32_t* __restrict__ status, int verify,
+                                             const uint8_t* __restrict__ msgs, const uint64_t* __restrict__ lens,
+                                             const uint64_t* __restrict__ off, uint8_t* __restrict__ sigs,
+                                             MsgInfo* __restrict__ infos, uint32_t* __restrict__ status, int verify,
                                              const uint8_t* __restrict__ prefix, uint32_t plen, int msb_first) {
     using S = MsgWarp<P>;
     constexpr int NW = P::NW, N = P::N, DW = S::DW, BW = S::BW, B = S::B, WKW = S::WKW;
@@ -566,8 +580,19 @@ __device__ __forceinline__ void message_warp(MsgWarp<P>& sm, uint32_t m, const K
         return;
     }
     const KeyBlock& kb = keys[key];
-    const uint8_t* M = msgs + off[m];
-    const uint64_t mlen = off[m + 1] - off[m];
+    // the message's offset: up to kSumLens messages, the warp sums the lengths
+    // before it and no launch is needed for a prefix sum (off is null)
+    uint64_t before = 0;
+    if (off) {
+        before = off[m];
+    } else {
+#pragma unroll 4
+        for (uint32_t i = lane; i < m; i += 32) before += lens[i];
+#pragma unroll
+        for (int w = 16; w > 0; w >>= 1) before += __shfl_xor_sync(0xFFFFFFFFu, before, w);
+    }
+    const uint8_t* M = msgs + before;
+    const uint64_t mlen = lens[m];
 
     uint32_t st[DW], outer[DW];
 #pragma unroll
@@ -750,14 +775,14 @@ constexpr int kMsgWarpsPerBlock = 2;
 template <class P>
 __global__ void __launch_bounds__(32 * kMsgWarpsPerBlock)
     message_warp_kernel(const KeyBlock* __restrict__ keys, uint32_t num_keys, const uint32_t* __restrict__ key_idx,
-                        const uint8_t* __restrict__ msgs, const uint64_t* __restrict__ off, uint32_t count,
-                        uint8_t* __restrict__ sigs, MsgInfo* __restrict__ infos, uint32_t* __restrict__ status,
+                        const uint8_t* __restrict__ msgs, const uint64_t* __restrict__ lens,
+                        const uint64_t* __restrict__ off, uint32_t count, uint8_t* __restrict__ sigs, MsgInfo* __restrict__ infos, uint32_t* __restrict__ status,
                         int verify, const uint8_t* __restrict__ prefix, uint32_t plen, int msb_first) {
     __shared__ __align__(16) MsgWarp<P> sm[kMsgWarpsPerBlock];
     const uint32_t warp = threadIdx.x >> 5;
     const uint32_t m = blockIdx.x * kMsgWarpsPerBlock + warp;
     if (m >= count) return;                        // the whole warp
-    message_warp<P>(sm[warp], m, keys, num_keys, key_idx, msgs, off, sigs, infos, status, verify, prefix, plen,
+    message_warp<P>(sm[warp], m, keys, num_keys, key_idx, msgs, lens, off, sigs, infos, status, verify, prefix, plen,
                     msb_first);
 }
 

@@ -28,6 +28,7 @@ __global__ void __launch_bounds__(128, MINB) bleaf_kernel(const KeyBlock* __rest
                                                           const MsgInfo* __restrict__ infos, uint32_t count,
                                                           uint32_t* __restrict__ leafv, uint32_t* __restrict__ chk,
                                                           uint32_t ck, uint32_t layers, uint32_t one) {
+    allow_next();
     constexpr int NW = P::NW, LV = P::LEAVES;
     const uint64_t gid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t per_msg = layers * LV;
@@ -72,6 +73,7 @@ __global__ void __launch_bounds__(TlShape<P>::THREADS) bleaf_from_ends_kernel(co
                                                                               const DedupDesc* __restrict__ desc,
                                                                               uint32_t ndesc,
                                                                               uint32_t* __restrict__ nodes_u) {
+    allow_next();
     constexpr int NW = P::NW, LV = P::LEAVES, LEN = P::LEN;
     static_assert(LV % 32 == 0, "a block is 32 leaves of one tree");
     __shared__ __align__(16) uint32_t smem[TlShape<P>::SMEM_WORDS];
@@ -149,6 +151,7 @@ __global__ void __launch_bounds__(kMergeThreads) bmerkle_kernel(const KeyBlock* 
                                                                 const uint32_t* __restrict__ leafv,
                                                                 uint8_t* __restrict__ sigs,
                                                                 uint32_t* __restrict__ roots, uint32_t layers) {
+    allow_next();
     constexpr int NW = P::NW, LV = P::LEAVES;
     __shared__ uint32_t sh[LV * NW];
     const uint32_t m = blockIdx.x / layers;

@@ -240,6 +240,7 @@ __global__ void __launch_bounds__(128, MINB) tree_kernel(const KeyBlock* __restr
                                                    uint8_t* __restrict__ sigs, uint32_t* __restrict__ roots,
                                                    uint32_t* __restrict__ chk, uint32_t ck, uint32_t layers,
                                                    uint32_t one) {
+    allow_next();
     constexpr int NW = P::NW, LV = P::LEAVES;
     const uint32_t gid = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t lane = threadIdx.x & 31;
@@ -292,6 +293,7 @@ __global__ void __launch_bounds__(128) chains_kernel(const KeyBlock* __restrict_
                                                      uint32_t ck, uint32_t layers,
                                                      const DedupDesc* __restrict__ desc, uint32_t ndesc,
                                                      uint32_t* __restrict__ chk_u, uint32_t one) {
+    allow_next();
     constexpr int NW = P::NW, LV = P::LEAVES, LEN = P::LEN;
     const uint64_t gid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t per_msg = layers * LV * LEN;
@@ -380,6 +382,7 @@ __global__ void __launch_bounds__(TlShape<P>::THREADS) leaves_kernel(const KeyBl
                                                                      uint32_t* __restrict__ roots, uint32_t layers,
                                                                      const DedupDesc* __restrict__ desc,
                                                                      uint32_t ndesc, uint32_t* __restrict__ nodes_u) {
+    allow_next();
     constexpr int NW = P::NW, LV = P::LEAVES, LEN = P::LEN;
     __shared__ __align__(16) uint32_t smem[TlShape<P>::SMEM_WORDS];
     const uint32_t lane = threadIdx.x & 31;

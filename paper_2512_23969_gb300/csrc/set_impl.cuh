@@ -14,6 +14,25 @@
 
 namespace hs {
 
+// Launch on s; beside = true: the launch may start beside the previous one
+// of the stream (hs_common.cuh), with the guard block that makes it end after
+// it.  The kernel's last parameter is the guard's block index.
+template <class... K, class... A>
+inline cudaError_t launch_beside(bool beside, void (*kernel)(K...), uint32_t grid, uint32_t threads, cudaStream_t s,
+                                 A... args) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid + (beside ? 1u : 0u));
+    cfg.blockDim = dim3(threads);
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = beside ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args..., beside ? grid : kNoGuard);
+    return e == cudaSuccess ? cudaGetLastError() : e;
+}
+
 template <class P>
 struct SetImpl {
     // XMSS trees wider than a warp (s sets) take the two-launch form of
@@ -25,7 +44,8 @@ struct SetImpl {
     static uint32_t own_layers(const Batch& b) { return b.dedup_layer ? b.dedup_layer : (uint32_t)P::D; }
 
     static cudaError_t keyprep(const Batch& b, bool from_pk, cudaStream_t s) {
-        const uint32_t T = 128, G = (b.num_keys + T - 1) / T;
+        const uint64_t threads = (uint64_t)b.num_keys * (P::BIG ? 2 : 1);
+        const uint32_t T = 128, G = (uint32_t)((threads + T - 1) / T);
         keyprep_kernel<P><<<G, T, 0, s>>>(b.keys_in, b.num_keys, from_pk ? 1 : 0, b.keys);
         return cudaGetLastError();
     }
@@ -33,7 +53,8 @@ struct SetImpl {
         if constexpr (!P::SHAKE) {
             if (b.msg_warp) {                               // a warp per message
                 const uint32_t T = 32 * kMsgWarpsPerBlock, G = (b.count + kMsgWarpsPerBlock - 1) / kMsgWarpsPerBlock;
-                message_warp_kernel<P><<<G, T, 0, s>>>(b.keys, b.num_keys, b.key_idx, b.msgs, b.offsets, b.count,
+                message_warp_kernel<P><<<G, T, 0, s>>>(b.keys, b.num_keys, b.key_idx, b.msgs, b.lens,
+                                                       needs_offsets(b) ? b.offsets : nullptr, b.count,
                                                        b.sigs, b.infos, b.status, verify ? 1 : 0, b.prefix,
                                                        b.prefix_len, b.fips ? 1 : 0);
                 return cudaGetLastError();
@@ -50,15 +71,31 @@ struct SetImpl {
         const uint64_t threads = (uint64_t)b.count * P::K * LPT;
         const uint32_t T = 256;
         const uint32_t G = (uint32_t)((threads + T - 1) / T);
-        fors_kernel<P, fors_pol<P>(), LPT><<<G, T, 0, s>>>(b.keys, b.infos, b.count, b.sigs, b.fors_roots, 1u);
-        return cudaGetLastError();
+        return launch_beside(b.beside, fors_kernel<P, fors_pol<P>(), LPT>, G, T, s, (const KeyBlock*)b.keys,
+                             (const MsgInfo*)b.infos, b.count, b.sigs, b.fors_roots, 1u);
+    }
+    // The widest form (the knob's value 32 at the f sets): a thread per leaf
+    // while that is the faster one, else lane groups of 32.  A block of the
+    // former holds its 2^a threads' registers while a few lanes climb the
+    // upper levels, so at a = 8 / 9 it pays for a few trees per SM only:
+    // measured on GB300, 256f 1 message 215 -> 61 us, 96 messages 632 -> 987;
+    // 192f 123 -> 47 and 360 -> 397; at a = 6 (128f) the blocks are small,
+    // 30 -> 20 us and 76 -> 65.
+    static cudaError_t fors_widest(const Batch& b, cudaStream_t s) {
+        constexpr int T = P::A < 7 ? 1 << (7 - P::A) : 1;          // trees per block: at least 128 threads
+        const uint64_t trees = (uint64_t)b.count * P::K;
+        if constexpr (P::A >= 8) {
+            if (trees > (uint64_t)sm_count() * (P::A == 8 ? 6 : 4)) return fors<32>(b, s);
+        }
+        return launch_beside(b.beside, fors_wide_kernel<P, fors_pol<P>(), T>, (uint32_t)((trees + T - 1) / T), T << P::A,
+                             s, (const KeyBlock*)b.keys, (const MsgInfo*)b.infos, b.count, b.sigs, b.fors_roots, 1u);
     }
     static cudaError_t fors_pk(const Batch& b, cudaStream_t s) {
-        fors_pk_kernel<P><<<(b.count + 31) / 32, TlShape<P>::THREADS, 0, s>>>(b.keys, b.infos, b.count, b.fors_roots, b.pk_fors);
-        return cudaGetLastError();
+        return launch_beside(b.beside, fors_pk_kernel<P>, (b.count + 31) / 32, TlShape<P>::THREADS, s,
+                             (const KeyBlock*)b.keys, (const MsgInfo*)b.infos, b.count, b.fors_roots, b.pk_fors);
     }
     template <int MINB, int POL = tree_pol<P>(), int ILP = 1>
-    static cudaError_t tree(const Batch& b, cudaStream_t s) {
+    static cudaError_t tree(const Batch& b, BesideFn beside, cudaStream_t s) {
         const uint32_t L = own_layers(b);
         const uint64_t threads = (uint64_t)b.count * L * P::LEAVES;
         const uint32_t T = 128;
@@ -70,12 +107,21 @@ struct SetImpl {
         if constexpr (kWide) {
             bleaf_kernel<P, POL, MINB, ILP><<<G, T, 0, s>>>(b.keys, b.infos, b.count, b.leafv, b.chk, b.ck, L, 1u);
             e = cudaGetLastError();
-            return e == cudaSuccess ? merge(b, s) : e;
+            if (e == cudaSuccess && beside) e = beside(b, 0, s);
+            if (e == cudaSuccess) e = merge(b, s);
+            if (e == cudaSuccess && beside) e = beside(b, 1, s);
         } else {
             tree_kernel<P, POL, MINB, ILP><<<G, T, 0, s>>>(b.keys, b.infos, b.count, b.sigs, b.roots, b.chk, b.ck,
                                                         L, 1u);
-            return cudaGetLastError();
+            e = cudaGetLastError();
+            if (e == cudaSuccess && beside) e = beside(b, 0, s);
+            if (e == cudaSuccess && beside) {           // T_k reads what the launch before it writes
+                Batch after = b;
+                after.beside = false;
+                e = beside(after, 1, s);
+            }
         }
+        return e;
     }
     // The descriptions of the trees this call builds for several messages.
     static cudaError_t describe_shared(const Batch& b, cudaStream_t s) {
@@ -131,11 +177,13 @@ struct SetImpl {
         return build_trees(keys, desc, (uint32_t)trees, nodes, chk, ck, s);
     }
     // Chain-parallel form: the messages' own trees and the ndesc trees of
-    // desc in the same launches (either may be none).
+    // desc in the same launches (either may be none).  T_len's launch starts
+    // after FORS_Sign's (it waits for the whole stream), so T_k beside it
+    // finds the FORS roots complete.
     static cudaError_t split_trees(const KeyBlock* keys, const MsgInfo* infos, uint32_t count, uint32_t L,
                                    uint32_t* ends, uint32_t* chk, uint32_t ck, const DedupDesc* desc, uint32_t ndesc,
                                    uint32_t* nodes_u, uint32_t* chk_u, uint32_t* leafv, uint8_t* sigs,
-                                   uint32_t* roots, cudaStream_t s) {
+                                   uint32_t* roots, const Batch* b, BesideFn beside, cudaStream_t s) {
         const uint32_t T = 128;
         const uint64_t own = (uint64_t)count * L * P::LEAVES, shared = (uint64_t)ndesc * P::LEAVES;
         const uint64_t chains = (own + shared) * P::LEN;
@@ -143,24 +191,29 @@ struct SetImpl {
         chains_kernel<P, tree_pol<P>()><<<(uint32_t)((chains + T - 1) / T), T, 0, s>>>(
             keys, infos, count, ends, chk, ck, L, desc, ndesc, chk_u, 1u);
         cudaError_t e = cudaGetLastError();
+        if (e == cudaSuccess && beside) e = beside(*b, 0, s);
         if (e != cudaSuccess) return e;
         const uint32_t G = (uint32_t)((own + 31) / 32 + (shared + 31) / 32);
         if constexpr (kWide) {
             bleaf_from_ends_kernel<P><<<G, TlShape<P>::THREADS, 0, s>>>(keys, infos, count, ends, leafv, L, desc,
                                                                         ndesc, nodes_u);
-            if ((e = cudaGetLastError()) != cudaSuccess || ndesc == 0) return e;
+            e = cudaGetLastError();
+            if (e == cudaSuccess && beside) e = beside(*b, 1, s);
+            if (e != cudaSuccess || ndesc == 0) return e;
             wtree_merge_kernel<P><<<ndesc, kMergeThreads, 0, s>>>(keys, desc, ndesc, nodes_u);
+            return cudaGetLastError();
         } else {
             leaves_kernel<P><<<G, TlShape<P>::THREADS, 0, s>>>(keys, infos, count, ends, sigs, roots, L, desc, ndesc,
                                                                nodes_u);
+            e = cudaGetLastError();
+            return e == cudaSuccess && beside ? beside(*b, 1, s) : e;
         }
-        return cudaGetLastError();
     }
-    static cudaError_t tree_split(const Batch& b, cudaStream_t s) {
+    static cudaError_t tree_split(const Batch& b, BesideFn beside, cudaStream_t s) {
         cudaError_t e = describe_shared(b, s);
         if (e == cudaSuccess)
             e = split_trees(b.keys, b.infos, b.count, own_layers(b), b.ends, b.chk, b.ck, b.desc, b.max_uniq,
-                            b.nodes_u, b.chk_u, b.leafv, b.sigs, b.roots, s);
+                            b.nodes_u, b.chk_u, b.leafv, b.sigs, b.roots, &b, beside, s);
         if constexpr (kWide) {
             if (e == cudaSuccess) e = merge(b, s);
         }
@@ -247,7 +300,7 @@ struct SetImpl {
             }
             if (e == cudaSuccess)
                 e = split_trees(kbs, nullptr, 0, 0, ends, nullptr, 0, desc, count, nodes, nullptr, nullptr, nullptr,
-                                nullptr, s);
+                                nullptr, nullptr, nullptr, s);
             if (e == cudaSuccess) {
                 const uint64_t bytes = (uint64_t)count * 4 * P::N;
                 keygen_out_kernel<P><<<(uint32_t)((bytes + T - 1) / T), T, 0, s>>>(seeds, count, nodes, pk, sk);
@@ -283,13 +336,13 @@ struct TreeVariants {
         if (MB_ALT != 0 && minb == MB_ALT && pol == PD && ilp == 1) return true;
         return kAlts && minb == 0 && ((pol == PA && ilp == 1) || (pol == PD && ilp == 2));
     }
-    static cudaError_t run(const Batch& b, int minb, int pol, int ilp, cudaStream_t s) {
-        if (minb == 0 && pol == PD && ilp == 1) return SetImpl<P>::template tree<1, PD, 1>(b, s);
+    static cudaError_t run(const Batch& b, int minb, int pol, int ilp, BesideFn beside, cudaStream_t s) {
+        if (minb == 0 && pol == PD && ilp == 1) return SetImpl<P>::template tree<1, PD, 1>(b, beside, s);
         if constexpr (MB_ALT != 0)
-            if (minb == MB_ALT && pol == PD && ilp == 1) return SetImpl<P>::template tree<MB_ALT, PD, 1>(b, s);
+            if (minb == MB_ALT && pol == PD && ilp == 1) return SetImpl<P>::template tree<MB_ALT, PD, 1>(b, beside, s);
         if constexpr (kAlts) {
-            if (minb == 0 && pol == PA && ilp == 1) return SetImpl<P>::template tree<1, PA, 1>(b, s);
-            if (minb == 0 && pol == PD && ilp == 2) return SetImpl<P>::template tree<1, PD, 2>(b, s);
+            if (minb == 0 && pol == PA && ilp == 1) return SetImpl<P>::template tree<1, PA, 1>(b, beside, s);
+            if (minb == 0 && pol == PD && ilp == 2) return SetImpl<P>::template tree<1, PD, 2>(b, beside, s);
         }
         return cudaErrorInvalidValue;
     }

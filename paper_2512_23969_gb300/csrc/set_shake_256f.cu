@@ -14,7 +14,7 @@ cudaError_t fors_variant(const Batch& b, int lpt, cudaStream_t s) {
     case 4: return SetImpl<P>::fors<4>(b, s);
     case 8: return SetImpl<P>::fors<8>(b, s);
     case 16: return SetImpl<P>::fors<16>(b, s);
-    case 32: return SetImpl<P>::fors<32>(b, s);
+    case 32: return SetImpl<P>::fors_widest(b, s);
     }
     return cudaErrorInvalidValue;
 }
