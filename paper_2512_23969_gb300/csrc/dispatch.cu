@@ -144,6 +144,19 @@ bool msg_warp(int pset, uint32_t count) {
     return !is_shake(pset) && count < (uint32_t)std::max(0, tune_get(pset, 8));
 }
 
+// Verification: the walk over every digit's chain ends runs 16 times the
+// chain steps in parallel in place of d serial chain launches, so it pays up
+// to a number of chains per layer that hardly depends on the set.  Measured
+// on GB300, walk against layer by layer (us): 128f 1 signature 536 / 1129,
+// 96 1064 / 1153, 128 1227 / 1151; 256f 1 1413 / 1971, 64 2101 / 2118, 96
+// 2367 / 2116; 128s 96 474 / 491, 128 527 / 491; shake-128f 64 2475 / 2957,
+// 96 3089 / 2956.
+bool verify_walk(int pset, uint32_t count) {
+    SetShape sh{};
+    if (!set_shape(pset, &sh)) return false;
+    return (uint64_t)count * (2 * sh.n + 3) <= (is_shake(pset) ? 3000u : 3500u);
+}
+
 // SM count of the current device (looked up once per device).
 int sm_count() {
     static std::atomic<int> cache[64];

@@ -134,7 +134,9 @@ static void scratch_layout(const Batch& b, const SetInfo& s, size_t sz[kRegions]
     sz[i++] = mu * 2 * s.leaves * nw * 4 +                           // nodes_u, then chk_u
               (b.ck ? mu * s.leaves * s.len * (16 / b.ck) * nw * 4 : 0);
     sz[i++] = s.leaves > 32 ? cnt * s.d * s.leaves * nw * 4 : 0;     // leafv
-    sz[i++] = b.verify ? 16 * (size_t)s.d * 4 + 2 * cnt * s.len * 4 : 0;   // vcnt, vsitem, vorder
+    sz[i++] = !b.verify ? 0                                          // vends, or vcnt, vsitem, vorder
+              : b.walk ? cnt * s.d * s.len * 16 * nw * 4
+                       : 16 * (size_t)s.d * 4 + 2 * cnt * s.len * 4;
     *n = i;
 }
 
@@ -178,9 +180,10 @@ void carve_scratch(Batch& b, void* base) {
     b.chk = b.ck ? reinterpret_cast<uint32_t*>(r[7]) : nullptr;
     b.ends = (b.split || b.verify) ? reinterpret_cast<uint32_t*>(r[8]) : nullptr;
     b.leafv = s.leaves > 32 ? reinterpret_cast<uint32_t*>(r[12]) : nullptr;
-    b.vcnt = b.verify ? reinterpret_cast<uint32_t*>(r[13]) : nullptr;
-    b.vsitem = b.verify ? b.vcnt + 16 * s.d : nullptr;
-    b.vorder = b.verify ? b.vsitem + (size_t)b.count * s.len : nullptr;
+    b.vends = b.walk ? reinterpret_cast<uint32_t*>(r[13]) : nullptr;
+    b.vcnt = b.verify && !b.walk ? reinterpret_cast<uint32_t*>(r[13]) : nullptr;
+    b.vsitem = b.vcnt ? b.vcnt + 16 * s.d : nullptr;
+    b.vorder = b.vcnt ? b.vsitem + (size_t)b.count * s.len : nullptr;
     b.mj_id = b.dedup_layer ? reinterpret_cast<uint32_t*>(r[9]) : nullptr;
     if (b.cached) return;             // nodes_u / chk_u belong to the keyset
     b.desc = b.max_uniq ? reinterpret_cast<DedupDesc*>(r[10]) : nullptr;
@@ -485,6 +488,7 @@ static hs_status run_batch(const hs_keyset* ks, bool verify, hs_params p, const 
     b.split = !verify && tree_split(p, count);
     b.msg_warp = msg_warp(p, count);
     b.verify = verify;
+    b.walk = verify && verify_walk(p, count);
     if (ks && ks->layers) {
         b.dedup_layer = ks->first_layer;
         b.cached = true;
@@ -505,9 +509,10 @@ static hs_status run_batch(const hs_keyset* ks, bool verify, hs_params p, const 
                          (h_sig ? align256(sig_total) : 0) + (h_ok ? align256(count) : 0) + align256(plen);
     void* base = nullptr;
     e = cudaMallocFromPoolAsync(&base, scratch + stage, d->pool, s);
-    if (e == cudaErrorMemoryAllocation && b.max_uniq) {      // the shared trees are extra scratch: without them
-        cudaGetLastError();
+    if (e == cudaErrorMemoryAllocation && (b.max_uniq || b.walk)) {
+        cudaGetLastError();                       // without the shared trees or every digit's ends: less scratch
         drop_dedup(b);
+        b.walk = false;
         scratch = need();
         e = cudaMallocFromPoolAsync(&base, scratch + stage, d->pool, s);
     }

@@ -33,6 +33,8 @@ struct Batch {
     uint32_t* vcnt;           // verify: 16 chain-length buckets per layer (16 D words)
     uint32_t* vsitem;         // verify: count * LEN words, steps << 28 | rank
     uint32_t* vorder;         // verify: count * LEN words, chains sorted by length
+    bool walk;                // verify: the form for few signatures (kern_verify.cuh)
+    uint32_t* vends;          // walk: chain ends for every digit, count * D * LEN * 16 * NW words
     // scratch
     KeyBlock* keys;           // num_keys
     uint64_t* offsets;        // count + 1
@@ -181,6 +183,9 @@ cudaError_t launch_tree(const Batch& b, cudaStream_t s);
 // captured.
 cudaError_t launch_sign_trees(const Batch& b, cudaStream_t s);
 cudaError_t launch_wots(const Batch& b, cudaStream_t s);
+// Whether a verification of 'count' signatures takes the form for few
+// (kern_verify.cuh).
+bool verify_walk(int pset, uint32_t count);
 cudaError_t launch_verify(const Batch& b, cudaStream_t s);
 cudaError_t launch_keygen(int pset, const uint8_t* seeds, uint32_t count, uint8_t* pk, uint8_t* sk,
                           cudaStream_t s);

@@ -146,8 +146,8 @@ __device__ __forceinline__ void tl_rounds512(uint64_t st[8], const uint64_t* row
 }
 
 // T_l of l = L n-byte values for the 32 items of a block (lane = item, the
-// same item in every warp); TlShape<P>::THREADS threads, all of them call
-// it.  p: the item's payload, complete before the launch; active: the lane
+// same item in every warp); TlShape<P>::THREADS threads or more, all of them
+// call it.  p: the item's payload, complete before the launch; active: the lane
 // has an item (others read nothing).  The result is in warp 0.  ms: the
 // midstate (SHAKE: PK.seed); pks: PK.seed (robust sets: the payload is
 // masked in place first).
@@ -156,7 +156,7 @@ __device__ __forceinline__ void tl_group(const uint32_t* ms, const Adrs& a, uint
                                          const uint32_t* pks, uint32_t* smem, uint32_t* out) {
     constexpr int NW = P::NW, PW = L * NW;
     if constexpr (P::SHAKE) {
-        if (active) {
+        if (active && threadIdx.x < 32) {
             TStreamP<P> ts;
             ts.init(ms, a);
 #pragma unroll 1
@@ -190,7 +190,7 @@ __device__ __forceinline__ void tl_group(const uint32_t* ms, const Adrs& a, uint
                     if constexpr (P::BIG) tl_rounds512(st64, reinterpret_cast<const uint64_t*>(rows), lane);
                     else tl_rounds256(st, rows, lane);
                 }
-            } else {
+            } else if (warp <= (uint32_t)S::CH) {
                 const int b = (c + 1) * S::CH + (int)warp - 1;
                 if (b < NB && active) {
                     uint32_t W[P::BIG ? 32 : 16];
@@ -206,6 +206,107 @@ __device__ __forceinline__ void tl_group(const uint32_t* ms, const Adrs& a, uint
         for (int i = 0; i < NW; i++) {
             if constexpr (P::BIG) out[i] = (i & 1) ? (uint32_t)st64[i / 2] : (uint32_t)(st64[i / 2] >> 32);
             else out[i] = st[i];
+        }
+    }
+}
+
+// H of two children for the same 32 items (SHA-2): one block each, warp 1
+// computing the next 16 rounds' schedule while warp 0 runs the current 16.
+// node (warp 0) is one child and receives the parent; right: it is the right
+// child.  sib: the other child (warp 1); nodes: 32 * NW words of shared
+// memory.
+template <class P>
+__device__ __forceinline__ void h_group(const KeyBlock& kb, const Adrs& a, bool right, const uint32_t* sib,
+                                        uint32_t* smem, uint32_t* nodes, uint32_t* node) {
+    constexpr int NW = P::NW, NCH = P::BIG ? 5 : 4, BW = P::BIG ? 32 : 16;
+    constexpr int ROW = 16 * 32 * (P::BIG ? 2 : 1);      // words of 16 rows
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp == 0) {
+#pragma unroll
+        for (int w = 0; w < NW; w++) nodes[w * 32 + lane] = node[w];
+    }
+    __syncthreads();
+    uint32_t W[16], v[8];
+    uint64_t W64[P::BIG ? 16 : 1], v64[P::BIG ? 8 : 1];
+    if (warp == 1) {
+        uint32_t lr[2 * NW], blk[BW];
+#pragma unroll
+        for (int w = 0; w < NW; w++) {
+            const uint32_t n = nodes[w * 32 + lane];
+            lr[w] = right ? sib[w] : n;
+            lr[NW + w] = right ? n : sib[w];
+        }
+        if constexpr (P::ROBUST) mask_regs<P::BIG, NW, 2 * NW>(kb.pk_seed, a, lr);
+        fill_block<BW, 2 * NW>(blk, a, lr);
+        blk[BW - 1] = ((P::BIG ? 128 : 64) + 22 + 8 * NW) * 8;
+#pragma unroll
+        for (int i = 0; i < 16; i++) {
+            if constexpr (P::BIG) W64[i] = ((uint64_t)blk[2 * i] << 32) | blk[2 * i + 1];
+            else W[i] = blk[i];
+        }
+    } else if (warp == 0) {
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+            if constexpr (P::BIG) v64[i] = ((uint64_t)kb.ms512[2 * i] << 32) | kb.ms512[2 * i + 1];
+            else v[i] = kb.ms256[i];
+        }
+    }
+#pragma unroll 1
+    for (int c = -1; c < NCH; c++) {
+        if (warp == 0 && c >= 0) {
+            const uint32_t* rows = smem + (c & 1) * ROW;
+            if constexpr (P::BIG) {
+                const uint64_t* r = reinterpret_cast<const uint64_t*>(rows) + lane;
+#pragma unroll
+                for (int j = 0; j < 16; j++) {
+                    uint64_t &a_ = v64[(16 - j) & 7], &b_ = v64[(17 - j) & 7], &c_ = v64[(18 - j) & 7],
+                             &d_ = v64[(19 - j) & 7], &e_ = v64[(20 - j) & 7], &f_ = v64[(21 - j) & 7],
+                             &g_ = v64[(22 - j) & 7], &h_ = v64[(23 - j) & 7];
+                    const uint64_t t1 = h_ + S1_512(e_) + ((e_ & f_) ^ (~e_ & g_)) + r[j * 32];
+                    const uint64_t t2 = S0_512(a_) + ((a_ & b_) | (c_ & (a_ | b_)));
+                    d_ += t1;
+                    h_ = t1 + t2;
+                }
+            } else {
+                const uint32_t* r = rows + lane;
+#pragma unroll
+                for (int j = 0; j < 16; j++) {
+                    uint32_t &a_ = v[(16 - j) & 7], &b_ = v[(17 - j) & 7], &c_ = v[(18 - j) & 7],
+                             &d_ = v[(19 - j) & 7], &e_ = v[(20 - j) & 7], &f_ = v[(21 - j) & 7],
+                             &g_ = v[(22 - j) & 7], &h_ = v[(23 - j) & 7];
+                    const uint32_t hx = h_ + r[j * 32];
+                    uint32_t dhx = d_ + hx;
+                    asm("" : "+r"(dhx));
+                    const uint32_t s1 = S1_256(e_), ch = ch32(e_, f_, g_);
+                    d_ = dhx + s1 + ch;
+                    h_ = (hx + s1 + ch) + S0_256(a_) + maj32(a_, b_, c_);
+                }
+            }
+        } else if (warp == 1 && c + 1 < NCH) {
+            const int t0 = 16 * (c + 1);
+            uint32_t* rows = smem + ((c + 1) & 1) * ROW;
+#pragma unroll
+            for (int i = 0; i < 16; i++) {
+                if constexpr (P::BIG) {
+                    if (t0 > 0) W64[i] += s1_512(W64[(i + 14) & 15]) + W64[(i + 9) & 15] + s0_512(W64[(i + 1) & 15]);
+                    reinterpret_cast<uint64_t*>(rows)[i * 32 + lane] = W64[i] + c_K512[t0 + i];
+                } else {
+                    if (t0 > 0) W[i] += s1_256(W[(i + 14) & 15]) + W[(i + 9) & 15] + s0_256(W[(i + 1) & 15]);
+                    rows[i * 32 + lane] = W[i] + c_K256[t0 + i];
+                }
+            }
+        }
+        __syncthreads();
+    }
+    if (warp == 0) {
+#pragma unroll
+        for (int i = 0; i < NW; i++) {
+            if constexpr (P::BIG) {
+                const uint64_t s = v64[i / 2] + (((uint64_t)kb.ms512[i & ~1] << 32) | kb.ms512[i | 1]);
+                node[i] = (i & 1) ? (uint32_t)s : (uint32_t)(s >> 32);
+            } else {
+                node[i] = v[i] + kb.ms256[i];
+            }
         }
     }
 }

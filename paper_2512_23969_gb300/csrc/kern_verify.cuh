@@ -35,7 +35,8 @@ template <class P>
 __global__ void __launch_bounds__(128) vfors_kernel(const KeyBlock* __restrict__ keys,
                                                     const MsgInfo* __restrict__ infos, uint32_t count,
                                                     const uint8_t* __restrict__ sigs,
-                                                    uint32_t* __restrict__ fors_roots) {
+                                                    uint32_t* __restrict__ fors_roots, uint32_t guard) {
+    if (blockIdx.x == guard) { wait_previous(); return; }
     constexpr int NW = P::NW, A = P::A, K = P::K;
     const uint64_t gid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const uint64_t m = gid / K;
@@ -264,6 +265,149 @@ __global__ void __launch_bounds__(TlShape<P>::THREADS) vleaf_kernel(const KeyBlo
     if (cnt_next) {                                // the next layer's chains
         __syncthreads();
         count_block<P>(c, smem, m0, min(32u, count - m0), cnt_next, sitem);
+    }
+}
+
+// ---------------------------------------------------------------- few signatures
+// With few signatures a layer's chains and T_len are each one warp's latency,
+// and the layers are serial.  The chains need not be: only the number of
+// steps of a chain depends on the layer below, so the ends of every chain for
+// each of the 16 digits it might have are computed for all layers at once
+// (120 steps a chain in place of 7.5, in parallel), and what remains serial is
+// picking the ends by digit, T_len and the climbs -- one launch that walks the
+// layers of 32 signatures per block.  Pays while the extra steps are cheaper
+// than d chain launches (verify_walk in dispatch.cu).
+
+// End of chain i of layer j of message m for digit d, at
+// [m][j][i][d][NW words]; the longest (d = 0) first.
+template <class P, int POL>
+__global__ void __launch_bounds__(128) vspec_kernel(const KeyBlock* __restrict__ keys,
+                                                    const MsgInfo* __restrict__ infos, uint32_t count,
+                                                    const uint8_t* __restrict__ sigs, uint32_t* __restrict__ vends,
+                                                    uint32_t one) {
+    allow_next();
+    constexpr int NW = P::NW, LEN = P::LEN, D = P::D;
+    const uint64_t gid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const uint64_t per = (uint64_t)count * D * LEN;
+    const uint32_t d = (uint32_t)(gid / per);
+    if (d > 15) return;
+    const uint64_t r = gid % per;
+    const uint32_t m = (uint32_t)(r / (D * LEN)), j = (uint32_t)(r / LEN) % D, i = (uint32_t)(r % LEN);
+    const MsgInfo& info = infos[m];
+    if (info.key == KEY_INVALID) return;
+    const KeyBlock& kb = keys[info.key];
+    const uint64_t tree = layer_tree<P>(info.idx_tree, (int)j);
+    const uint32_t kp = layer_leaf<P>(info.idx_tree, info.idx_leaf, (int)j);
+    uint32_t ms256[8], x[NW];
+#pragma unroll
+    for (int w = 0; w < 8; w++) ms256[w] = kb.ms256[w];
+    load_be<NW>(sigs + (size_t)m * P::SIG_BYTES + P::N + P::FORS_BYTES + (size_t)j * P::LAYER_BYTES +
+                    (size_t)i * P::N, x);
+    const Pipes<POL> pp(one);
+    if constexpr (P::SHAKE) {
+#pragma unroll 1
+        for (uint32_t q = d; q < 15u; q++) hashF_p<P, POL>(ms256, make_adrs(j, tree, T_WOTS_HASH, kp, i, q), x, x, pp);
+    } else {
+        const Adrs ah = make_adrs(j, tree, T_WOTS_HASH, kp, i, 0);
+        ChainCtx cx;
+        MaskCtx<NW> mk;
+        chain_ctx<POL>(ms256, ah, cx, pp);
+        if constexpr (P::ROBUST) mask_ctx<POL, NW>(kb.pk_seed, ah, mk, pp);
+#pragma unroll 1
+        for (uint32_t q = d; q < 15u; q++) chain_step_p<P, POL>(cx, mk, ms256, q, x, x, pp);
+    }
+    uint32_t* e = vends + (r * 16 + d) * NW;
+#pragma unroll
+    for (int w = 0; w < NW; w++) e[w] = x[w];
+}
+
+// PK_FORS, then every layer of 32 signatures, then the comparison.  ends:
+// count * LEN * NW words (the picked ends of the current layer).
+constexpr int kWalkThreads = 256;
+template <class P>
+__global__ void __launch_bounds__(kWalkThreads) vwalk_kernel(const KeyBlock* __restrict__ keys,
+                                                             const MsgInfo* __restrict__ infos, uint32_t count,
+                                                             const uint8_t* __restrict__ sigs,
+                                                             const uint32_t* __restrict__ vends, uint32_t* ends,
+                                                             uint32_t* fors_roots, uint8_t* __restrict__ ok) {
+    constexpr int NW = P::NW, LEN = P::LEN, HP = P::HP, D = P::D;
+    __shared__ __align__(16) uint32_t smem[TlShape<P>::SMEM_WORDS];
+    __shared__ uint32_t nodes[32 * NW], msg[32 * NW], csum[32], valid[32];
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t m0 = blockIdx.x * 32, m = m0 + lane, nmsg = min(32u, count - m0);
+    const uint32_t key = m < count ? infos[m].key : KEY_INVALID;
+    const bool active = key != KEY_INVALID;
+    const MsgInfo& info = infos[active ? m : 0];
+    const KeyBlock& kb = keys[active ? key : 0];
+    const uint64_t idx_tree = info.idx_tree;
+    const uint32_t idx_leaf = info.idx_leaf;
+    const uint32_t* msT = P::BIG ? kb.ms512 : kb.ms256;
+    uint32_t node[NW];
+    if (warp == 0) valid[lane] = active ? 1u : 0u;
+    tl_group<P, P::K>(msT, make_adrs(0, idx_tree, T_FORS_ROOTS, idx_leaf, 0, 0), fors_roots + (size_t)m * P::K * NW,
+                      active, kb.pk_seed, smem, node);
+#pragma unroll 1
+    for (uint32_t j = 0; j < (uint32_t)D; j++) {
+        if (warp == 0) {
+            uint32_t cs = 0;
+#pragma unroll
+            for (int w = 0; w < NW; w++) {
+                msg[lane * NW + w] = node[w];
+#pragma unroll
+                for (int b = 0; b < 8; b++) cs += 15u - ((node[w] >> (28 - 4 * b)) & 15u);
+            }
+            csum[lane] = cs << 4;
+        }
+        __syncthreads();
+        for (uint32_t it = threadIdx.x; it < nmsg * LEN; it += kWalkThreads) {
+            const uint32_t mm = it / LEN, i = it % LEN;
+            if (!valid[mm]) continue;
+            const uint32_t d = i < (uint32_t)P::LEN1 ? (msg[mm * NW + (i >> 3)] >> (28 - 4 * (i & 7))) & 15u
+                                                     : (csum[mm] >> (12 - 4 * (i - P::LEN1))) & 15u;
+            const uint32_t* e = vends + ((((size_t)(m0 + mm) * D + j) * LEN + i) * 16 + d) * NW;
+            uint32_t* o = ends + ((size_t)(m0 + mm) * LEN + i) * NW;
+#pragma unroll
+            for (int w = 0; w < NW; w += 2) *reinterpret_cast<uint2*>(o + w) = *reinterpret_cast<const uint2*>(e + w);
+        }
+        __syncthreads();
+        const uint64_t tree = layer_tree<P>(idx_tree, (int)j);
+        const uint32_t kp = layer_leaf<P>(idx_tree, idx_leaf, (int)j);
+        const uint8_t* auth = sigs + (size_t)(active ? m : 0) * P::SIG_BYTES + P::N + P::FORS_BYTES +
+                              (size_t)j * P::LAYER_BYTES + (size_t)LEN * P::N;
+        tl_group<P, LEN>(msT, make_adrs(j, tree, T_WOTS_PK, kp, 0, 0), ends + (size_t)m * LEN * NW, active, kb.pk_seed,
+                         smem, node);
+        uint32_t au[NW], nx[NW];
+        const bool loads = active && warp == (P::SHAKE ? 0u : 1u);
+#pragma unroll
+        for (int w = 0; w < NW; w++) au[w] = nx[w] = 0;
+        if (loads) load_be<NW>(auth, au);
+#pragma unroll 1
+        for (int z = 0; z < HP; z++) {
+            const uint32_t iz = kp >> z;
+            const Adrs a = make_adrs(j, tree, T_TREE, 0, z + 1, iz >> 1);
+            if (loads && z + 1 < HP) load_be<NW>(auth + (size_t)(z + 1) * P::N, nx);
+            if constexpr (P::SHAKE) {
+                if (loads) {
+                    uint32_t lr[2 * NW];
+#pragma unroll
+                    for (int w = 0; w < NW; w++) {
+                        lr[w] = (iz & 1) ? au[w] : node[w];
+                        lr[NW + w] = (iz & 1) ? node[w] : au[w];
+                    }
+                    hashH_ms<P>(kb.ms256, nullptr, a, lr, node, nullptr);
+                }
+            } else {
+                h_group<P>(kb, a, iz & 1, au, smem, nodes, node);
+            }
+#pragma unroll
+            for (int w = 0; w < NW; w++) au[w] = nx[w];
+        }
+    }
+    if (warp == 0 && m < count) {
+        uint32_t diff = active ? 0u : 1u;
+#pragma unroll
+        for (int w = 0; w < NW; w++) diff |= active ? node[w] ^ kb.pk_root[w] : 0u;
+        ok[m] = diff == 0 ? 1 : 0;
     }
 }
 

@@ -227,6 +227,28 @@ struct SetImpl {
                                                    b.ck, own_layers(b), b.mj_id, b.chk_u, 1u);
         return cudaGetLastError();
     }
+    // Few signatures: the chain ends for every digit, the FORS roots beside
+    // them, then one walk over the layers (scratch: fors_roots, vends, ends).
+    static cudaError_t verify_few(const Batch& b, cudaStream_t s) {
+        const uint32_t T = 128;
+        const uint64_t ct = (uint64_t)b.count * P::D * P::LEN * 16, ft = (uint64_t)b.count * P::K;
+        vspec_kernel<P, kChainPol><<<(uint32_t)((ct + T - 1) / T), T, 0, s>>>(b.keys, b.infos, b.count, b.sigs, b.vends,
+                                                                              1u);
+        cudaError_t e = cudaGetLastError();
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        bool beside = true;
+        if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+            cudaGetLastError();
+            beside = false;
+        }
+        if (e == cudaSuccess)
+            e = launch_beside(beside, vfors_kernel<P>, (uint32_t)((ft + T - 1) / T), T, s, (const KeyBlock*)b.keys,
+                              (const MsgInfo*)b.infos, b.count, (const uint8_t*)b.sigs, b.fors_roots);
+        if (e != cudaSuccess) return e;
+        vwalk_kernel<P><<<(b.count + 31) / 32, kWalkThreads, 0, s>>>(b.keys, b.infos, b.count, b.sigs, b.vends, b.ends,
+                                                                     b.fors_roots, b.ok);
+        return cudaGetLastError();
+    }
     // Verification: FORS roots, PK_FORS, then per layer chains and T_len +
     // climbs (layers are serial), then the comparison with PK.root.  The
     // layer messages live in pk_fors (layer 0) and roots (layers >= 1).
@@ -234,12 +256,13 @@ struct SetImpl {
     // ends (chain ends of one layer), vcnt (16 step buckets per layer),
     // vsitem / vorder (one word per chain of a layer).
     static cudaError_t verify(const Batch& b, cudaStream_t s) {
+        if (b.walk) return verify_few(b, s);
         const uint32_t T = 128;
         cudaError_t e = cudaMemsetAsync(b.vcnt, 0, sizeof(uint32_t) * 16 * P::D, s);
         const uint64_t ft = (uint64_t)b.count * P::K;
         if (e == cudaSuccess) {
             vfors_kernel<P><<<(uint32_t)((ft + T - 1) / T), T, 0, s>>>(b.keys, b.infos, b.count, b.sigs,
-                                                                       b.fors_roots);
+                                                                       b.fors_roots, kNoGuard);
             e = cudaGetLastError();
         }
         if (e == cudaSuccess) e = fors_pk(b, s);
