@@ -138,6 +138,7 @@ struct ServerImpl {
     std::deque<uint64_t> completed;
     uint64_t next_id = 1;
     bool stop = false;
+    bool has_idle = true;            // a slot is free: a submission wakes the scheduler
     std::thread th;
     // stats
     uint64_t n_done = 0, n_batches = 0, n_batched_reqs = 0, max_dev_used = 0, n_failed = 0, n_cancelled = 0;
@@ -164,31 +165,38 @@ Need batch_need(int pset, size_t count, size_t msg_bytes, const hs_keyset* ks) {
     return n;
 }
 
-// Retire finished batches (lock held).
-void retire(ServerImpl& sv) {
+// Retire finished batches (lock held; released while the signatures are
+// copied out, so that submissions do not wait for it).  Only the scheduler
+// thread touches slots and arenas, and a request in a batch stays in the
+// table until it is marked done here.
+void retire(ServerImpl& sv, std::unique_lock<std::mutex>& lk) {
     for (auto& s : sv.slots) {
         if (!s.busy) continue;
         cudaError_t e = cudaSuccess;
         if (!s.failed) {
             e = cudaEventQuery(s.done);            // recorded after the signature copy
             if (e == cudaErrorNotReady) continue;
-        } else {
-            cudaStreamSynchronize(s.stream);       // whatever was queued before the failure
+        }
+        std::vector<Request*> rs;
+        rs.reserve(s.ids.size());
+        for (uint64_t id : s.ids) {
+            auto it = sv.reqs.find(id);
+            rs.push_back(it == sv.reqs.end() ? nullptr : &it->second);
         }
         const int S = sig_bytes_of(s.pset);
+        const bool good = !s.failed && e == cudaSuccess;
+        lk.unlock();
+        if (s.failed) cudaStreamSynchronize(s.stream);       // whatever was queued before the failure
+        if (good)
+            for (size_t i = 0; i < rs.size(); i++)
+                if (rs[i] && rs[i]->out) memcpy(rs[i]->out, sv.host_base + s.host_off + s.sig_host + i * (size_t)S, S);
         const uint64_t t = now_ns();
-        for (size_t i = 0; i < s.ids.size(); i++) {
-            auto it = sv.reqs.find(s.ids[i]);
-            if (it == sv.reqs.end()) continue;
-            Request& r = it->second;
-            if (!s.failed && e == cudaSuccess) {
-                if (r.out) memcpy(r.out, sv.host_base + s.host_off + s.sig_host + (size_t)i * S, S);
-                r.status = HS_OK;
-            } else {
-                r.status = HS_ECUDA;
-                sv.n_failed++;
-            }
-            r.t_done = t;
+        lk.lock();
+        for (size_t i = 0; i < rs.size(); i++) {
+            if (!rs[i]) continue;
+            rs[i]->status = good ? HS_OK : HS_ECUDA;
+            if (!good) sv.n_failed++;
+            rs[i]->t_done = t;
             sv.completed.push_back(s.ids[i]);
             sv.n_done++;
         }
@@ -204,9 +212,11 @@ void retire(ServerImpl& sv) {
 
 constexpr size_t kMinShare = 256;
 
-// Form and launch one batch on a free slot (lock held).  Returns false if
-// nothing could be launched (no pending request, or no memory for even one).
-bool admit(ServerImpl& sv, Slot& slot) {
+// Form and launch one batch on a free slot (lock held; released while the
+// batch is staged and launched: a submission waits for the queue, not for
+// CUDA calls).  Returns false if nothing could be launched (no pending
+// request, or no memory for even one).
+bool admit(ServerImpl& sv, Slot& slot, std::unique_lock<std::mutex>& lk) {
     int best = -1;
     uint64_t oldest = UINT64_MAX;
     for (int p = 0; p < kNumSets; p++)
@@ -268,17 +278,24 @@ bool admit(ServerImpl& sv, Slot& slot) {
     const size_t o_lens = al256(msg_bytes), o_kidx = o_lens + al256(count * 8),
                  o_sigs = o_kidx + al256(count * 4), o_scr = o_sigs + al256(count * (size_t)sig_bytes_of(p));
     slot.ids.clear();
-    size_t mo = 0;
+    std::vector<Request*> rs(count);
     for (size_t i = 0; i < count; i++) {
         const uint64_t id = sv.pending[p].front();
         sv.pending[p].pop_front();
-        Request& r = sv.reqs[id];
+        rs[i] = &sv.reqs[id];                     // stays in the table until the batch is retired
+        slot.ids.push_back(id);
+    }
+    const bool injected = sv.inject_failures > 0;   // a fake failed launch: nothing reaches the GPU
+    if (injected) sv.inject_failures--;
+    lk.unlock();
+    size_t mo = 0;
+    for (size_t i = 0; i < count; i++) {
+        Request& r = *rs[i];
         if (!r.msg.empty()) memcpy(h + mo, r.msg.data(), r.msg.size());
         mo += r.msg.size();
         reinterpret_cast<uint64_t*>(h + o_lens)[i] = r.msg.size();
         reinterpret_cast<uint32_t*>(h + o_kidx)[i] = r.key;
         std::vector<uint8_t>().swap(r.msg);       // staged: the copy is no longer needed
-        slot.ids.push_back(id);
     }
     Batch b{};
     b.pset = p;
@@ -305,11 +322,7 @@ bool admit(ServerImpl& sv, Slot& slot) {
     b.chk_u = ks->chk;
     cudaStream_t s = slot.stream;
     cudaError_t e = cudaSuccess;
-    const bool injected = sv.inject_failures > 0;   // a fake failed launch: nothing reaches the GPU
-    if (injected) {
-        sv.inject_failures--;
-        e = cudaErrorLaunchFailure;
-    }
+    if (injected) e = cudaErrorLaunchFailure;
     if (e == cudaSuccess) e = cudaMemcpyAsync(d, h, o_sigs, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = launch_offsets(b, s);
     if (e == cudaSuccess) e = launch_message(b, false, s);
@@ -326,6 +339,7 @@ bool admit(ServerImpl& sv, Slot& slot) {
     slot.busy = true;
     slot.failed = false;
     if (e == cudaSuccess) e = cudaEventRecord(slot.done, s);
+    lk.lock();
     if (e != cudaSuccess) {
         slot.failed = true;             // retire() marks the requests failed
         if (!injected) {                // a real CUDA error: the server stops taking work
@@ -343,21 +357,24 @@ void scheduler(ServerImpl* sv) {
     cudaSetDevice(sv->device);
     std::unique_lock<std::mutex> lk(sv->mu);
     while (!sv->stop) {
-        retire(*sv);
+        retire(*sv, lk);
         bool launched = true;
         while (launched) {
             launched = false;
             for (auto& s : sv->slots)
-                if (!s.busy && admit(*sv, s)) { launched = true; break; }
+                if (!s.busy && admit(*sv, s, lk)) { launched = true; break; }
         }
         uint32_t busy = 0;
         for (auto& s : sv->slots) busy += s.busy ? 1 : 0;
         sv->max_inflight_seen = std::max(sv->max_inflight_seen, busy);
+        // with every slot taken a submission has nothing to wake it for: it
+        // looks for finished batches by the clock
+        sv->has_idle = busy < sv->slots.size();
         // sleep until a submit or a short timeout (batch completions are polled)
-        if (busy) sv->cv_sched.wait_for(lk, std::chrono::microseconds(100));
+        if (busy) sv->cv_sched.wait_for(lk, std::chrono::microseconds(40));
         else sv->cv_sched.wait_for(lk, std::chrono::milliseconds(50));
     }
-    retire(*sv);
+    retire(*sv, lk);
 }
 
 }  // namespace
@@ -428,13 +445,15 @@ static hs_status submit_at(hs_server* s, hs_params p, uint32_t key, const uint8_
     if (one.dev > sv.dev_arena.cap() || one.host > sv.host_arena.cap())
         return sv_fail(HS_EBUDGET, "hs_server_submit: request larger than the memory budget");
     uint64_t rid;
+    bool wake;
     {
         std::lock_guard<std::mutex> lk(sv.mu);
+        wake = sv.has_idle;
         rid = sv.next_id++;
         sv.reqs.emplace(rid, std::move(r));
         sv.pending[p].push_back(rid);
     }
-    sv.cv_sched.notify_one();
+    if (wake) sv.cv_sched.notify_one();
     if (id) *id = rid;
     return HS_OK;
 }

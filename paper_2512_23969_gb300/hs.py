@@ -467,9 +467,8 @@ class Server:
             if not isinstance(out, np.ndarray) and out.is_cuda:
                 raise ValueError("out: host memory expected (the server writes it on the host)")
             _buf(out, "out", 1, sig_bytes(params))
-        rid = C.c_uint64()
-        buf = C.create_string_buffer(msg, len(msg)) if msg else None
-        _check(load().hs_server_submit(self._h, _pid(params), int(key), buf, len(msg), _ptr(out), C.byref(rid)))
+        rid = C.c_uint64()                # msg's own buffer: the server copies it before it returns
+        _check(load().hs_server_submit(self._h, _pid(params), int(key), msg or None, len(msg), _ptr(out), C.byref(rid)))
         return rid.value, out
 
     def wait(self, rid, timeout_ms=60000):
