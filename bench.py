@@ -70,10 +70,10 @@ STAGE_WORK = {
 
 # The SHAKE instantiation: every hash is Keccak-f[1600] permutations.  ALU
 # work of one permutation on 32-bit lane halves, per round: column parities
-# 20 (2 LOP3 per half), D 20 (rotate-by-1 and XOR), theta's XOR into the
-# 25 lanes 50, rho 48 funnel shifts (lanes rotated by 0 or 32 cost nothing),
-# chi 50 LOP3, iota 2 -> 190 x 24 = 4560.
-ALU_KECCAK = 4560
+# 20 (2 LOP3 per half), their rotations by one 10, theta's three-input XOR
+# into the 25 lanes 50, rho 48 funnel shifts (lanes rotated by 0 or 32 cost
+# nothing), chi 50 LOP3, iota 2 -> 180 x 24 = 4320.
+ALU_KECCAK = 4320
 
 
 def _keccak_work(n, d, hp, a, k, length):
@@ -746,6 +746,10 @@ def run_own(args):
     from paper_2512_23969_gb300 import autotune, hs, inputs
     hs.load()
     tuned = autotune.apply()
+    # the line's definition: every message builds all of its trees; the
+    # library's default, repeated upper-layer trees built once per batch, is
+    # measured beside it (other_configs.128f_tree_sharing)
+    hs.hs_set_tree_sharing(False)
     props = torch.cuda.get_device_properties(local)
     sm_count = props.multi_processor_count
 

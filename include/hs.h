@@ -226,7 +226,7 @@ int hs_probe_int_pipes(float *rates, int max);
  */
 int hs_probe_sha_mix(float *rates, int max);
 
-/* Number of kernels one hs_sign_batch call launches (for launch accounting). */
+/* Kernels a bulk hs_sign_batch call launches at least: one per stage (for launch accounting). */
 int hs_sign_kernel_count(void);
 
 /*

@@ -32,6 +32,7 @@ __global__ void __launch_bounds__(128) utree_kernel(const KeyBlock* __restrict__
                                                     const DedupDesc* __restrict__ desc, uint32_t ndesc,
                                                     uint32_t* __restrict__ nodes, uint32_t* __restrict__ chk_u,
                                                     uint32_t ck, uint32_t one) {
+    allow_next();
     constexpr int NW = P::NW, LV = P::LEAVES;
     const uint64_t gid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t lane = threadIdx.x & 31;

@@ -73,6 +73,11 @@ __device__ __forceinline__ void wots_leaf(const uint32_t* ms256, const uint32_t*
     if constexpr (P::SHAKE) ts.init(msT, make_adrs(layer, tree, T_WOTS_PK, kp, 0, 0));
     const Adrs aprf = make_adrs(layer, tree, T_WOTS_PRF, kp, 0, 0);
     const Adrs ahash = make_adrs(layer, tree, T_WOTS_HASH, kp, 0, 0);
+    LeafCtx lf[P::SHAKE ? 1 : 2];            // PRF, F; read at a run-time index (local memory)
+    if constexpr (!P::SHAKE) {
+        leaf_ctx<POL>(ms256, aprf, lf[0], pp);
+        leaf_ctx<POL>(ms256, ahash, lf[1], pp);
+    }
     // ck is a power of two (1, 2, 4 or 8 when chk is set): test and index
     // positions with a mask and a shift, not a run-time division per step
     const uint32_t per_chain = ck ? 16u >> (__ffs(ck) - 1) : 0u;
@@ -93,11 +98,8 @@ __device__ __forceinline__ void wots_leaf(const uint32_t* ms256, const uint32_t*
 #pragma unroll 1
             for (uint32_t s = 0; s < 16; s++) {
                 if (s <= 1) {
-                    Adrs a = (s == 0) ? aprf : ahash;
-                    a.w4 = i0 << 16;
-                    chain_ctx<POL>(ms256, a, c0, pp);
-                    a.w4 = (i0 + 1) << 16;
-                    chain_ctx<POL>(ms256, a, c1, pp);
+                    chain_ctx<POL>(lf[s], i0 << 16, c0, pp);
+                    chain_ctx<POL>(lf[s], (i0 + 1) << 16, c1, pp);
                 }
                 const uint32_t half = s == 0 ? 0u : s - 1u;
                 chain_step<POL, NW>(c0, ms256, half, x0, x0, pp);
@@ -130,10 +132,12 @@ __device__ __forceinline__ void wots_leaf(const uint32_t* ms256, const uint32_t*
                 hashF_p<P, POL>(ms256, a, x, x, pp);
             } else if constexpr (P::ROBUST) {
                 if (s <= 1) {
-                    Adrs a = (s == 0) ? aprf : ahash;
-                    a.w4 = i << 16;
-                    chain_ctx<POL>(ms256, a, cx, pp);
-                    if (s == 1) mask_ctx<POL, NW>(pks, a, mk, pp);
+                    chain_ctx<POL>(lf[s], i << 16, cx, pp);
+                    if (s == 1) {
+                        Adrs a = ahash;
+                        a.w4 = i << 16;
+                        mask_ctx<POL, NW>(pks, a, mk, pp);
+                    }
                 }
                 // F steps hash x masked with their own address; PRF (s = 0) does not
                 uint32_t xm[NW];
@@ -148,9 +152,7 @@ __device__ __forceinline__ void wots_leaf(const uint32_t* ms256, const uint32_t*
                 chain_step<POL, NW>(cx, ms256, s == 0 ? 0u : s - 1u, xm, x, pp);
             } else {
                 if (s <= 1) {
-                    Adrs a = (s == 0) ? aprf : ahash;
-                    a.w4 = i << 16;              // chain i (< 2^16) | hash >> 16 (= 0)
-                    chain_ctx<POL>(ms256, a, cx, pp);
+                    chain_ctx<POL>(lf[s], i << 16, cx, pp);     // chain i (< 2^16) | hash >> 16 (= 0)
                 }
                 chain_step<POL, NW>(cx, ms256, s == 0 ? 0u : s - 1u, x, x, pp);
             }
@@ -239,8 +241,9 @@ __global__ void __launch_bounds__(128, MINB) tree_kernel(const KeyBlock* __restr
                                                    const MsgInfo* __restrict__ infos, uint32_t count,
                                                    uint8_t* __restrict__ sigs, uint32_t* __restrict__ roots,
                                                    uint32_t* __restrict__ chk, uint32_t ck, uint32_t layers,
-                                                   uint32_t one) {
+                                                   uint32_t one, uint32_t guard) {
     allow_next();
+    if (blockIdx.x == guard) { wait_previous(); return; }
     constexpr int NW = P::NW, LV = P::LEAVES;
     const uint32_t gid = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t lane = threadIdx.x & 31;

@@ -111,9 +111,10 @@ struct SetImpl {
             if (e == cudaSuccess) e = merge(b, s);
             if (e == cudaSuccess && beside) e = beside(b, 1, s);
         } else {
-            tree_kernel<P, POL, MINB, ILP><<<G, T, 0, s>>>(b.keys, b.infos, b.count, b.sigs, b.roots, b.chk, b.ck,
-                                                        L, 1u);
-            e = cudaGetLastError();
+            // beside the shared trees' launch, whose last wave is far from full
+            e = launch_beside(beside != nullptr && b.max_uniq != 0, tree_kernel<P, POL, MINB, ILP>, G, T, s,
+                              (const KeyBlock*)b.keys, (const MsgInfo*)b.infos, b.count, b.sigs, b.roots, b.chk, b.ck,
+                              L, 1u);
             if (e == cudaSuccess && beside) e = beside(b, 0, s);
             if (e == cudaSuccess && beside) {           // T_k reads what the launch before it writes
                 Batch after = b;

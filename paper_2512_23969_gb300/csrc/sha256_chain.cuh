@@ -137,17 +137,36 @@ struct ChainCtx {
     uint32_t k[3];
 };
 
+// What all chains of a leaf share of their contexts: words 0..3 of the
+// address (layer, tree, type, key pair) are the leaf's, only word 4 holds the
+// chain, so rounds 0..3 and the terms of words 0..3 are computed once per leaf
+// and hash type.
+struct LeafCtx {
+    uint32_t s[8];     // after rounds 0..3, in the rotating layout
+    uint32_t c[3];     // the terms of message words 16..18
+    uint32_t w3;
+};
+
 template <int POL>
-__device__ __forceinline__ void chain_ctx(const uint32_t ms[8], const Adrs& a, ChainCtx& x, const Pipes<POL>& p) {
-    uint32_t W[16];
-    W[0] = a.w0; W[1] = a.w1; W[2] = a.w2; W[3] = a.w3; W[4] = a.w4;
+__device__ __forceinline__ void leaf_ctx(const uint32_t ms[8], const Adrs& a, LeafCtx& x, const Pipes<POL>& p) {
 #pragma unroll
     for (int i = 0; i < 8; i++) x.s[i] = ms[i];
-    round256<POL, 0>(x.s, W[0], p);
-    round256<POL, 1>(x.s, W[1], p);
-    round256<POL, 2>(x.s, W[2], p);
-    round256<POL, 3>(x.s, W[3], p);
-    round256<POL, 4>(x.s, W[4], p);
+    round256<POL, 0>(x.s, a.w0, p);
+    round256<POL, 1>(x.s, a.w1, p);
+    round256<POL, 2>(x.s, a.w2, p);
+    round256<POL, 3>(x.s, a.w3, p);
+    x.c[0] = s0_256(a.w1) + a.w0;
+    x.c[1] = s0_256(a.w2) + a.w1;
+    x.c[2] = s0_256(a.w3) + a.w2;
+    x.w3 = a.w3;
+}
+
+// The context of the chain whose address word 4 is w4.
+template <int POL>
+__device__ __forceinline__ void chain_ctx(const LeafCtx& lf, uint32_t w4, ChainCtx& x, const Pipes<POL>& p) {
+#pragma unroll
+    for (int i = 0; i < 8; i++) x.s[i] = lf.s[i];
+    round256<POL, 4>(x.s, w4, p);
     {   // round 5 without W_5 (a = s[3], b = s[4], c = s[5], d = s[6], e = s[7], f = s[0], g = s[1], h = s[2])
         const uint32_t e = x.s[7], f = x.s[0], g = x.s[1], a = x.s[3], b = x.s[4], c = x.s[5];
         const uint32_t t1 = x.s[2] + S1_256(e) + ((e & f) ^ (~e & g)) + detail::kK256[5];
@@ -155,17 +174,24 @@ __device__ __forceinline__ void chain_ctx(const uint32_t ms[8], const Adrs& a, C
         x.s[6] += t1;
         x.s[2] = t1 + t2;
     }
-    x.c[0] = s0_256(W[1]) + W[0];
-    x.c[1] = s0_256(W[2]) + W[1];
-    x.c[2] = s0_256(W[3]) + W[2];
-    x.c[3] = s0_256(W[4]) + W[3];
-    x.c[4] = W[4];
+    x.c[0] = lf.c[0];
+    x.c[1] = lf.c[1];
+    x.c[2] = lf.c[2];
+    x.c[3] = s0_256(w4) + lf.w3;
+    x.c[4] = w4;
     // n = 16: W17 = sigma1(W15) + W10 + c[1], W19 = sigma1(W17) + W12 + c[3]
     // (unused, and removed by the compiler, at the other widths)
     constexpr uint32_t kLen16 = (64 + 22 + 16) * 8;
     x.k[0] = s1_256(kLen16) + x.c[1];
     x.k[1] = s1_256(x.k[0]) + x.c[3];
     x.k[2] = s1_256(x.k[1]);
+}
+
+template <int POL>
+__device__ __forceinline__ void chain_ctx(const uint32_t ms[8], const Adrs& a, ChainCtx& x, const Pipes<POL>& p) {
+    LeafCtx lf;
+    leaf_ctx<POL>(ms, a, lf, p);
+    chain_ctx<POL>(lf, a.w4, x, p);
 }
 
 // ---- robust F masks with a per-chain context --------------------------
