@@ -246,10 +246,24 @@ static cudaError_t tree_beside(const Batch& b, BesideFn beside, cudaStream_t s) 
     return e;
 }
 cudaError_t launch_tree(const Batch& b, cudaStream_t s) { return tree_beside(b, nullptr, s); }
-cudaError_t launch_sign_trees(const Batch& b, cudaStream_t s) {
+bool can_overlap(cudaStream_t s) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-        cudaGetLastError();
+    if (cudaStreamIsCapturing(s, &cap) == cudaSuccess) return cap == cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return false;
+}
+cudaError_t launch_prep(const Batch& b, bool verify, cudaStream_t s) {
+    cudaError_t e = launch_keyprep(b, verify, s);
+    if (needs_offsets(b) || !can_overlap(s)) {
+        if (e == cudaSuccess) e = launch_offsets(b, s);
+        return e == cudaSuccess ? launch_message(b, verify, s) : e;
+    }
+    Batch c = b;                          // the warp form reads the keys themselves
+    c.beside = true;
+    return e == cudaSuccess ? launch_message(c, verify, s) : e;
+}
+cudaError_t launch_sign_trees(const Batch& b, cudaStream_t s) {
+    if (!can_overlap(s)) {
         cudaError_t e = launch_fors(b, s);
         if (e == cudaSuccess) e = launch_fors_pk(b, s);
         return e == cudaSuccess ? launch_tree(b, s) : e;

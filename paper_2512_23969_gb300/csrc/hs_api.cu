@@ -557,12 +557,16 @@ static hs_status run_batch(const hs_keyset* ks, bool verify, hs_params p, const 
 
     const bool prof = g_prof && !verify;
     if (prof) prof_mark(0, s);
-    e = ks ? cudaSuccess : launch_keyprep(b, verify, s);
-    if (prof) prof_mark(1, s);
-    if (e == cudaSuccess) e = launch_offsets(b, s);
-    if (prof) prof_mark(2, s);
-    if (e == cudaSuccess) e = launch_message(b, verify, s);
-    if (prof) prof_mark(3, s);
+    if (prof || ks) {
+        e = ks ? cudaSuccess : launch_keyprep(b, verify, s);
+        if (prof) prof_mark(1, s);
+        if (e == cudaSuccess) e = launch_offsets(b, s);
+        if (prof) prof_mark(2, s);
+        if (e == cudaSuccess) e = launch_message(b, verify, s);
+        if (prof) prof_mark(3, s);
+    } else {
+        e = launch_prep(b, verify, s);
+    }
     if (!verify) {
         if (prof) {                                  // a stage at a time, each between its events
             if (e == cudaSuccess) e = launch_fors(b, s);

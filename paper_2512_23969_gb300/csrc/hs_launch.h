@@ -68,8 +68,8 @@ struct Batch {
     // message stage: a warp per message (SHA-2 sets, small batches; the
     // form is fixed with the batch, like 'split')
     bool msg_warp;
-    // FORS launches: start beside the previous launch of the stream instead
-    // of behind it (sign_trees)
+    // message and FORS launches: start beside the previous launch of the
+    // stream instead of behind it (launch_prep, launch_sign_trees)
     bool beside;
 };
 
@@ -178,6 +178,12 @@ cudaError_t launch_message(const Batch& b, bool verify, cudaStream_t s);
 cudaError_t launch_fors(const Batch& b, cudaStream_t s);
 cudaError_t launch_fors_pk(const Batch& b, cudaStream_t s);
 cudaError_t launch_tree(const Batch& b, cudaStream_t s);
+// Whether launches on s may start beside the one before them: not while the
+// stream is captured.
+bool can_overlap(cudaStream_t s);
+// Key preparation and the message stage, beside each other where the message
+// stage runs in its warp form.
+cudaError_t launch_prep(const Batch& b, bool verify, cudaStream_t s);
 // FORS_Sign, T_k and TREE_Sign of a batch on one stream, the FORS stages
 // beside TREE_Sign (independent given the digest) unless the stream is being
 // captured.

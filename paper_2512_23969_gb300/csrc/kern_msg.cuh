@@ -328,6 +328,7 @@ struct ByteSha {
 template <class P>
 __global__ void keyprep_kernel(const uint8_t* __restrict__ in, uint32_t num_keys, int from_pk,
                                KeyBlock* __restrict__ out) {
+    allow_next();
     constexpr int NW = P::NW, TPK = P::BIG ? 2 : 1;
     const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, k = t / TPK;
     if (k >= num_keys) return;
@@ -550,7 +551,7 @@ struct MsgWarp {
 };
 
 template <class P>
-__device__ __forceinline__ void message_warp(MsgWarp<P>& sm, uint32_t m, const KeyBlock* __restrict__ keys,
+__device__ __forceinline__ void message_warp(MsgWarp<P>& sm, uint32_t m, const uint8_t* __restrict__ raw_keys,
                                              uint32_t num_keys, const uint32_t* __restrict__ key_idx,
                                              const uint8_t* __restrict__ msgs, const uint64_t* __restrict__ lens,
                                              const uint64_t* __restrict__ off, uint8_t* __restrict__ sigs,
@@ -579,7 +580,11 @@ __device__ __forceinline__ void message_warp(MsgWarp<P>& sm, uint32_t m, const K
         }
         return;
     }
-    const KeyBlock& kb = keys[key];
+    // SK.prf, PK.seed and PK.root from the caller's key bytes, so that the
+    // launch need not wait for keyprep
+    const uint8_t* kb = raw_keys + (verify ? (size_t)key * 2 * N : (size_t)key * 4 * N + 2 * N);     // PK.seed
+    auto key_word = [&](int at) { uint32_t w; load_be_unaligned<1>(kb + at, &w); return w; };
+    const uint32_t pk_seed = lane < NW ? key_word(4 * lane) : 0u, pk_root = lane < NW ? key_word(N + 4 * lane) : 0u;
     // the message's offset: up to kSumLens messages, the warp sums the lengths
     // before it and no launch is needed for a prefix sum (off is null)
     uint64_t before = 0;
@@ -609,7 +614,7 @@ __device__ __forceinline__ void message_warp(MsgWarp<P>& sm, uint32_t m, const K
                 outer[i] = __shfl_sync(0xFFFFFFFFu, st[i], 16);
                 st[i] = __shfl_sync(0xFFFFFFFFu, st[i], 0);
             }
-            if (lane < NW) sm.hdr[0][lane] = kb.pk_seed[lane];
+            if (lane < NW) sm.hdr[0][lane] = pk_seed;
             hl = N;
             done = B;
         } else if (ph == 2) {
@@ -624,7 +629,7 @@ __device__ __forceinline__ void message_warp(MsgWarp<P>& sm, uint32_t m, const K
         } else {
             if (ph == 0) {
                 if (lane < BW) {
-                    const uint32_t kw = lane < NW ? kb.sk_prf[lane] : 0u;
+                    const uint32_t kw = lane < NW ? key_word(4 * (int)lane - N) : 0u;
                     sm.hdr[0][lane] = kw ^ 0x36363636u;
                     sm.hdr[1][lane] = kw ^ 0x5c5c5c5cu;
                 }
@@ -643,8 +648,8 @@ __device__ __forceinline__ void message_warp(MsgWarp<P>& sm, uint32_t m, const K
                     for (int i = 0; i < NW; i++) sm.R[i] = sm.hdr[0][i] = R[i];
                 }
                 if (lane < NW) {
-                    sm.hdr[0][NW + lane] = kb.pk_seed[lane];
-                    sm.hdr[0][2 * NW + lane] = kb.pk_root[lane];
+                    sm.hdr[0][NW + lane] = pk_seed;
+                    sm.hdr[0][2 * NW + lane] = pk_root;
                 }
                 hl = 3 * N;
             } else {
@@ -652,7 +657,7 @@ __device__ __forceinline__ void message_warp(MsgWarp<P>& sm, uint32_t m, const K
                 for (int h = 0; h < 2; h++) {
                     if (lane < NW) {
                         sm.hdr[h][lane] = sm.R[lane];
-                        sm.hdr[h][NW + lane] = kb.pk_seed[lane];
+                        sm.hdr[h][NW + lane] = pk_seed;
                     }
                     if (lane == 0) {
 #pragma unroll
@@ -774,16 +779,18 @@ __device__ __forceinline__ void message_warp(MsgWarp<P>& sm, uint32_t m, const K
 constexpr int kMsgWarpsPerBlock = 2;
 template <class P>
 __global__ void __launch_bounds__(32 * kMsgWarpsPerBlock)
-    message_warp_kernel(const KeyBlock* __restrict__ keys, uint32_t num_keys, const uint32_t* __restrict__ key_idx,
-                        const uint8_t* __restrict__ msgs, const uint64_t* __restrict__ lens,
-                        const uint64_t* __restrict__ off, uint32_t count, uint8_t* __restrict__ sigs, MsgInfo* __restrict__ infos, uint32_t* __restrict__ status,
-                        int verify, const uint8_t* __restrict__ prefix, uint32_t plen, int msb_first) {
+    message_warp_kernel(const uint8_t* __restrict__ raw_keys, uint32_t num_keys,
+                        const uint32_t* __restrict__ key_idx, const uint8_t* __restrict__ msgs,
+                        const uint64_t* __restrict__ lens, const uint64_t* __restrict__ off, uint32_t count,
+                        uint8_t* __restrict__ sigs, MsgInfo* __restrict__ infos, uint32_t* __restrict__ status,
+                        int verify, const uint8_t* __restrict__ prefix, uint32_t plen, int msb_first, uint32_t guard) {
+    if (blockIdx.x == guard) { wait_previous(); return; }
     __shared__ __align__(16) MsgWarp<P> sm[kMsgWarpsPerBlock];
     const uint32_t warp = threadIdx.x >> 5;
     const uint32_t m = blockIdx.x * kMsgWarpsPerBlock + warp;
     if (m >= count) return;                        // the whole warp
-    message_warp<P>(sm[warp], m, keys, num_keys, key_idx, msgs, lens, off, sigs, infos, status, verify, prefix, plen,
-                    msb_first);
+    message_warp<P>(sm[warp], m, raw_keys, num_keys, key_idx, msgs, lens, off, sigs, infos, status, verify, prefix,
+                    plen, msb_first);
 }
 
 }  // namespace hs

@@ -27,8 +27,10 @@ template <class P, int POL, int MINB, int ILP = 1>
 __global__ void __launch_bounds__(128, MINB) bleaf_kernel(const KeyBlock* __restrict__ keys,
                                                           const MsgInfo* __restrict__ infos, uint32_t count,
                                                           uint32_t* __restrict__ leafv, uint32_t* __restrict__ chk,
-                                                          uint32_t ck, uint32_t layers, uint32_t one) {
+                                                          uint32_t ck, uint32_t layers, uint32_t one,
+                                                          uint32_t guard) {
     allow_next();
+    if (blockIdx.x == guard) { wait_previous(); return; }
     constexpr int NW = P::NW, LV = P::LEAVES;
     const uint64_t gid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t per_msg = layers * LV;
@@ -190,6 +192,7 @@ __global__ void __launch_bounds__(128) wtree_leaf_kernel(const KeyBlock* __restr
                                                          const DedupDesc* __restrict__ desc, uint32_t ndesc,
                                                          uint32_t* __restrict__ nodes, uint32_t* __restrict__ chk_u,
                                                          uint32_t ck, uint32_t one) {
+    allow_next();
     constexpr int NW = P::NW, LV = P::LEAVES;
     const uint64_t gid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const uint64_t id = gid / LV;

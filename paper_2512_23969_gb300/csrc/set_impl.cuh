@@ -53,11 +53,10 @@ struct SetImpl {
         if constexpr (!P::SHAKE) {
             if (b.msg_warp) {                               // a warp per message
                 const uint32_t T = 32 * kMsgWarpsPerBlock, G = (b.count + kMsgWarpsPerBlock - 1) / kMsgWarpsPerBlock;
-                message_warp_kernel<P><<<G, T, 0, s>>>(b.keys, b.num_keys, b.key_idx, b.msgs, b.lens,
-                                                       needs_offsets(b) ? b.offsets : nullptr, b.count,
-                                                       b.sigs, b.infos, b.status, verify ? 1 : 0, b.prefix,
-                                                       b.prefix_len, b.fips ? 1 : 0);
-                return cudaGetLastError();
+                return launch_beside(b.beside, message_warp_kernel<P>, G, T, s, b.keys_in, b.num_keys, b.key_idx, b.msgs,
+                                     b.lens, (const uint64_t*)(needs_offsets(b) ? b.offsets : nullptr), b.count,
+                                     b.sigs, b.infos, b.status, verify ? 1 : 0, b.prefix, b.prefix_len,
+                                     b.fips ? 1 : 0);
             }
         }
         const uint32_t T = 64, G = (b.count + T - 1) / T;
@@ -101,20 +100,22 @@ struct SetImpl {
         const uint32_t T = 128;
         const uint32_t G = (uint32_t)((threads + T - 1) / T);
         if (threads == 0) return cudaSuccess;
+        // the shared trees first; the messages' own start beside them, as their
+        // last wave is far from full
         cudaError_t e = describe_shared(b, s);
-        if (e == cudaSuccess && b.max_uniq) e = build_trees(b.keys, b.desc, b.max_uniq, b.nodes_u, b.chk_u, b.ck, s);
+        if (e == cudaSuccess && b.max_uniq) e = build_leaves(b.keys, b.desc, b.max_uniq, b.nodes_u, b.chk_u, b.ck, s);
         if (e != cudaSuccess) return e;
+        const bool own_beside = beside != nullptr && b.max_uniq != 0;
         if constexpr (kWide) {
-            bleaf_kernel<P, POL, MINB, ILP><<<G, T, 0, s>>>(b.keys, b.infos, b.count, b.leafv, b.chk, b.ck, L, 1u);
-            e = cudaGetLastError();
+            e = launch_beside(own_beside, bleaf_kernel<P, POL, MINB, ILP>, G, T, s, (const KeyBlock*)b.keys,
+                              (const MsgInfo*)b.infos, b.count, b.leafv, b.chk, b.ck, L, 1u);
             if (e == cudaSuccess && beside) e = beside(b, 0, s);
+            if (e == cudaSuccess) e = build_merge(b.keys, b.desc, b.max_uniq, b.nodes_u, s);
             if (e == cudaSuccess) e = merge(b, s);
             if (e == cudaSuccess && beside) e = beside(b, 1, s);
         } else {
-            // beside the shared trees' launch, whose last wave is far from full
-            e = launch_beside(beside != nullptr && b.max_uniq != 0, tree_kernel<P, POL, MINB, ILP>, G, T, s,
-                              (const KeyBlock*)b.keys, (const MsgInfo*)b.infos, b.count, b.sigs, b.roots, b.chk, b.ck,
-                              L, 1u);
+            e = launch_beside(own_beside, tree_kernel<P, POL, MINB, ILP>, G, T, s, (const KeyBlock*)b.keys,
+                              (const MsgInfo*)b.infos, b.count, b.sigs, b.roots, b.chk, b.ck, L, 1u);
             if (e == cudaSuccess && beside) e = beside(b, 0, s);
             if (e == cudaSuccess && beside) {           // T_k reads what the launch before it writes
                 Batch after = b;
@@ -140,20 +141,23 @@ struct SetImpl {
         return cudaGetLastError();
     }
     // The ndesc trees of desc, all nodes and the checkpoints of every leaf: a
-    // thread per leaf.
-    static cudaError_t build_trees(const KeyBlock* keys, const DedupDesc* desc, uint32_t ndesc, uint32_t* nodes,
-                                   uint32_t* chk, uint32_t ck, cudaStream_t s) {
+    // thread per leaf; wide trees leave the levels above to build_merge.
+    static cudaError_t build_leaves(const KeyBlock* keys, const DedupDesc* desc, uint32_t ndesc, uint32_t* nodes,
+                                    uint32_t* chk, uint32_t ck, cudaStream_t s) {
         const uint32_t T = 128;
         const uint64_t th = (uint64_t)ndesc * P::LEAVES;
         if (th == 0) return cudaSuccess;
         const uint32_t G = (uint32_t)((th + T - 1) / T);
-        if constexpr (kWide) {
+        if constexpr (kWide)
             wtree_leaf_kernel<P, tree_pol<P>()><<<G, T, 0, s>>>(keys, desc, ndesc, nodes, chk, ck, 1u);
-            cudaError_t e = cudaGetLastError();
-            if (e != cudaSuccess) return e;
-            wtree_merge_kernel<P><<<ndesc, kMergeThreads, 0, s>>>(keys, desc, ndesc, nodes);
-        } else {
+        else
             utree_kernel<P, tree_pol<P>()><<<G, T, 0, s>>>(keys, desc, ndesc, nodes, chk, ck, 1u);
+        return cudaGetLastError();
+    }
+    static cudaError_t build_merge(const KeyBlock* keys, const DedupDesc* desc, uint32_t ndesc, uint32_t* nodes,
+                                   cudaStream_t s) {
+        if constexpr (kWide) {
+            if (ndesc) wtree_merge_kernel<P><<<ndesc, kMergeThreads, 0, s>>>(keys, desc, ndesc, nodes);
         }
         return cudaGetLastError();
     }
@@ -175,7 +179,8 @@ struct SetImpl {
         cache_desc_kernel<P><<<(uint32_t)((trees + T - 1) / T), T, 0, s>>>(num_keys, L, tpk, desc);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        return build_trees(keys, desc, (uint32_t)trees, nodes, chk, ck, s);
+        e = build_leaves(keys, desc, (uint32_t)trees, nodes, chk, ck, s);
+        return e == cudaSuccess ? build_merge(keys, desc, (uint32_t)trees, nodes, s) : e;
     }
     // Chain-parallel form: the messages' own trees and the ndesc trees of
     // desc in the same launches (either may be none).  T_len's launch starts
@@ -236,14 +241,8 @@ struct SetImpl {
         vspec_kernel<P, kChainPol><<<(uint32_t)((ct + T - 1) / T), T, 0, s>>>(b.keys, b.infos, b.count, b.sigs, b.vends,
                                                                               1u);
         cudaError_t e = cudaGetLastError();
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        bool beside = true;
-        if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-            cudaGetLastError();
-            beside = false;
-        }
         if (e == cudaSuccess)
-            e = launch_beside(beside, vfors_kernel<P>, (uint32_t)((ft + T - 1) / T), T, s, (const KeyBlock*)b.keys,
+            e = launch_beside(can_overlap(s), vfors_kernel<P>, (uint32_t)((ft + T - 1) / T), T, s, (const KeyBlock*)b.keys,
                               (const MsgInfo*)b.infos, b.count, (const uint8_t*)b.sigs, b.fors_roots);
         if (e != cudaSuccess) return e;
         vwalk_kernel<P><<<(b.count + 31) / 32, kWalkThreads, 0, s>>>(b.keys, b.infos, b.count, b.sigs, b.vends, b.ends,
