@@ -252,13 +252,15 @@ hs_status hs_set_chain_checkpoint(uint32_t stride);
  *                           (each lane builds a subtree of 2^a / lanes
  *                           leaves, the rest merges by shuffles); a batch
  *                           too small to give FORS_Sign about 1024 threads
- *                           per SM takes the next wider compiled value
+ *                           per SM takes the next wider compiled value; at
+ *                           the f sets 32 runs a thread per leaf while few
+ *                           trees are in flight
  *   HS_TUNE_TREE_MIN_BLOCKS minimum resident 128-thread blocks per SM that
  *                           TREE_Sign is compiled for (0 = compiler's choice)
  *   HS_TUNE_TREE_SPLIT_BELOW batches of fewer messages than this run
  *                           TREE_Sign chain-parallel (a thread per WOTS+
- *                           chain, then a thread per leaf for T_len and the
- *                           Merkle levels); 0 = never.  Any value >= 0 is
+ *                           chain, then T_len and the Merkle levels 32 leaves
+ *                           to a block); 0 = never.  Any value >= 0 is
  *                           accepted; hs_tune_options lists suggestions.
  *                           Extra scratch: len * n bytes per hypertree leaf.
  *   HS_TUNE_TREE_POLICY     where TREE_Sign's SHA-256 additions run: 7 =
@@ -271,13 +273,15 @@ hs_status hs_set_chain_checkpoint(uint32_t stride);
  *                           8; see hs_set_chain_checkpoint, which sets every
  *                           set's stride at once)
  *   HS_TUNE_TREE_STEP_US,   measured costs of the two TREE_Sign forms (0 =
- *   HS_TUNE_TREE_SPLIT_NS   not measured): the per-leaf form's time for one
+ *   HS_TUNE_TREE_SPLIT_NS   not used; defaults measured on GB300): the
+ *                           per-leaf form's time for one
  *                           warp per SM sub-partition, in us, and the
  *                           chain-parallel form's time per message, in ns.
  *                           At or above HS_TUNE_TREE_SPLIT_BELOW, a batch
  *                           within four such per-leaf steps takes the form
  *                           they predict faster (the per-leaf time grows in
- *                           whole steps); any value >= 0 is accepted
+ *                           whole steps), and so does key generation; any
+ *                           value >= 0 is accepted
  *   HS_TUNE_MSG_WARP_BELOW  batches of fewer messages than this hash each
  *                           message (PRF_msg, H_msg; Sec. II-A) with a whole
  *                           warp: the message schedules of up to 32 blocks

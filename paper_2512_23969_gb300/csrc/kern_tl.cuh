@@ -33,14 +33,28 @@ struct TlShape {
 };
 
 // Block b of T_l's input after the midstate (as tl_block), its payload words
-// loaded in one batch: the words around the payload are what the 2-byte
+// loaded in one batch (p is 8-byte aligned: whole nodes from an aligned
+// base): the words around the payload are what the 2-byte
 // offset reads there -- the address's last half word before it, the pad byte
 // and zeros behind it.
 template <bool BIG, int PW>
 __device__ __forceinline__ void tl_block_batch(const Adrs& a, const uint32_t* p, int b, uint32_t* W) {
     constexpr int BW = BIG ? 32 : 16;
     constexpr int NB = tl_blocks<BIG, PW>();
-    uint32_t raw[BW + 1];
+    static_assert(PW % 2 == 0, "pairs of payload words");
+    uint32_t raw[BW + 2];
+    if (BIG && b > 0 && b < NB - 1) {          // inside the payload: 8-byte loads (b BW - 6 is even)
+#pragma unroll
+        for (int k = 0; k <= BW; k += 2) {
+            const int q = b * BW + k - 6;
+            const uint2 t = q < PW ? *reinterpret_cast<const uint2*>(p + q) : make_uint2(q == PW ? 0x80000000u : 0u, 0u);
+            raw[k] = t.x;
+            raw[k + 1] = t.y;
+        }
+#pragma unroll
+        for (int k = 0; k < BW; k++) W[k] = mid16(raw[k], raw[k + 1]);
+        return;
+    }
 #pragma unroll
     for (int k = 0; k <= BW; k++) {
         const int q = b * BW + k - 6;
@@ -52,7 +66,9 @@ __device__ __forceinline__ void tl_block_batch(const Adrs& a, const uint32_t* p,
     if (b == NB - 1) W[BW - 1] = ((BIG ? 128u : 64u) + 22u + 4u * PW) * 8u;
 }
 
-// W_t + K_t of one block into rows[t * 32 + lane].
+// One block's schedule into rows[t * 32 + lane]: W_t + K_t (SHA-256), W_t
+// alone (SHA-512, where the producer is the slower side and the rounds add
+// K_t).
 __device__ __forceinline__ void tl_rows256(uint32_t W[16], uint32_t* rows, uint32_t lane) {
 #pragma unroll 1
     for (int t0 = 0; t0 < 64; t0 += 16) {
@@ -72,7 +88,7 @@ __device__ __forceinline__ void tl_rows512(const uint32_t blk[32], uint64_t* row
 #pragma unroll
         for (int i = 0; i < 16; i++) {
             if (t0 > 0) W[i] += s1_512(W[(i + 14) & 15]) + W[(i + 9) & 15] + s0_512(W[(i + 1) & 15]);
-            rows[(t0 + i) * 32 + lane] = W[i] + c_K512[t0 + i];
+            rows[(t0 + i) * 32 + lane] = W[i];
         }
     }
 }
@@ -119,10 +135,10 @@ __device__ __forceinline__ void tl_rounds512(uint64_t st[8], const uint64_t* row
     for (int i = 0; i < 8; i++) v[i] = st[i];
 #pragma unroll
     for (int i = 0; i < 4; i++) xa[i] = rows[i * 32 + lane];
-    auto round = [&](int j, uint64_t x) {
+    auto round = [&](int j, uint64_t x, uint64_t k) {
         uint64_t &a = v[(8 - j) & 7], &b = v[(9 - j) & 7], &c = v[(10 - j) & 7], &d = v[(11 - j) & 7];
         uint64_t &e = v[(12 - j) & 7], &f = v[(13 - j) & 7], &g = v[(14 - j) & 7], &h = v[(15 - j) & 7];
-        const uint64_t t1 = h + S1_512(e) + ((e & f) ^ (~e & g)) + x;
+        const uint64_t t1 = h + S1_512(e) + ((e & f) ^ (~e & g)) + (x + k);
         const uint64_t t2 = S0_512(a) + ((a & b) | (c & (a | b)));
         d += t1;
         h = t1 + t2;
@@ -133,13 +149,13 @@ __device__ __forceinline__ void tl_rounds512(uint64_t st[8], const uint64_t* row
 #pragma unroll
         for (int i = 0; i < 4; i++) xb[i] = r[(4 + i) * 32];
 #pragma unroll
-        for (int i = 0; i < 4; i++) round(i, xa[i]);
+        for (int i = 0; i < 4; i++) round(i, xa[i], c_K512[t + i]);
         if (t < 72) {
 #pragma unroll
             for (int i = 0; i < 4; i++) xa[i] = r[(8 + i) * 32];
         }
 #pragma unroll
-        for (int i = 0; i < 4; i++) round(4 + i, xb[i]);
+        for (int i = 0; i < 4; i++) round(4 + i, xb[i], c_K512[t + 4 + i]);
     }
 #pragma unroll
     for (int i = 0; i < 8; i++) st[i] += v[i];
@@ -262,7 +278,7 @@ __device__ __forceinline__ void h_group(const KeyBlock& kb, const Adrs& a, bool 
                     uint64_t &a_ = v64[(16 - j) & 7], &b_ = v64[(17 - j) & 7], &c_ = v64[(18 - j) & 7],
                              &d_ = v64[(19 - j) & 7], &e_ = v64[(20 - j) & 7], &f_ = v64[(21 - j) & 7],
                              &g_ = v64[(22 - j) & 7], &h_ = v64[(23 - j) & 7];
-                    const uint64_t t1 = h_ + S1_512(e_) + ((e_ & f_) ^ (~e_ & g_)) + r[j * 32];
+                    const uint64_t t1 = h_ + S1_512(e_) + ((e_ & f_) ^ (~e_ & g_)) + (r[j * 32] + c_K512[16 * c + j]);
                     const uint64_t t2 = S0_512(a_) + ((a_ & b_) | (c_ & (a_ | b_)));
                     d_ += t1;
                     h_ = t1 + t2;
@@ -289,7 +305,7 @@ __device__ __forceinline__ void h_group(const KeyBlock& kb, const Adrs& a, bool 
             for (int i = 0; i < 16; i++) {
                 if constexpr (P::BIG) {
                     if (t0 > 0) W64[i] += s1_512(W64[(i + 14) & 15]) + W64[(i + 9) & 15] + s0_512(W64[(i + 1) & 15]);
-                    reinterpret_cast<uint64_t*>(rows)[i * 32 + lane] = W64[i] + c_K512[t0 + i];
+                    reinterpret_cast<uint64_t*>(rows)[i * 32 + lane] = W64[i];
                 } else {
                     if (t0 > 0) W[i] += s1_256(W[(i + 14) & 15]) + W[(i + 9) & 15] + s0_256(W[(i + 1) & 15]);
                     rows[i * 32 + lane] = W[i] + c_K256[t0 + i];
