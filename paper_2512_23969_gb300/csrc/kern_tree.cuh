@@ -289,6 +289,49 @@ __global__ void __launch_bounds__(128, MINB) tree_kernel(const KeyBlock* __restr
 // more parallelism per message.  The trees built for several messages (desc,
 // ndesc of them, checkpoints of every leaf) follow the messages' own in both
 // launches, so they cost no serial step of their own.
+// Chain gid of the messages' own trees, [m][j][l][i], or behind them of the
+// trees of desc, [id][l][i]: false if there is none.  chk: where its
+// checkpoints go (null: nowhere).
+struct ChainAt {
+    uint32_t key, j, l, i;
+    uint64_t tree;
+    uint32_t* chk;
+};
+template <class P>
+__device__ __forceinline__ bool chain_at(uint64_t gid, const MsgInfo* __restrict__ infos, uint32_t count,
+                                         uint32_t layers, const DedupDesc* __restrict__ desc, uint32_t ndesc,
+                                         uint32_t* __restrict__ chk, uint32_t* __restrict__ chk_u,
+                                         uint32_t per_chain, ChainAt& c) {
+    constexpr int NW = P::NW, LV = P::LEAVES, LEN = P::LEN;
+    const uint32_t per_msg = layers * LV * LEN;
+    const uint64_t own = (uint64_t)count * per_msg;
+    c.chk = nullptr;
+    if (gid < own) {
+        const uint64_t m = gid / per_msg;
+        const uint32_t r = (uint32_t)(gid % per_msg);
+        c.j = r / (LV * LEN);
+        c.l = (r / LEN) % LV;
+        c.i = r % LEN;
+        const MsgInfo& info = infos[m];
+        c.key = info.key;
+        if (c.key == KEY_INVALID) return false;
+        c.tree = layer_tree<P>(info.idx_tree, (int)c.j);
+        if (per_chain != 0 && c.l == layer_leaf<P>(info.idx_tree, info.idx_leaf, (int)c.j))
+            c.chk = chk + (((size_t)m * P::D + c.j) * (size_t)LEN + c.i) * per_chain * NW;
+        return true;
+    }
+    const uint64_t sid = gid - own, id = sid / (LV * LEN);
+    if (id >= ndesc) return false;
+    const DedupDesc d = desc[id];
+    c.key = d.key;
+    c.j = d.layer;
+    c.tree = d.tree;
+    c.l = (uint32_t)((sid / LEN) % LV);
+    c.i = (uint32_t)(sid % LEN);
+    if (per_chain != 0) c.chk = chk_u + (((size_t)id * LV + c.l) * (size_t)LEN + c.i) * per_chain * NW;
+    return true;
+}
+
 template <class P, int POL>
 __global__ void __launch_bounds__(128) chains_kernel(const KeyBlock* __restrict__ keys,
                                                      const MsgInfo* __restrict__ infos, uint32_t count,
@@ -297,38 +340,15 @@ __global__ void __launch_bounds__(128) chains_kernel(const KeyBlock* __restrict_
                                                      const DedupDesc* __restrict__ desc, uint32_t ndesc,
                                                      uint32_t* __restrict__ chk_u, uint32_t one) {
     allow_next();
-    constexpr int NW = P::NW, LV = P::LEAVES, LEN = P::LEN;
+    constexpr int NW = P::NW;
     const uint64_t gid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const uint32_t per_msg = layers * LV * LEN;
-    const uint64_t own = (uint64_t)count * per_msg;
     const uint32_t per_chain = ck ? 16u >> (__ffs(ck) - 1) : 0u;      // ck: a power of two
     const uint32_t ck_mask = ck ? ck - 1u : 0u, ck_shift = ck ? (uint32_t)(__ffs(ck) - 1) : 0u;
-    uint32_t key, j, l, i;
-    uint64_t tree;
-    uint32_t* mychk = nullptr;
-    if (gid < own) {
-        const uint64_t m = gid / per_msg;
-        const uint32_t r = (uint32_t)(gid % per_msg);
-        j = r / (LV * LEN);
-        l = (r / LEN) % LV;
-        i = r % LEN;
-        const MsgInfo& info = infos[m];
-        key = info.key;
-        if (key == KEY_INVALID) return;
-        tree = layer_tree<P>(info.idx_tree, (int)j);
-        if (ck != 0 && l == layer_leaf<P>(info.idx_tree, info.idx_leaf, (int)j))
-            mychk = chk + (((size_t)m * P::D + j) * (size_t)LEN + i) * per_chain * NW;
-    } else {
-        const uint64_t sid = gid - own, id = sid / (LV * LEN);
-        if (id >= ndesc) return;
-        const DedupDesc d = desc[id];
-        key = d.key;
-        j = d.layer;
-        tree = d.tree;
-        l = (uint32_t)((sid / LEN) % LV);
-        i = (uint32_t)(sid % LEN);
-        if (ck != 0) mychk = chk_u + (((size_t)id * LV + l) * (size_t)LEN + i) * per_chain * NW;
-    }
+    ChainAt at;
+    if (!chain_at<P>(gid, infos, count, layers, desc, ndesc, chk, chk_u, per_chain, at)) return;
+    const uint32_t key = at.key, j = at.j, l = at.l, i = at.i;
+    const uint64_t tree = at.tree;
+    uint32_t* mychk = at.chk;
     const KeyBlock& kb = keys[key];
     uint32_t ms256[8], x[NW];
 #pragma unroll

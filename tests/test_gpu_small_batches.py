@@ -27,7 +27,7 @@ def _sign(hs, ps, sk, wl):
 
 # a tree group holds 4 trees at 128f / 192f, 2 at 256f; FORS a thread per leaf
 # up to 17 messages at 256f, 27 at 192f (152 SMs)
-@pytest.mark.parametrize("ps,count", [("128f", 1), ("128f", 3), ("128f", 5), ("192f", 27), ("192f", 28), ("256f", 1),
+@pytest.mark.parametrize("ps,count", [("128f", 1), ("128f", 2), ("128f", 3), ("128f", 5), ("192f", 1), ("192f", 27), ("192f", 28), ("256f", 1),
                                       ("256f", 17), ("256f", 18), ("robust-128f", 2), ("shake-192f", 3),
                                       ("192s", 1), ("toy", 9)])
 def test_sign_small(hs, O, ps, count):
@@ -59,7 +59,7 @@ def test_sharing_line(hs, ps, count, keys):
     assert int(on[1].sum()) == 0 and int(on[0].sum()) != 0
 
 
-@pytest.mark.parametrize("ps,count", [("128f", 1), ("128f", 5), ("192f", 4), ("256f", 3), ("128s", 1), ("256s", 2),
+@pytest.mark.parametrize("ps,count", [("128f", 1), ("128f", 34), ("128f", 35), ("192f", 4), ("256f", 3), ("128s", 1), ("256s", 2),
                                       ("shake-128f", 5), ("robust-192f", 3), ("toy", 9)])
 def test_keygen_forms(hs, O, ps, count):
     import torch
