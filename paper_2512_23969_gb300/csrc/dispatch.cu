@@ -40,10 +40,12 @@ struct TuneSlots {
 TuneSlots g_slots;
 auto& g_tune = g_slots.v;
 std::atomic<int> g_ck_default{2};
-// TREE_Sign's form without a tuned cache, per set, as the tuner measured it
-// on GB300: the batch size below which it runs chain-parallel, and above
-// that the cost model's coefficients (split_faster below).
-constexpr int kSplitDefault[kNumSets] = {2048, 1024, 64, 0, 16, 16, 0, 16384, 16384, 16384, 256, 256, 256,
+// TREE_Sign's form without a tuned cache, per set, as measured on GB300: the
+// batch size below which it runs chain-parallel (chain-parallel / per leaf,
+// ms: 128f 1024 messages 5.84 / 5.87, 2048 11.63 / 11.12; 192f 256 2.54 /
+// 2.71, 1024 9.99 / 8.88; 256f 32 0.76 / 1.27, 64 1.46 / 1.26), and above that
+// the cost model's coefficients (split_faster below).
+constexpr int kSplitDefault[kNumSets] = {1024, 256, 64, 0, 16, 16, 0, 16384, 16384, 16384, 256, 256, 256,
                                          16384, 16384, 16384};
 constexpr int kStepUsDefault[kNumSets] = {637, 958, 1262, 0, 655, 1015, 1300, 2379, 3510, 4615, 2414, 3534, 4635,
                                           2379, 3606, 6405};

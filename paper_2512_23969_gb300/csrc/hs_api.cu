@@ -509,10 +509,10 @@ static hs_status run_batch(const hs_keyset* ks, bool verify, hs_params p, const 
                          (h_sig ? align256(sig_total) : 0) + (h_ok ? align256(count) : 0) + align256(plen);
     void* base = nullptr;
     e = cudaMallocFromPoolAsync(&base, scratch + stage, d->pool, s);
-    if (e == cudaErrorMemoryAllocation && (b.max_uniq || b.walk)) {
-        cudaGetLastError();                       // without the shared trees or every digit's ends: less scratch
-        drop_dedup(b);
-        b.walk = false;
+    if (e == cudaErrorMemoryAllocation && (b.max_uniq || b.walk || b.split)) {
+        cudaGetLastError();            // without shared trees, chain ends or every digit's ends: less scratch
+        if (!b.cached) drop_dedup(b);
+        b.walk = b.split = false;
         scratch = need();
         e = cudaMallocFromPoolAsync(&base, scratch + stage, d->pool, s);
     }

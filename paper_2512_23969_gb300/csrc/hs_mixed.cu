@@ -225,12 +225,13 @@ HS_API hs_status hs_sign_mixed(const hs_sign_job* jobs, uint32_t njobs, int use_
         return ea;
     };
     cudaError_t e = reserve();
-    if (e == cudaErrorMemoryAllocation) {     // the shared trees are extra scratch: without them
+    if (e == cudaErrorMemoryAllocation) {     // shared trees and chain ends are extra scratch: without them
         bool any = false;
         total = 0;
         for (size_t j = 0; j < bs.size(); j++) {
-            any = any || bs[j].max_uniq != 0;
+            any = any || bs[j].max_uniq != 0 || bs[j].split;
             drop_dedup(bs[j]);
+            bs[j].split = false;
             off[j] = total;
             total += scratch_bytes(bs[j]);
         }

@@ -166,7 +166,7 @@ __device__ __forceinline__ void tl_rounds512(uint64_t st[8], const uint64_t* row
 // call it.  p: the item's payload, complete before the launch; active: the lane
 // has an item (others read nothing).  The result is in warp 0.  ms: the
 // midstate (SHAKE: PK.seed); pks: PK.seed (robust sets: the payload is
-// masked in place first).
+// masked in place first, the mask's blocks shared by the warps).
 template <class P, int L>
 __device__ __forceinline__ void tl_group(const uint32_t* ms, const Adrs& a, uint32_t* p, bool active,
                                          const uint32_t* pks, uint32_t* smem, uint32_t* out) {
@@ -184,7 +184,7 @@ __device__ __forceinline__ void tl_group(const uint32_t* ms, const Adrs& a, uint
         constexpr int NB = tl_blocks<P::BIG, PW>(), NC = (NB + S::CH - 1) / S::CH;
         const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
         if constexpr (P::ROBUST) {
-            if (warp == 0 && active) mask_mem<P::BIG, NW, PW>(pks, a, p);
+            if (active) mask_mem<P::BIG, NW, PW>(pks, a, p, (int)warp, (int)(blockDim.x >> 5));
             __syncthreads();
         }
         uint32_t st[P::BIG ? 1 : 8];

@@ -73,8 +73,13 @@ __device__ __forceinline__ void wots_leaf(const uint32_t* ms256, const uint32_t*
     if constexpr (P::SHAKE) ts.init(msT, make_adrs(layer, tree, T_WOTS_PK, kp, 0, 0));
     const Adrs aprf = make_adrs(layer, tree, T_WOTS_PRF, kp, 0, 0);
     const Adrs ahash = make_adrs(layer, tree, T_WOTS_HASH, kp, 0, 0);
-    LeafCtx lf[P::SHAKE ? 1 : 2];            // PRF, F; read at a run-time index (local memory)
-    if constexpr (!P::SHAKE) {
+    // Leaf contexts of PRF and F, read at a run-time index (local memory), at n
+    // = 16 and 24 (192f TREE_Sign 66.1 -> 64.9 ms per 8192); at n = 32, with
+    // its longer payload in registers, they cost more than they save (256f
+    // 136.6 -> 138.2).
+    constexpr bool kLeaf = !P::SHAKE && !P::ROBUST && NW < 8;
+    LeafCtx lf[kLeaf ? 2 : 1];
+    if constexpr (kLeaf) {
         leaf_ctx<POL>(ms256, aprf, lf[0], pp);
         leaf_ctx<POL>(ms256, ahash, lf[1], pp);
     }
@@ -98,8 +103,11 @@ __device__ __forceinline__ void wots_leaf(const uint32_t* ms256, const uint32_t*
 #pragma unroll 1
             for (uint32_t s = 0; s < 16; s++) {
                 if (s <= 1) {
-                    chain_ctx<POL>(lf[s], i0 << 16, c0, pp);
-                    chain_ctx<POL>(lf[s], (i0 + 1) << 16, c1, pp);
+                    Adrs a = (s == 0) ? aprf : ahash;
+                    a.w4 = i0 << 16;
+                    chain_ctx<POL>(ms256, a, c0, pp);
+                    a.w4 = (i0 + 1) << 16;
+                    chain_ctx<POL>(ms256, a, c1, pp);
                 }
                 const uint32_t half = s == 0 ? 0u : s - 1u;
                 chain_step<POL, NW>(c0, ms256, half, x0, x0, pp);
@@ -132,12 +140,10 @@ __device__ __forceinline__ void wots_leaf(const uint32_t* ms256, const uint32_t*
                 hashF_p<P, POL>(ms256, a, x, x, pp);
             } else if constexpr (P::ROBUST) {
                 if (s <= 1) {
-                    chain_ctx<POL>(lf[s], i << 16, cx, pp);
-                    if (s == 1) {
-                        Adrs a = ahash;
-                        a.w4 = i << 16;
-                        mask_ctx<POL, NW>(pks, a, mk, pp);
-                    }
+                    Adrs a = (s == 0) ? aprf : ahash;
+                    a.w4 = i << 16;
+                    chain_ctx<POL>(ms256, a, cx, pp);
+                    if (s == 1) mask_ctx<POL, NW>(pks, a, mk, pp);
                 }
                 // F steps hash x masked with their own address; PRF (s = 0) does not
                 uint32_t xm[NW];
@@ -152,7 +158,13 @@ __device__ __forceinline__ void wots_leaf(const uint32_t* ms256, const uint32_t*
                 chain_step<POL, NW>(cx, ms256, s == 0 ? 0u : s - 1u, xm, x, pp);
             } else {
                 if (s <= 1) {
-                    chain_ctx<POL>(lf[s], i << 16, cx, pp);     // chain i (< 2^16) | hash >> 16 (= 0)
+                    if constexpr (kLeaf) {
+                        chain_ctx<POL>(lf[s], i << 16, cx, pp);     // chain i (< 2^16) | hash >> 16 (= 0)
+                    } else {
+                        Adrs a = (s == 0) ? aprf : ahash;
+                        a.w4 = i << 16;
+                        chain_ctx<POL>(ms256, a, cx, pp);
+                    }
                 }
                 chain_step<POL, NW>(cx, ms256, s == 0 ? 0u : s - 1u, x, x, pp);
             }

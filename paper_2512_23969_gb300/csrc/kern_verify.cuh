@@ -11,15 +11,15 @@
 // come from root_{j-1}), but a batch has count x len independent chains in
 // every layer.  So: one thread per (message, FORS tree) for the FORS roots
 // (then the signer's T_k kernel for PK_FORS); then for each layer one
-// thread per (message, chain) advancing its chain to the end, and one
-// thread per message for T_len and the h' climbs, which leaves root_j in
+// thread per (message, chain) advancing its chain to the end, and a block
+// per 32 messages for T_len and the h' climbs, which leaves root_j in
 // scratch for the next layer; finally a comparison with PK.root.
 // A chain needs w - 1 - digit steps (0 .. 15), so a warp of chains in
 // message order waits for its longest.  The chains of a layer are
-// therefore bucketed by their step count (the thread that produced msg_j
-// counts its message's digits), scattered
-// longest first, and the chain kernel runs them in that order: the chains
-// of a warp then have the same length.
+// therefore bucketed by their step count (the block that produced msg_j
+// counts its messages' digits), scattered longest first, and the chain
+// kernel runs them in that order: the chains of a warp then have the same
+// length.  Few signatures take another form (vwalk_kernel).
 #pragma once
 #include <cuda_runtime.h>
 #include "hs_common.cuh"

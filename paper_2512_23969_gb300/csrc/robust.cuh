@@ -80,12 +80,14 @@ __device__ __forceinline__ void mask_regs(const uint32_t* pks, const Adrs& a, ui
 }
 
 // The same over PW words in memory (T_l payloads: chain ends, FORS roots),
-// in place, one MGF1 block at a time.
+// in place, one MGF1 block at a time: blocks first, first + step, ... (the
+// blocks are independent, so warps that share a payload share its mask).
 template <bool BIG, int NW, int PW>
-__device__ __forceinline__ void mask_mem(const uint32_t* pks, const Adrs& a, uint32_t* p) {
+__device__ __forceinline__ void mask_mem(const uint32_t* pks, const Adrs& a, uint32_t* p, int first = 0,
+                                         int step = 1) {
     constexpr int DW = BIG ? 16 : 8;
 #pragma unroll 1
-    for (int c = 0; c * DW < PW; c++) {
+    for (int c = first; c * DW < PW; c += step) {
         uint32_t m[DW];
         if constexpr (BIG) mgf1_512_block<NW>(pks, a, (uint32_t)c, m);
         else mgf1_256_block<NW>(pks, a, (uint32_t)c, m);
