@@ -101,50 +101,52 @@ struct SibStack<R, RI, NW, false> {
 // (local memory): 60 registers instead of 79 for a register select, and as
 // fast or faster (FORS 128f 6.39 -> 6.19 ms, 256f 45.2 -> 43.6 ms per 16384 /
 // 8192 signatures).
+template <class P>
+inline constexpr bool kForsCtx = !P::SHAKE && ((uint64_t)P::K << P::A) <= 65536u;
+
 template <class P, int POL>
-struct ForsLeaf {
-    static constexpr int NW = P::NW;
-    static constexpr bool kCtx = !P::SHAKE && ((uint64_t)P::K << P::A) <= 65536u;
-    ChainCtx cxs[kCtx ? 2 : 1];
-    MaskCtx<NW> mk;                                // robust sets: the leaf F masks
-    __device__ __forceinline__ ForsLeaf(const KeyBlock& kb, const uint32_t* ms256, uint64_t tree, uint32_t kp,
-                                        const Pipes<POL>& pp) {
-        if constexpr (kCtx) {
-            chain_ctx<POL>(ms256, make_adrs(0, tree, T_FORS_PRF, kp, 0, 0), cxs[0], pp);
-            chain_ctx<POL>(ms256, make_adrs(0, tree, T_FORS_TREE, kp, 0, 0), cxs[1], pp);
-            if constexpr (P::ROBUST) mask_ctx<POL, NW>(kb.pk_seed, make_adrs(0, tree, T_FORS_TREE, kp, 0, 0), mk, pp);
-        }
+__device__ __forceinline__ void fors_leaf_ctx(const KeyBlock& kb, const uint32_t* ms256, uint64_t tree, uint32_t kp,
+                                              ChainCtx* cxs, MaskCtx<P::NW>& mk, const Pipes<POL>& pp) {
+    if constexpr (kForsCtx<P>) {
+        chain_ctx<POL>(ms256, make_adrs(0, tree, T_FORS_PRF, kp, 0, 0), cxs[0], pp);
+        chain_ctx<POL>(ms256, make_adrs(0, tree, T_FORS_TREE, kp, 0, 0), cxs[1], pp);
+        if constexpr (P::ROBUST)
+            mask_ctx<POL, P::NW>(kb.pk_seed, make_adrs(0, tree, T_FORS_TREE, kp, 0, 0), mk, pp);
     }
-    // node = leaf g; the secret goes to sk_out if it is not null
-    __device__ __forceinline__ void hash(const KeyBlock& kb, const uint32_t* ms256, const uint32_t* skseed,
-                                         uint64_t tree, uint32_t kp, uint32_t g, uint32_t* node, uint8_t* sk_out,
-                                         const Pipes<POL>& pp) const {
+}
+// node = leaf g; the secret goes to sk_out if it is not null.  mk: the robust
+// sets' leaf F masks.
+template <class P, int POL>
+__device__ __forceinline__ void fors_leaf(const KeyBlock& kb, const uint32_t* ms256, const uint32_t* skseed,
+                                          uint64_t tree, uint32_t kp, uint32_t g, const ChainCtx* cxs,
+                                          const MaskCtx<P::NW>& mk, uint32_t* node, uint8_t* sk_out,
+                                          const Pipes<POL>& pp) {
+    constexpr int NW = P::NW;
 #pragma unroll
-        for (int w = 0; w < NW; w++) node[w] = skseed[w];
+    for (int w = 0; w < NW; w++) node[w] = skseed[w];
 #pragma unroll 1
-        for (int s = 0; s < 2; s++) {
-            if constexpr (kCtx && P::ROBUST) {
-                // the leaf F (s = 1) hashes sk masked with its own address; PRF does not
-                uint32_t xm[NW];
+    for (int s = 0; s < 2; s++) {
+        if constexpr (kForsCtx<P> && P::ROBUST) {
+            // the leaf F (s = 1) hashes sk masked with its own address; PRF does not
+            uint32_t xm[NW];
 #pragma unroll
-                for (int w = 0; w < NW; w++) xm[w] = node[w];
-                if (s == 1) {
-                    uint32_t m[NW];
-                    mask_step<POL, NW>(mk, g, m, pp);
+            for (int w = 0; w < NW; w++) xm[w] = node[w];
+            if (s == 1) {
+                uint32_t m[NW];
+                mask_step<POL, NW>(mk, g, m, pp);
 #pragma unroll
-                    for (int w = 0; w < NW; w++) xm[w] ^= m[w];
-                }
-                chain_step<POL, NW>(cxs[s], ms256, g, xm, node, pp);
-            } else if constexpr (kCtx) {
-                chain_step<POL, NW>(cxs[s], ms256, g, node, node, pp);
-            } else {
-                hashF_p<P, POL>(ms256, make_adrs(0, tree, s == 0 ? T_FORS_PRF : T_FORS_TREE, kp, 0, g), node, node, pp,
-                                s == 0 ? nullptr : kb.pk_seed);
+                for (int w = 0; w < NW; w++) xm[w] ^= m[w];
             }
-            if (s == 0 && sk_out != nullptr) store_be<NW>(sk_out, node);
+            chain_step<POL, NW>(cxs[s], ms256, g, xm, node, pp);
+        } else if constexpr (kForsCtx<P>) {
+            chain_step<POL, NW>(cxs[s], ms256, g, node, node, pp);
+        } else {
+            hashF_p<P, POL>(ms256, make_adrs(0, tree, s == 0 ? T_FORS_PRF : T_FORS_TREE, kp, 0, g), node, node, pp,
+                            s == 0 ? nullptr : kb.pk_seed);
         }
+        if (s == 0 && sk_out != nullptr) store_be<NW>(sk_out, node);
     }
-};
+}
 
 template <class P, int POL, int LPT>
 __global__ void __launch_bounds__(256) fors_kernel(const KeyBlock* __restrict__ keys,
@@ -185,7 +187,9 @@ __global__ void __launch_bounds__(256) fors_kernel(const KeyBlock* __restrict__ 
     uint8_t* sf = sigs + (size_t)m * P::SIG_BYTES + P::N + (size_t)i * (A + 1) * P::N;
 
     const Pipes<POL> pp(one);
-    const ForsLeaf<P, POL> leaf(kb, ms256, tree, kp, pp);
+    ChainCtx cxs[kForsCtx<P> ? 2 : 1];
+    MaskCtx<NW> mk;
+    fors_leaf_ctx<P, POL>(kb, ms256, tree, kp, cxs, mk, pp);
     SibStack<R, RI, NW, (R <= 7)> stk;                 // left siblings, levels 0..R-1
     uint32_t node[NW];
     const uint32_t base = L << R;                  // first leaf of this lane (within tree)
@@ -195,7 +199,7 @@ __global__ void __launch_bounds__(256) fors_kernel(const KeyBlock* __restrict__ 
         for (uint32_t p = 0; p < (1u << RI); p++) {
             const uint32_t t = base + (ob << RI) + p;  // leaf index within tree
             const uint32_t g = (i << A) + t;           // global leaf index
-            leaf.hash(kb, ms256, skseed, tree, kp, g, node, t == gs ? sf : nullptr, pp);
+            fors_leaf<P, POL>(kb, ms256, skseed, tree, kp, g, cxs, mk, node, t == gs ? sf : nullptr, pp);
             if (t == (gs ^ 1u)) store_be<NW>(sf + P::N, node);
             // merge with stacked left siblings while this node is a right child
             uint32_t z = 0, idx = t;
@@ -286,8 +290,10 @@ __global__ void __launch_bounds__(T << P::A) fors_wide_kernel(const KeyBlock* __
 #pragma unroll
             for (int w = 0; w < NW; w++) skseed[w] = kb.sk_seed[w];
             const Pipes<POL> pp(one);
-            const ForsLeaf<P, POL> leaf(kb, ms256, tree, kp, pp);
-            leaf.hash(kb, ms256, skseed, tree, kp, (i << A) + l, node, l == gs ? sf : nullptr, pp);
+            ChainCtx cxs[kForsCtx<P> ? 2 : 1];
+            MaskCtx<NW> mk;
+            fors_leaf_ctx<P, POL>(kb, ms256, tree, kp, cxs, mk, pp);
+            fors_leaf<P, POL>(kb, ms256, skseed, tree, kp, (i << A) + l, cxs, mk, node, l == gs ? sf : nullptr, pp);
             if (l == (gs ^ 1u)) store_be<NW>(sf + P::N, node);
 #pragma unroll
             for (int w = 0; w < NW; w++) sh[t * NW + w] = node[w];

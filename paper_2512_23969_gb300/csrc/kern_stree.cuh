@@ -64,9 +64,9 @@ __global__ void __launch_bounds__(128, MINB) bleaf_kernel(const KeyBlock* __rest
 // Chain-parallel form, second half: T_len over the len chain ends that
 // chains_kernel wrote for each leaf, 32 leaves per block (kern_tl.cuh); the
 // blocks behind the messages' own leaves take the trees of desc, whose
-// leaves go to nodes_u.
-template <class P>
-__global__ void __launch_bounds__(TlShape<P>::THREADS) bleaf_from_ends_kernel(const KeyBlock* __restrict__ keys,
+// leaves go to nodes_u.  GROUP = false: a thread per leaf alone, 128 per block.
+template <class P, bool GROUP>
+__global__ void __launch_bounds__(GROUP ? TlShape<P>::THREADS : 128) bleaf_from_ends_kernel(const KeyBlock* __restrict__ keys,
                                                                               const MsgInfo* __restrict__ infos,
                                                                               uint32_t count,
                                                                               uint32_t* __restrict__ ends,
@@ -77,9 +77,10 @@ __global__ void __launch_bounds__(TlShape<P>::THREADS) bleaf_from_ends_kernel(co
                                                                               uint32_t* __restrict__ nodes_u) {
     allow_next();
     constexpr int NW = P::NW, LV = P::LEAVES, LEN = P::LEN;
-    static_assert(LV % 32 == 0, "a block is 32 leaves of one tree");
-    __shared__ __align__(16) uint32_t smem[TlShape<P>::SMEM_WORDS];
-    const uint64_t gid = (uint64_t)blockIdx.x * 32 + (threadIdx.x & 31);
+    static_assert(LV % 128 == 0, "a block's leaves are of one tree");
+    __shared__ __align__(16) uint32_t smem[GROUP ? TlShape<P>::SMEM_WORDS : 1];
+    const uint64_t gid = GROUP ? (uint64_t)blockIdx.x * 32 + (threadIdx.x & 31)
+                               : (uint64_t)blockIdx.x * 128 + threadIdx.x;
     const uint32_t per_msg = layers * LV;
     const uint64_t own = (uint64_t)count * per_msg;
     const uint32_t l = (uint32_t)(gid % LV);
@@ -103,9 +104,9 @@ __global__ void __launch_bounds__(TlShape<P>::THREADS) bleaf_from_ends_kernel(co
     }
     const KeyBlock& kb = keys[key];
     uint32_t node[NW];
-    tl_group<P, LEN>(P::BIG ? kb.ms512 : kb.ms256, make_adrs(j, tree, T_WOTS_PK, l, 0, 0),
+    tl_group<P, LEN, GROUP>(P::BIG ? kb.ms512 : kb.ms256, make_adrs(j, tree, T_WOTS_PK, l, 0, 0),
                      ends + (size_t)gid * LEN * NW, true, kb.pk_seed, smem, node);
-    if (threadIdx.x >= 32) return;
+    if (GROUP && threadIdx.x >= 32) return;
 #pragma unroll
     for (int w = 0; w < NW; w++) out[w] = node[w];
 }

@@ -23,6 +23,9 @@
 
 namespace hs {
 
+// Groups of 32 items an SM holds (40 KB of shared memory each at SHA-512).
+constexpr uint32_t kTlGroupsPerSm = 5;
+
 template <class P>
 struct TlShape {
     static constexpr int CH = P::SHAKE ? 0 : (P::BIG ? 1 : 2);       // producer warps = blocks per buffer
@@ -167,12 +170,18 @@ __device__ __forceinline__ void tl_rounds512(uint64_t st[8], const uint64_t* row
 // has an item (others read nothing).  The result is in warp 0.  ms: the
 // midstate (SHAKE: PK.seed); pks: PK.seed (robust sets: the payload is
 // masked in place first, the mask's blocks shared by the warps).
-template <class P, int L>
+// GROUP = false: every thread hashes its own item alone (tl_groups_pay).
+template <class P, int L, bool GROUP = true>
 __device__ __forceinline__ void tl_group(const uint32_t* ms, const Adrs& a, uint32_t* p, bool active,
                                          const uint32_t* pks, uint32_t* smem, uint32_t* out) {
     constexpr int NW = P::NW, PW = L * NW;
-    if constexpr (P::SHAKE) {
-        if (active && threadIdx.x < 32) {
+    if constexpr (!P::SHAKE && !GROUP) {
+        if (active) {
+            if constexpr (P::ROBUST) mask_mem<P::BIG, NW, PW>(pks, a, p);
+            tl_from_mem<P::BIG, PW, NW>(ms, a, p, out);
+        }
+    } else if constexpr (P::SHAKE) {
+        if (active && (!GROUP || threadIdx.x < 32)) {
             TStreamP<P> ts;
             ts.init(ms, a);
 #pragma unroll 1

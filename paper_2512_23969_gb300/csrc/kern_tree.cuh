@@ -408,9 +408,9 @@ __global__ void __launch_bounds__(128) chains_kernel(const KeyBlock* __restrict_
 // T_len and the Merkle levels over the chain ends, 32 leaves per block (whole
 // trees), T_len's schedules by the block's other warps (kern_tl.cuh); the
 // blocks behind the messages' own leaves take the trees of desc, whose nodes
-// go to nodes_u.
-template <class P>
-__global__ void __launch_bounds__(TlShape<P>::THREADS) leaves_kernel(const KeyBlock* __restrict__ keys,
+// go to nodes_u.  GROUP = false: a thread per leaf alone, 128 per block.
+template <class P, bool GROUP>
+__global__ void __launch_bounds__(GROUP ? TlShape<P>::THREADS : 128) leaves_kernel(const KeyBlock* __restrict__ keys,
                                                                      const MsgInfo* __restrict__ infos,
                                                                      uint32_t count, uint32_t* __restrict__ ends,
                                                                      uint8_t* __restrict__ sigs,
@@ -419,22 +419,23 @@ __global__ void __launch_bounds__(TlShape<P>::THREADS) leaves_kernel(const KeyBl
                                                                      uint32_t ndesc, uint32_t* __restrict__ nodes_u) {
     allow_next();
     constexpr int NW = P::NW, LV = P::LEAVES, LEN = P::LEN;
-    __shared__ __align__(16) uint32_t smem[TlShape<P>::SMEM_WORDS];
-    const uint32_t lane = threadIdx.x & 31;
+    constexpr uint32_t ITEMS = GROUP ? 32 : 128;     // leaves per block
+    __shared__ __align__(16) uint32_t smem[GROUP ? TlShape<P>::SMEM_WORDS : 1];
+    const uint32_t lane = threadIdx.x & 31, item = GROUP ? lane : threadIdx.x;
     const uint32_t per_msg = layers * LV;
     const uint64_t own = (uint64_t)count * per_msg;
-    const uint32_t own_blocks = (uint32_t)((own + 31) / 32);
+    const uint32_t own_blocks = (uint32_t)((own + ITEMS - 1) / ITEMS);
     const bool shared = blockIdx.x >= own_blocks;    // block-uniform
     uint32_t m = 0, id = 0, j = 0, key = KEY_INVALID;
     uint64_t tree = 0, leaf;                         // leaf: its place in ends
     if (!shared) {
-        leaf = (uint64_t)blockIdx.x * 32 + lane;
+        leaf = (uint64_t)blockIdx.x * ITEMS + item;
         m = (uint32_t)(leaf / per_msg);
         j = (uint32_t)(leaf % per_msg) / LV;
         if (m < count) key = infos[m].key;
         if (key != KEY_INVALID) tree = layer_tree<P>(infos[m].idx_tree, (int)j);
     } else {
-        const uint64_t sid = (uint64_t)(blockIdx.x - own_blocks) * 32 + lane;
+        const uint64_t sid = (uint64_t)(blockIdx.x - own_blocks) * ITEMS + item;
         leaf = own + sid;
         id = (uint32_t)(sid / LV);
         if (id < ndesc) {
@@ -447,9 +448,9 @@ __global__ void __launch_bounds__(TlShape<P>::THREADS) leaves_kernel(const KeyBl
     const bool active = key != KEY_INVALID;          // the same for a whole tree
     const KeyBlock& kb = keys[active ? key : 0];
     uint32_t node[NW];
-    tl_group<P, LEN>(P::BIG ? kb.ms512 : kb.ms256, make_adrs(j, tree, T_WOTS_PK, l, 0, 0), ends + leaf * LEN * NW,
+    tl_group<P, LEN, GROUP>(P::BIG ? kb.ms512 : kb.ms256, make_adrs(j, tree, T_WOTS_PK, l, 0, 0), ends + leaf * LEN * NW,
                      active, kb.pk_seed, smem, node);
-    if (threadIdx.x >= 32 || !active) return;
+    if ((GROUP && threadIdx.x >= 32) || !active) return;
     const unsigned gmask = ((LV == 32) ? 0xFFFFFFFFu : ((1u << LV) - 1u)) << (lane & ~(uint32_t)(LV - 1));
     uint32_t ms256[8], msT[P::BIG ? 16 : 8];
 #pragma unroll

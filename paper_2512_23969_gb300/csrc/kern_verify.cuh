@@ -213,8 +213,9 @@ __global__ void __launch_bounds__(128) vchain_kernel(const KeyBlock* __restrict_
 // Layer j of 32 messages per block: T_len over the chain ends (kern_tl.cuh),
 // then h' climbs with the auth path; root_j replaces msg_j in vroot and its
 // digits are counted for the next layer.
-template <class P>
-__global__ void __launch_bounds__(TlShape<P>::THREADS) vleaf_kernel(const KeyBlock* __restrict__ keys,
+// GROUP = false: one warp per block, a thread per message alone.
+template <class P, bool GROUP>
+__global__ void __launch_bounds__(GROUP ? TlShape<P>::THREADS : 32) vleaf_kernel(const KeyBlock* __restrict__ keys,
                                                                     const MsgInfo* __restrict__ infos, uint32_t count,
                                                                     const uint8_t* __restrict__ sigs,
                                                                     uint32_t* __restrict__ ends,
@@ -222,7 +223,7 @@ __global__ void __launch_bounds__(TlShape<P>::THREADS) vleaf_kernel(const KeyBlo
                                                                     uint32_t* __restrict__ cnt_next,
                                                                     uint32_t* __restrict__ sitem) {
     constexpr int NW = P::NW, LEN = P::LEN, HP = P::HP;
-    constexpr int BUF = TlShape<P>::SMEM_WORDS > 32 * LEN ? TlShape<P>::SMEM_WORDS : 32 * LEN;
+    constexpr int TLW = GROUP ? TlShape<P>::SMEM_WORDS : 1, BUF = TLW > 32 * LEN ? TLW : 32 * LEN;
     __shared__ __align__(16) uint32_t smem[BUF];
     __shared__ CountSmem<P> c;
     const uint32_t lane = threadIdx.x & 31;
@@ -234,7 +235,7 @@ __global__ void __launch_bounds__(TlShape<P>::THREADS) vleaf_kernel(const KeyBlo
     const uint64_t tree = layer_tree<P>(info.idx_tree, (int)j);
     const uint32_t kp = layer_leaf<P>(info.idx_tree, info.idx_leaf, (int)j);
     uint32_t node[NW];
-    tl_group<P, LEN>(P::BIG ? kb.ms512 : kb.ms256, make_adrs(j, tree, T_WOTS_PK, kp, 0, 0),
+    tl_group<P, LEN, GROUP>(P::BIG ? kb.ms512 : kb.ms256, make_adrs(j, tree, T_WOTS_PK, kp, 0, 0),
                      ends + (size_t)m * LEN * NW, active, kb.pk_seed, smem, node);
     if (threadIdx.x < 32) {
         if (active) {

@@ -39,6 +39,10 @@ struct SetImpl {
     // kern_stree.cuh, also for the shared and cached trees.
     static constexpr bool kWide = P::LEAVES > 32;
 
+    // Whether a T_l launch over this many groups of 32 items runs by groups:
+    // while the SMs hold them all at once.
+    static bool tl_groups_pay(uint64_t groups) { return groups <= (uint64_t)kTlGroupsPerSm * sm_count(); }
+
     // layers each message builds itself: all of them unless the upper
     // layers are shared within the batch (dedup_layer = first shared layer)
     static uint32_t own_layers(const Batch& b) { return b.dedup_layer ? b.dedup_layer : (uint32_t)P::D; }
@@ -199,18 +203,24 @@ struct SetImpl {
         cudaError_t e = cudaGetLastError();
         if (e == cudaSuccess && beside) e = beside(*b, 0, s);
         if (e != cudaSuccess) return e;
-        const uint32_t G = (uint32_t)((own + 31) / 32 + (shared + 31) / 32);
+        const bool group = tl_groups_pay((own + 31) / 32 + (shared + 31) / 32);
+        const uint32_t per = group ? 32 : 128, TL = group ? TlShape<P>::THREADS : 128;
+        const uint32_t G = (uint32_t)((own + per - 1) / per + (shared + per - 1) / per);
         if constexpr (kWide) {
-            bleaf_from_ends_kernel<P><<<G, TlShape<P>::THREADS, 0, s>>>(keys, infos, count, ends, leafv, L, desc,
-                                                                        ndesc, nodes_u);
+            if (group)
+                bleaf_from_ends_kernel<P, true><<<G, TL, 0, s>>>(keys, infos, count, ends, leafv, L, desc, ndesc, nodes_u);
+            else
+                bleaf_from_ends_kernel<P, false><<<G, TL, 0, s>>>(keys, infos, count, ends, leafv, L, desc, ndesc, nodes_u);
             e = cudaGetLastError();
             if (e == cudaSuccess && beside) e = beside(*b, 1, s);
             if (e != cudaSuccess || ndesc == 0) return e;
             wtree_merge_kernel<P><<<ndesc, kMergeThreads, 0, s>>>(keys, desc, ndesc, nodes_u);
             return cudaGetLastError();
         } else {
-            leaves_kernel<P><<<G, TlShape<P>::THREADS, 0, s>>>(keys, infos, count, ends, sigs, roots, L, desc, ndesc,
-                                                               nodes_u);
+            if (group)
+                leaves_kernel<P, true><<<G, TL, 0, s>>>(keys, infos, count, ends, sigs, roots, L, desc, ndesc, nodes_u);
+            else
+                leaves_kernel<P, false><<<G, TL, 0, s>>>(keys, infos, count, ends, sigs, roots, L, desc, ndesc, nodes_u);
             e = cudaGetLastError();
             return e == cudaSuccess && beside ? beside(*b, 1, s) : e;
         }
@@ -279,8 +289,13 @@ struct SetImpl {
             vchain_kernel<P, kChainPol><<<(uint32_t)((ct + T - 1) / T), T, 0, s>>>(
                 b.keys, b.infos, b.count, b.sigs, b.vorder, b.vsitem, b.ends, j, 1u);
             if ((e = cudaGetLastError()) != cudaSuccess) break;
-            vleaf_kernel<P><<<G32, TlShape<P>::THREADS, 0, s>>>(b.keys, b.infos, b.count, b.sigs, b.ends, b.roots, j,
-                                             j + 1 < (uint32_t)P::D ? b.vcnt + 16 * (j + 1) : nullptr, b.vsitem);
+            uint32_t* next = j + 1 < (uint32_t)P::D ? b.vcnt + 16 * (j + 1) : nullptr;
+            if (tl_groups_pay(G32))
+                vleaf_kernel<P, true><<<G32, TlShape<P>::THREADS, 0, s>>>(b.keys, b.infos, b.count, b.sigs, b.ends,
+                                                                          b.roots, j, next, b.vsitem);
+            else
+                vleaf_kernel<P, false><<<G32, 32, 0, s>>>(b.keys, b.infos, b.count, b.sigs, b.ends, b.roots, j, next,
+                                                          b.vsitem);
             e = cudaGetLastError();
         }
         if (e != cudaSuccess) return e;

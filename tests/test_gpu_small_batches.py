@@ -84,10 +84,12 @@ def test_keygen_forms(hs, O, ps, count):
 
 
 # the walk takes 3500 (SHAKE: 3000) chains a layer: 100 signatures at n = 16
-# (SHAKE 85), 68 at n = 24, 52 at n = 32; 32 signatures to a block
+# (SHAKE 85), 68 at n = 24, 52 at n = 32; 32 signatures to a block; above 5
+# groups of 32 signatures per SM (24320 on 152) T_len runs a thread per item
 @pytest.mark.parametrize("ps,count", [("128f", 1), ("128f", 33), ("128f", 100), ("128f", 101), ("192f", 68),
                                       ("256f", 52), ("256f", 53), ("shake-128f", 85), ("shake-256f", 2),
-                                      ("robust-128f", 34), ("128s", 3), ("256s", 2), ("toy", 40)])
+                                      ("robust-128f", 34), ("128s", 3), ("256s", 2), ("toy", 40),
+                                      ("toy", 24400)])
 def test_verify_forms(hs, O, ps, count):
     import torch
     wl = inputs.make(ps, count, num_keys=2, lengths=("uniform", 0, 100), seed=60 + count, key_mode="random")
