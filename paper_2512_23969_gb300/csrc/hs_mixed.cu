@@ -198,7 +198,9 @@ HS_API hs_status hs_sign_mixed(const hs_sign_job* jobs, uint32_t njobs, int use_
         b.sigs = jb.sigs;
         b.ck = chain_checkpoint_stride(b.pset);
         b.split = tree_split(b.pset, b.count);
-        b.msg_warp = msg_warp(b.pset, b.count);
+        // beside other jobs the warp form's redundant rounds take their ALU
+        // time, so only the small jobs, whose latency it shortens, use it
+        b.msg_warp = msg_warp(b.pset, b.count) && (njobs == 1 || b.count < 512);
         plan_dedup(b);
         bs.push_back(b);
         off.push_back(total);
