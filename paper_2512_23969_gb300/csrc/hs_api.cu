@@ -118,7 +118,7 @@ static void scratch_layout(const Batch& b, const SetInfo& s, size_t sz[kRegions]
     const size_t nw = (size_t)s.n / 4, cnt = b.count;
     int i = 0;
     sz[i++] = sizeof(uint32_t);                                      // reserved
-    sz[i++] = (size_t)b.num_keys * sizeof(KeyBlock);                 // keys
+    sz[i++] = b.resident ? 0 : (size_t)b.num_keys * sizeof(KeyBlock);   // keys
     sz[i++] = (cnt + 1) * sizeof(uint64_t);                          // offsets
     sz[i++] = cnt * sizeof(MsgInfo);                                 // infos
     sz[i++] = cnt * s.k * nw * 4;                                    // fors_roots
@@ -153,7 +153,7 @@ size_t scratch_bytes(const Batch& b) {
 size_t scratch_bytes(int pset, uint32_t num_keys, uint32_t count, uint32_t ck, bool split, uint32_t cached_from) {
     Batch b{};
     b.pset = pset;
-    b.num_keys = num_keys;
+    b.num_keys = num_keys;            // 0: the keys are resident
     b.count = count;
     b.ck = ck;
     b.split = split;
@@ -162,7 +162,7 @@ size_t scratch_bytes(int pset, uint32_t num_keys, uint32_t count, uint32_t ck, b
     return scratch_bytes(b);
 }
 
-void carve_scratch(Batch& b, void* base) {
+size_t carve_scratch(Batch& b, void* base) {
     SetInfo s{};
     set_info(b.pset, &s);
     size_t sz[kRegions];
@@ -171,7 +171,7 @@ void carve_scratch(Batch& b, void* base) {
     char* p = static_cast<char*>(base);
     char* r[kRegions];
     for (int i = 0; i < n; i++) { r[i] = p; p += align256(sz[i]); }
-    b.keys = reinterpret_cast<KeyBlock*>(r[1]);
+    if (!b.resident) b.keys = reinterpret_cast<KeyBlock*>(r[1]);
     b.offsets = reinterpret_cast<uint64_t*>(r[2]);
     b.infos = reinterpret_cast<MsgInfo*>(r[3]);
     b.fors_roots = reinterpret_cast<uint32_t*>(r[4]);
@@ -185,10 +185,12 @@ void carve_scratch(Batch& b, void* base) {
     b.vsitem = b.vcnt ? b.vcnt + 16 * s.d : nullptr;
     b.vorder = b.vcnt ? b.vsitem + (size_t)b.count * s.len : nullptr;
     b.mj_id = b.dedup_layer ? reinterpret_cast<uint32_t*>(r[9]) : nullptr;
-    if (b.cached) return;             // nodes_u / chk_u belong to the keyset
+    const size_t total = (size_t)(p - static_cast<char*>(base));
+    if (b.cached) return total;       // nodes_u / chk_u belong to the keyset
     b.desc = b.max_uniq ? reinterpret_cast<DedupDesc*>(r[10]) : nullptr;
     b.nodes_u = b.max_uniq ? reinterpret_cast<uint32_t*>(r[11]) : nullptr;
     b.chk_u = (b.max_uniq && b.ck) ? b.nodes_u + (size_t)b.max_uniq * 2 * s.leaves * (s.n / 4) : nullptr;
+    return total;
 }
 
 // ----------------------------------------------------------- device state
@@ -496,14 +498,8 @@ static hs_status run_batch(const hs_keyset* ks, bool verify, hs_params p, const 
     } else if (!verify) {
         plan_dedup(b);
     }
-    // scratch: no key blocks with a keyset, they are resident
-    auto need = [&] {
-        b.num_keys = ks ? 0 : num_keys;
-        const size_t n = scratch_bytes(b);
-        b.num_keys = num_keys;
-        return n;
-    };
-    size_t scratch = need();
+    b.resident = ks != nullptr;
+    size_t scratch = scratch_bytes(b);
     const size_t stage = (h_keys ? align256(key_bytes) : 0) + (h_idx ? align256((size_t)count * 4) : 0) +
                          (h_lens ? align256((size_t)count * 8) : 0) + (h_msgs ? align256(msg_total) : 0) +
                          (h_sig ? align256(sig_total) : 0) + (h_ok ? align256(count) : 0) + align256(plen);
@@ -513,7 +509,7 @@ static hs_status run_batch(const hs_keyset* ks, bool verify, hs_params p, const 
         cudaGetLastError();            // without shared trees, chain ends or every digit's ends: less scratch
         if (!b.cached) drop_dedup(b);
         b.walk = b.split = false;
-        scratch = need();
+        scratch = scratch_bytes(b);
         e = cudaMallocFromPoolAsync(&base, scratch + stage, d->pool, s);
     }
     if (e != cudaSuccess) return cuda_fail(e, "cudaMallocFromPoolAsync(scratch)");

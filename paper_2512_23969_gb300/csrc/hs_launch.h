@@ -37,6 +37,7 @@ struct Batch {
     uint32_t* vends;          // walk: chain ends for every digit, count * D * LEN * 16 * NW words
     // scratch
     KeyBlock* keys;           // num_keys
+    bool resident;            // keys belong to a keyset: the scratch holds no key blocks
     uint64_t* offsets;        // count + 1
     MsgInfo* infos;           // count
     uint32_t* fors_roots;     // count * K * NW words
@@ -100,7 +101,8 @@ size_t scratch_bytes(const Batch& b);
 // cached_from: first layer taken from a keyset's cache (0 = none).
 size_t scratch_bytes(int pset, uint32_t num_keys, uint32_t count, uint32_t ck, bool split = false,
                      uint32_t cached_from = 0);
-void carve_scratch(Batch& b, void* base);
+// Lays the regions out from base on and returns their total, scratch_bytes(b).
+size_t carve_scratch(Batch& b, void* base);
 
 // Per-parameter-set kernel launchers (one table per set_<name>.cu).  The
 // FORS and TREE launchers take the tuned launch shape: lanes per FORS tree

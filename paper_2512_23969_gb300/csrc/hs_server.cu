@@ -300,7 +300,9 @@ bool admit(ServerImpl& sv, Slot& slot, std::unique_lock<std::mutex>& lk) {
     Batch b{};
     b.pset = p;
     b.keys_in = ks->sk;
-    b.num_keys = 0;                               // scratch holds no key blocks (see below)
+    b.num_keys = ks->num_keys;
+    b.resident = true;                            // scratch holds no key blocks
+    b.keys = ks->kb;
     b.key_idx = reinterpret_cast<const uint32_t*>(d + o_kidx);
     b.msgs = msg_bytes ? d : d + o_lens;          // never read when all lengths are 0
     b.lens = reinterpret_cast<const uint64_t*>(d + o_lens);
@@ -316,8 +318,6 @@ bool admit(ServerImpl& sv, Slot& slot, std::unique_lock<std::mutex>& lk) {
     b.msg_warp = alone && msg_warp(p, (uint32_t)count);
     b.status = device_status_word();
     carve_scratch(b, d + o_scr);
-    b.keys = ks->kb;                              // resident midstates, not scratch
-    b.num_keys = ks->num_keys;
     b.nodes_u = ks->nodes;
     b.chk_u = ks->chk;
     cudaStream_t s = slot.stream;
