@@ -112,6 +112,19 @@ void plan_dedup(Batch& b) {
     b.max_uniq = (uint32_t)(tpk * b.num_keys);
 }
 
+void use_keyset(Batch& b, const hs_keyset& ks) {
+    b.resident = true;
+    b.num_keys = ks.num_keys;
+    b.keys = ks.kb;
+    b.ck = ks.ck;
+    if (!ks.layers) return;
+    b.cached = true;
+    b.dedup_layer = ks.first_layer;
+    b.cache_tpk = ks.tpk;
+    b.nodes_u = ks.nodes;
+    b.chk_u = ks.chk;
+}
+
 // Every scratch region of a batch, in carve order (256-byte aligned each).
 static constexpr int kRegions = 14;
 static void scratch_layout(const Batch& b, const SetInfo& s, size_t sz[kRegions], int* n) {
@@ -486,19 +499,13 @@ static hs_status run_batch(const hs_keyset* ks, bool verify, hs_params p, const 
     b.num_keys = num_keys;
     b.count = count;
     b.status = d->status;
-    b.ck = verify ? 0u : (ks ? ks->ck : chain_checkpoint_stride(p));
+    b.ck = verify ? 0u : chain_checkpoint_stride(p);
     b.split = !verify && tree_split(p, count);
     b.msg_warp = msg_warp(p, count);
     b.verify = verify;
     b.walk = verify && verify_walk(p, count);
-    if (ks && ks->layers) {
-        b.dedup_layer = ks->first_layer;
-        b.cached = true;
-        b.cache_tpk = ks->tpk;
-    } else if (!verify) {
-        plan_dedup(b);
-    }
-    b.resident = ks != nullptr;
+    if (ks) use_keyset(b, *ks);
+    if (!verify && !b.cached) plan_dedup(b);
     size_t scratch = scratch_bytes(b);
     const size_t stage = (h_keys ? align256(key_bytes) : 0) + (h_idx ? align256((size_t)count * 4) : 0) +
                          (h_lens ? align256((size_t)count * 8) : 0) + (h_msgs ? align256(msg_total) : 0) +
@@ -514,11 +521,6 @@ static hs_status run_batch(const hs_keyset* ks, bool verify, hs_params p, const 
     }
     if (e != cudaSuccess) return cuda_fail(e, "cudaMallocFromPoolAsync(scratch)");
     carve_scratch(b, base);
-    if (ks) {
-        b.keys = ks->kb;
-        b.nodes_u = ks->nodes;
-        b.chk_u = ks->chk;
-    }
     Staging sg;
     sg.base = static_cast<char*>(base) + scratch;
 

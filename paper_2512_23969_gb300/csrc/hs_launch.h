@@ -8,6 +8,8 @@
 #include <cstdint>
 #include "hs_params.cuh"
 
+struct hs_keyset;             // resident keys, defined below
+
 namespace hs {
 
 // An XMSS tree built for several messages or as a key's root (kern_dedup.cuh).
@@ -95,6 +97,10 @@ uint32_t chain_checkpoint_stride(int pset);
 // (all 0 when sharing is off or not worth it).
 void plan_dedup(Batch& b);
 void drop_dedup(Batch& b);    // back to every message's own trees
+// The batch signs with a keyset's keys: its resident key blocks and, if it has
+// any, its prebuilt top layers.  Before carve_scratch, which gives the shared
+// trees of a keyset without layers their scratch (plan_dedup).
+void use_keyset(Batch& b, const hs_keyset& ks);
 size_t scratch_bytes(const Batch& b);
 
 // Scratch bytes for a batch (each region 256-byte aligned).

@@ -300,26 +300,16 @@ bool admit(ServerImpl& sv, Slot& slot, std::unique_lock<std::mutex>& lk) {
     Batch b{};
     b.pset = p;
     b.keys_in = ks->sk;
-    b.num_keys = ks->num_keys;
-    b.resident = true;                            // scratch holds no key blocks
-    b.keys = ks->kb;
     b.key_idx = reinterpret_cast<const uint32_t*>(d + o_kidx);
     b.msgs = msg_bytes ? d : d + o_lens;          // never read when all lengths are 0
     b.lens = reinterpret_cast<const uint64_t*>(d + o_lens);
     b.count = (uint32_t)count;
     b.sigs = d + o_sigs;
-    b.ck = ks->ck;
-    if (ks->layers) {                             // top layers from the keyset's cache
-        b.dedup_layer = ks->first_layer;
-        b.cached = true;
-        b.cache_tpk = ks->tpk;
-    }
+    use_keyset(b, *ks);                           // resident keys, top layers from its cache
     b.split = tree_split(p, (uint32_t)count);
     b.msg_warp = alone && msg_warp(p, (uint32_t)count);
     b.status = device_status_word();
     carve_scratch(b, d + o_scr);
-    b.nodes_u = ks->nodes;
-    b.chk_u = ks->chk;
     cudaStream_t s = slot.stream;
     cudaError_t e = cudaSuccess;
     if (injected) e = cudaErrorLaunchFailure;

@@ -95,6 +95,36 @@ int main() {
 """
 
 
+KEYSET = COMMON + r"""
+int main() {
+    uint32_t own_nodes = 0, own_chk = 0;
+    for (int p = 0; p < kNumSets; p++)
+        for (unsigned layers : {0u, 1u})
+            for (unsigned count : {3u, 4u, 5000u}) {
+                SetShape s;
+                set_shape(p, &s);
+                hs_keyset ks;
+                ks.pset = p; ks.num_keys = 2; ks.layers = layers; ks.first_layer = s.d - layers; ks.tpk = layers; ks.ck = 2;
+                ks.kb = reinterpret_cast<KeyBlock*>(64);
+                if (layers) { ks.nodes = &own_nodes; ks.chk = &own_chk; }      // null without layers
+                Batch b;
+                memset(&b, 0, sizeof b);
+                b.pset = p; b.count = count;
+                use_keyset(b, ks);
+                if (!b.cached) plan_dedup(b);
+                carve_scratch(b, reinterpret_cast<char*>(1 << 20));
+                const bool built = b.max_uniq != 0;
+                bool ok = b.keys == ks.kb && b.num_keys == 2 && b.ck == 2 && (b.cached != 0) == (layers != 0);
+                ok = ok && built == (layers == 0 && count >= 4);
+                if (built) ok = ok && b.desc && b.nodes_u > reinterpret_cast<uint32_t*>(1 << 20);
+                if (layers) ok = ok && b.nodes_u == &own_nodes && b.chk_u == &own_chk && b.dedup_layer == (unsigned)s.d - 1;
+                if (!ok) { printf("set %d layers %u count %u: nodes_u %p\n", p, layers, count, (void*)b.nodes_u); bad++; }
+            }
+    return bad != 0;
+}
+"""
+
+
 @pytest.fixture(scope="module")
 def run_cpp(tmp_path_factory):
     """Compile a program against the library's objects and run it."""
@@ -122,4 +152,11 @@ def run_cpp(tmp_path_factory):
 
 def test_layout_matches_size(run_cpp):
     r = run_cpp("layout", LAYOUT)
+    assert r.returncode == 0, r.stdout[-2000:]
+
+
+def test_keyset_trees_have_memory(run_cpp):
+    """The trees a keyset call builds itself live in its scratch; only a
+    keyset with prebuilt layers brings its own."""
+    r = run_cpp("keyset", KEYSET)
     assert r.returncode == 0, r.stdout[-2000:]
