@@ -335,9 +335,10 @@ __global__ void __launch_bounds__(T << P::A) fors_wide_kernel(const KeyBlock* __
 }
 
 // PK_FORS = T_k(FORS_ROOTS(layer 0, idx_tree, keypair idx_leaf), roots), 32
-// messages per block (kern_tl.cuh).
-template <class P>
-__global__ void __launch_bounds__(TlShape<P>::THREADS) fors_pk_kernel(const KeyBlock* __restrict__ keys,
+// messages per block (kern_tl.cuh); GROUP = false: a thread per message
+// alone, 128 per block.
+template <class P, bool GROUP>
+__global__ void __launch_bounds__(GROUP ? TlShape<P>::THREADS : 128) fors_pk_kernel(const KeyBlock* __restrict__ keys,
                                                                       const MsgInfo* __restrict__ infos,
                                                                       uint32_t count,
                                                                       uint32_t* __restrict__ fors_roots,
@@ -345,16 +346,16 @@ __global__ void __launch_bounds__(TlShape<P>::THREADS) fors_pk_kernel(const KeyB
                                                                       uint32_t guard) {
     if (blockIdx.x == guard) { wait_previous(); return; }
     constexpr int NW = P::NW;
-    __shared__ __align__(16) uint32_t smem[TlShape<P>::SMEM_WORDS];
-    const uint32_t m = blockIdx.x * 32 + (threadIdx.x & 31);
+    __shared__ __align__(16) uint32_t smem[GROUP ? TlShape<P>::SMEM_WORDS : 1];
+    const uint32_t m = GROUP ? blockIdx.x * 32 + (threadIdx.x & 31) : blockIdx.x * 128 + threadIdx.x;
     const uint32_t key = m < count ? infos[m].key : KEY_INVALID;
     const bool active = key != KEY_INVALID;
     const MsgInfo& info = infos[active ? m : 0];
     const KeyBlock& kb = keys[active ? key : 0];
     uint32_t out[NW];
-    tl_group<P, P::K>(P::BIG ? kb.ms512 : kb.ms256, make_adrs(0, info.idx_tree, T_FORS_ROOTS, info.idx_leaf, 0, 0),
-                      fors_roots + (size_t)m * P::K * NW, active, kb.pk_seed, smem, out);
-    if (threadIdx.x >= 32 || !active) return;
+    tl_group<P, P::K, GROUP>(P::BIG ? kb.ms512 : kb.ms256, make_adrs(0, info.idx_tree, T_FORS_ROOTS, info.idx_leaf, 0, 0),
+                             fors_roots + (size_t)m * P::K * NW, active, kb.pk_seed, smem, out);
+    if ((GROUP && threadIdx.x >= 32) || !active) return;
 #pragma unroll
     for (int w = 0; w < NW; w++) pk_fors[(size_t)m * NW + w] = out[w];
 }

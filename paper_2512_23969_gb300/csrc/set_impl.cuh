@@ -93,9 +93,19 @@ struct SetImpl {
         return launch_beside(b.beside, fors_wide_kernel<P, fors_pol<P>(), T>, (uint32_t)((trees + T - 1) / T), T << P::A,
                              s, (const KeyBlock*)b.keys, (const MsgInfo*)b.infos, b.count, b.sigs, b.fors_roots, 1u);
     }
+    // T_k has no climbs behind it, so its groups pay a little beyond what the
+    // SMs hold at once (robust sets: no further, the mask is hashed by the
+    // group's warps in turn).  Measured on GB300, groups / a thread per message
+    // (us): 128f 24352 messages 37 / 43, 32768 45 / 47, 65536 74 / 68, 131072
+    // 131 / 109; 192f 24352 59 / 78, 49152 109 / 102; 256f 24352 82 / 100,
+    // 49152 150 / 137; robust-256f 24352 263 / 242.
     static cudaError_t fors_pk(const Batch& b, cudaStream_t s) {
-        return launch_beside(b.beside, fors_pk_kernel<P>, (b.count + 31) / 32, TlShape<P>::THREADS, s,
-                             (const KeyBlock*)b.keys, (const MsgInfo*)b.infos, b.count, b.fors_roots, b.pk_fors);
+        const uint32_t G = (b.count + 31) / 32;
+        if (G <= (P::ROBUST ? kTlGroupsPerSm : 7u) * (uint32_t)sm_count())
+            return launch_beside(b.beside, fors_pk_kernel<P, true>, G, TlShape<P>::THREADS, s, (const KeyBlock*)b.keys,
+                                 (const MsgInfo*)b.infos, b.count, b.fors_roots, b.pk_fors);
+        return launch_beside(b.beside, fors_pk_kernel<P, false>, (b.count + 127) / 128, 128u, s, (const KeyBlock*)b.keys,
+                             (const MsgInfo*)b.infos, b.count, b.fors_roots, b.pk_fors);
     }
     template <int MINB, int POL = tree_pol<P>(), int ILP = 1>
     static cudaError_t tree(const Batch& b, BesideFn beside, cudaStream_t s) {
