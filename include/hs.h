@@ -408,9 +408,11 @@ hs_status hs_server_inject_launch_failures(hs_server *s, uint32_t n);
  * and copies every message's auth path and root from them.  Signatures are
  * byte-identical either way; nothing is kept from one call to the next
  * (128f, 16384 messages over 16 keys: 9360 trees in place of 65536, about
- * 15 % of the call).  Extra scratch per shared tree: its nodes and the
- * checkpoints of all its leaves; where that cannot be allocated the batch
- * is signed without sharing.
+ * 15 % of the call).  Extra scratch per shared tree: its nodes and, at the f
+ * sets, the checkpoints of all its leaves (stride 2: 36 KB per tree at 128f,
+ * 79 KB at 192f, 275 KB at 256f; 16 KB, 24 KB and 16 KB of nodes alone at
+ * 128s, 192s and 256s); where that cannot be allocated the batch is signed
+ * without sharing.
  */
 hs_status hs_set_tree_sharing(int on);
 

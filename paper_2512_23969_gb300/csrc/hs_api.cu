@@ -125,6 +125,12 @@ void use_keyset(Batch& b, const hs_keyset& ks) {
     b.chk_u = ks.chk;
 }
 
+// Checkpoint stride of the trees built for several messages: none for the
+// wide trees (2^h' = 256 or 512 leaves).  Checkpoints of every leaf are 2.3 MB
+// per 128s tree (16384 messages over 16 keys: 18 GB) to save WOTS+_Sign half
+// of one signed chain in 512 of a tree's.
+static uint32_t shared_ck(const Batch& b, const SetInfo& s) { return s.leaves > 32 ? 0u : b.ck; }
+
 // Every scratch region of a batch, in carve order (256-byte aligned each).
 static constexpr int kRegions = 14;
 static void scratch_layout(const Batch& b, const SetInfo& s, size_t sz[kRegions], int* n) {
@@ -144,8 +150,9 @@ static void scratch_layout(const Batch& b, const SetInfo& s, size_t sz[kRegions]
                        : (b.split ? (cnt * own + mu) * s.leaves * s.len * nw * 4 : 0);
     sz[i++] = b.dedup_layer ? cnt * (s.d - b.dedup_layer) * 4 : 0;   // mj_id
     sz[i++] = mu * sizeof(DedupDesc);                                // desc
+    const uint32_t ck_u = shared_ck(b, s);
     sz[i++] = mu * 2 * s.leaves * nw * 4 +                           // nodes_u, then chk_u
-              (b.ck ? mu * s.leaves * s.len * (16 / b.ck) * nw * 4 : 0);
+              (ck_u ? mu * s.leaves * s.len * (16 / ck_u) * nw * 4 : 0);
     sz[i++] = s.leaves > 32 ? cnt * s.d * s.leaves * nw * 4 : 0;     // leafv
     sz[i++] = !b.verify ? 0                                          // vends, or vcnt, vsitem, vorder
               : b.walk ? cnt * s.d * s.len * 16 * nw * 4
@@ -202,7 +209,7 @@ size_t carve_scratch(Batch& b, void* base) {
     if (b.cached) return total;       // nodes_u / chk_u belong to the keyset
     b.desc = b.max_uniq ? reinterpret_cast<DedupDesc*>(r[10]) : nullptr;
     b.nodes_u = b.max_uniq ? reinterpret_cast<uint32_t*>(r[11]) : nullptr;
-    b.chk_u = (b.max_uniq && b.ck) ? b.nodes_u + (size_t)b.max_uniq * 2 * s.leaves * (s.n / 4) : nullptr;
+    b.chk_u = (b.max_uniq && shared_ck(b, s)) ? b.nodes_u + (size_t)b.max_uniq * 2 * s.leaves * (s.n / 4) : nullptr;
     return total;
 }
 

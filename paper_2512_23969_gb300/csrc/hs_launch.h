@@ -52,15 +52,16 @@ struct Batch {
     uint32_t* leafv;          // wide trees (2^h' > 32): leaves, count * D * 2^h' * NW words
     // shared layers dedup_layer .. D-1 (dedup_layer == 0: none, every message
     // builds all its layers): their trees are built once per (key, layer,
-    // tree), all max_uniq = num_keys * cache_tpk of them, with every node and
-    // the checkpoints of every leaf, and each message copies its auth paths
+    // tree), all max_uniq = num_keys * cache_tpk of them, with every node and,
+    // but for wide trees, the checkpoints of every leaf, and each message
+    // copies its auth paths
     uint32_t dedup_layer;
     uint32_t cache_tpk;       // shared trees per key
     uint32_t max_uniq;        // shared trees built by this call (0 when cached)
     uint32_t* mj_id;          // count * (D - L): the tree of each (message, shared layer)
     DedupDesc* desc;          // max_uniq
     uint32_t* nodes_u;        // 2 * 2^h' * NW words per tree
-    uint32_t* chk_u;          // 2^h' * LEN * (16 / ck) * NW words per tree
+    uint32_t* chk_u;          // 2^h' * LEN * (16 / ck) * NW words per tree, or null
     bool cached;              // the trees come prebuilt from a keyset, which owns nodes_u / chk_u
     // FIPS 205 mode: FORS indices MSB first; prefix bytes hashed before
     // every message (0x00 || len(ctx) || ctx for pure signing; none = 0)

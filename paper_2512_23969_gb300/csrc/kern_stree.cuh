@@ -186,8 +186,8 @@ __global__ void __launch_bounds__(kMergeThreads) bmerkle_kernel(const KeyBlock* 
 // ---------------------------------------------------------------- shared / cached trees
 // Trees built for several messages (within a batch, keyset caches) for wide
 // trees: one thread per (tree, leaf) for the leaves, with the chain
-// checkpoints of every leaf, stored heap-ordered; then one block per tree
-// for the internal nodes.
+// checkpoints of every leaf where chk_u is not null (keyset caches), stored
+// heap-ordered; then one block per tree for the internal nodes.
 template <class P, int POL>
 __global__ void __launch_bounds__(128) wtree_leaf_kernel(const KeyBlock* __restrict__ keys,
                                                          const DedupDesc* __restrict__ desc, uint32_t ndesc,
@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(128) wtree_leaf_kernel(const KeyBlock* __restr
 #pragma unroll
     for (int w = 0; w < NW; w++) skseed[w] = kb.sk_seed[w];
     const Pipes<POL> pp(one);
-    uint32_t* mychk = ck ? chk_u + ((size_t)id * LV + l) * (size_t)P::LEN * (16u / ck) * NW : nullptr;
+    uint32_t* mychk = (ck != 0 && chk_u != nullptr) ? chk_u + ((size_t)id * LV + l) * (size_t)P::LEN * (16u / ck) * NW : nullptr;
     uint32_t node[NW];
     wots_leaf<P, POL>(ms256, msT, skseed, d.layer, d.tree, l, node, mychk, ck, pp, kb.pk_seed);
     uint32_t* tn = nodes + (size_t)id * 2 * LV * NW;

@@ -340,7 +340,7 @@ __device__ __forceinline__ bool chain_at(uint64_t gid, const MsgInfo* __restrict
     c.tree = d.tree;
     c.l = (uint32_t)((sid / LEN) % LV);
     c.i = (uint32_t)(sid % LEN);
-    if (per_chain != 0) c.chk = chk_u + (((size_t)id * LV + c.l) * (size_t)LEN + c.i) * per_chain * NW;
+    if (per_chain != 0 && chk_u != nullptr) c.chk = chk_u + (((size_t)id * LV + c.l) * (size_t)LEN + c.i) * per_chain * NW;
     return true;
 }
 

@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(256) wots_kernel(const KeyBlock* __restrict__ 
     for (int w = 0; w < 8; w++) ms256[w] = kb.ms256[w];
     const Pipes<POL> pp(one);
     uint32_t x[NW];
-    if (ck != 0) {
+    if (ck != 0 && (j < L || chk_u != nullptr)) {      // shared wide trees keep no checkpoints
         const uint32_t per_chain = 16u / ck;
         const uint32_t base = (digit / ck) * ck;
         // checkpoints of the message's own tree, or of the shared tree of

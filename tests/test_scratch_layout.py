@@ -125,6 +125,27 @@ int main() {
 """
 
 
+WIDE = COMMON + r"""
+int main() {
+    for (int p = 0; p < kNumSets; p++) {
+        SetShape s;
+        set_shape(p, &s);
+        if (s.leaves <= 32) continue;
+        for (unsigned keys : {1u, 16u}) {
+            Batch b;
+            memset(&b, 0, sizeof b);
+            b.pset = p; b.num_keys = keys; b.count = 16384; b.ck = 2;
+            const size_t own = scratch_bytes(b);
+            plan_dedup(b);
+            const size_t shared = scratch_bytes(b);
+            if (!b.max_uniq || shared > own + (own >> 2)) { printf("set %d, %u keys: %zu bytes alone, %zu shared\n", p, keys, own, shared); bad++; }
+        }
+    }
+    return bad != 0;
+}
+"""
+
+
 @pytest.fixture(scope="module")
 def run_cpp(tmp_path_factory):
     """Compile a program against the library's objects and run it."""
@@ -159,4 +180,12 @@ def test_keyset_trees_have_memory(run_cpp):
     """The trees a keyset call builds itself live in its scratch; only a
     keyset with prebuilt layers brings its own."""
     r = run_cpp("keyset", KEYSET)
+    assert r.returncode == 0, r.stdout[-2000:]
+
+
+def test_sharing_wide_trees_adds_little_memory(run_cpp):
+    """16384 messages of an s set with shared top layers: at most a quarter
+    more scratch than with every message's own trees (a checkpoint of every
+    chain of every leaf of those trees would be 18 GB and more)."""
+    r = run_cpp("wide", WIDE)
     assert r.returncode == 0, r.stdout[-2000:]
