@@ -44,9 +44,13 @@ std::atomic<int> g_ck_default{2};
 // batch size below which it runs chain-parallel (chain-parallel / per leaf,
 // ms: 128f 1024 messages 5.84 / 5.87, 2048 11.63 / 11.12; 192f 256 2.54 /
 // 2.71, 1024 9.99 / 8.88; 256f 32 0.76 / 1.27, 64 1.46 / 1.26), and above that
-// the cost model's coefficients (split_faster below).
-constexpr int kSplitDefault[kNumSets] = {1024, 256, 64, 0, 16, 16, 0, 16384, 16384, 16384, 256, 256, 256,
-                                         16384, 16384, 16384};
+// the cost model's coefficients (split_faster below).  At the SHAKE and robust
+// f sets the chain-parallel form is ahead at every size measured (TREE_Sign,
+// ms: shake-256f 4096 226 / 232, 8192 437 / 442; robust-256f 4096 193 / 215),
+// so there the line bounds its scratch: the chain ends (98, 215 and 583 KB a
+// message) stay at 2.4 GB or less.
+constexpr int kSplitDefault[kNumSets] = {1024, 256, 64, 0, 16, 16, 0, 16384, 8192, 4096, 256, 256, 256,
+                                         16384, 8192, 4096};
 constexpr int kStepUsDefault[kNumSets] = {637, 958, 1262, 0, 655, 1015, 1300, 2379, 3510, 4615, 2414, 3534, 4635,
                                           2379, 3606, 6405};
 constexpr int kSplitNsDefault[kNumSets] = {5741, 9833, 22514, 0, 116992, 197938, 167196, 20966, 30673, 62918,

@@ -146,6 +146,21 @@ int main() {
 """
 
 
+ENDS = COMMON + r"""
+int main() {
+    for (int p = 0; p < kNumSets; p++) {
+        const int below = tune_get(p, 2);                    // no tuned cache: the default line
+        if (below <= 1) continue;
+        SetShape s;
+        set_shape(p, &s);
+        const double ends = (below - 1.0) * s.d * s.leaves * (2 * s.n + 3) * s.n;
+        if (ends > 2.5e9) { printf("set %d: %.2f GB of chain ends at %d messages\n", p, ends / 1e9, below - 1); bad++; }
+    }
+    return bad != 0;
+}
+"""
+
+
 @pytest.fixture(scope="module")
 def run_cpp(tmp_path_factory):
     """Compile a program against the library's objects and run it."""
@@ -188,4 +203,9 @@ def test_sharing_wide_trees_adds_little_memory(run_cpp):
     more scratch than with every message's own trees (a checkpoint of every
     chain of every leaf of those trees would be 18 GB and more)."""
     r = run_cpp("wide", WIDE)
+    assert r.returncode == 0, r.stdout[-2000:]
+
+
+def test_default_forms_bound_the_chain_ends(run_cpp):
+    r = run_cpp("ends", ENDS)
     assert r.returncode == 0, r.stdout[-2000:]
