@@ -275,7 +275,7 @@ cudaError_t launch_prep(const Batch& b, bool verify, cudaStream_t s) {
     return e == cudaSuccess ? launch_message(c, verify, s) : e;
 }
 cudaError_t launch_sign_trees(const Batch& b, cudaStream_t s) {
-    if (!can_overlap(s)) {
+    if (b.crowded || !can_overlap(s)) {
         cudaError_t e = launch_fors(b, s);
         if (e == cudaSuccess) e = launch_fors_pk(b, s);
         return e == cudaSuccess ? launch_tree(b, s) : e;

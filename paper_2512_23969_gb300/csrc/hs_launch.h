@@ -75,6 +75,11 @@ struct Batch {
     // message and FORS launches: start beside the previous launch of the
     // stream instead of behind it (launch_prep, launch_sign_trees)
     bool beside;
+    // other batches run beside this one (the server): without the forms that
+    // shorten a small batch alone at the others' cost -- T_l by groups,
+    // launches beside each other, FORS_Sign a thread per leaf above 2 trees
+    // per SM
+    bool crowded;
 };
 
 // Called by the TREE_Sign launchers behind their first launch (stage 0) and
@@ -195,7 +200,7 @@ bool can_overlap(cudaStream_t s);
 cudaError_t launch_prep(const Batch& b, bool verify, cudaStream_t s);
 // FORS_Sign, T_k and TREE_Sign of a batch on one stream, the FORS stages
 // beside TREE_Sign (independent given the digest) unless the stream is being
-// captured.
+// captured or the batch is crowded.
 cudaError_t launch_sign_trees(const Batch& b, cudaStream_t s);
 cudaError_t launch_wots(const Batch& b, cudaStream_t s);
 // Whether a verification of 'count' signatures takes the form for few

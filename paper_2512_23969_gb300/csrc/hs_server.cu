@@ -234,12 +234,12 @@ bool admit(ServerImpl& sv, Slot& slot, std::unique_lock<std::mutex>& lk) {
     size_t pending_all = 0;
     for (int q = 0; q < kNumSets; q++) pending_all += sv.pending[q].size();
     const size_t share = std::max<size_t>(kMinShare, pending_all / sv.cfg.max_inflight);
-    // The message stage's warp form (a warp per message) only for a batch
-    // that has the GPU to itself: it shortens a small batch's serial message
-    // hashing when the GPU is otherwise idle, but in a server whose batches
-    // overlap it measured worse at high load (the serving mix at 85k
-    // requests/s: p99 17.5-18.0 ms with it, 11.6-12.2 ms without; at 75k
-    // 4.3 vs 4.6 ms).
+    // The forms that shorten a small batch on an otherwise idle GPU only for
+    // a batch that has it to itself: they take warps and issue slots from
+    // batches beside it.  Measured on GB300, the serving mix, with and without
+    // them there: the message stage's warp form at 85k requests/s p99
+    // 17.5-18.0 and 11.6-12.2 ms; the forms of Batch::crowded p50 / p99 at 76k
+    // 3.9 / 6.4 and 2.96 / 5.2 ms, at 84k 10.2 / 15.8 and 6.1 / 11.6 ms.
     bool alone = true;
     for (const Slot& o : sv.slots) alone = alone && (&o == &slot || !o.busy);
     // take requests while the cumulative need fits what the arenas could give
@@ -307,6 +307,7 @@ bool admit(ServerImpl& sv, Slot& slot, std::unique_lock<std::mutex>& lk) {
     use_keyset(b, *ks);                           // resident keys, top layers from its cache
     b.split = tree_split(p, (uint32_t)count);
     b.msg_warp = alone && msg_warp(p, (uint32_t)count);
+    b.crowded = !alone;
     b.status = device_status_word();
     carve_scratch(b, d + o_scr);
     cudaStream_t s = slot.stream;

@@ -83,10 +83,14 @@ struct SetImpl {
     // upper levels, so at a = 8 / 9 it pays for a few trees per SM only:
     // measured on GB300, 256f 1 message 215 -> 61 us, 96 messages 632 -> 987;
     // 192f 123 -> 47 and 360 -> 397; at a = 6 (128f) the blocks are small,
-    // 30 -> 20 us and 76 -> 65.
+    // 30 -> 20 us and 76 -> 65.  Beside other batches (crowded) the line lies
+    // at 2 trees per SM at every set: serving mix, p50 at 20k / 40k / 60k / 76k
+    // requests/s 0.55 / 0.85 / 1.48 / 2.96 ms; without a line 0.55 / 0.85 /
+    // 1.51 / 3.04, never a thread per leaf 0.64 / 0.94 / 1.42 / 2.94.
     static cudaError_t fors_widest(const Batch& b, cudaStream_t s) {
         constexpr int T = P::A < 7 ? 1 << (7 - P::A) : 1;          // trees per block: at least 128 threads
         const uint64_t trees = (uint64_t)b.count * P::K;
+        if (b.crowded && trees > (uint64_t)sm_count() * 2) return fors<32>(b, s);
         if constexpr (P::A >= 8) {
             if (trees > (uint64_t)sm_count() * (P::A == 8 ? 6 : 4)) return fors<32>(b, s);
         }
@@ -101,7 +105,7 @@ struct SetImpl {
     // 49152 150 / 137; robust-256f 24352 263 / 242.
     static cudaError_t fors_pk(const Batch& b, cudaStream_t s) {
         const uint32_t G = (b.count + 31) / 32;
-        if (G <= (P::ROBUST ? kTlGroupsPerSm : 7u) * (uint32_t)sm_count())
+        if (!b.crowded && G <= (P::ROBUST ? kTlGroupsPerSm : 7u) * (uint32_t)sm_count())
             return launch_beside(b.beside, fors_pk_kernel<P, true>, G, TlShape<P>::THREADS, s, (const KeyBlock*)b.keys,
                                  (const MsgInfo*)b.infos, b.count, b.fors_roots, b.pk_fors);
         return launch_beside(b.beside, fors_pk_kernel<P, false>, (b.count + 127) / 128, 128u, s, (const KeyBlock*)b.keys,
@@ -213,7 +217,7 @@ struct SetImpl {
         cudaError_t e = cudaGetLastError();
         if (e == cudaSuccess && beside) e = beside(*b, 0, s);
         if (e != cudaSuccess) return e;
-        const bool group = tl_groups_pay((own + 31) / 32 + (shared + 31) / 32);
+        const bool group = !(b && b->crowded) && tl_groups_pay((own + 31) / 32 + (shared + 31) / 32);
         const uint32_t per = group ? 32 : 128, TL = group ? TlShape<P>::THREADS : 128;
         const uint32_t G = (uint32_t)((own + per - 1) / per + (shared + per - 1) / per);
         if constexpr (kWide) {
