@@ -155,14 +155,15 @@ int sig_bytes_of(int p) {
     return set_shape(p, &sh) ? sh.sig : 0;
 }
 
-// Bytes a batch needs from each arena.
-struct Need { size_t dev, host; };
+// Bytes a batch needs from each arena, and the TREE_Sign form they are for
+// (the tuning knobs may change at any time: the form is chosen once).
+struct Need { size_t dev, host; bool split; };
 Need batch_need(int pset, size_t count, size_t msg_bytes, const hs_keyset* ks) {
     const size_t sig = (size_t)count * sig_bytes_of(pset);
     Need n;
     n.host = al256(msg_bytes) + al256(count * 8) + al256(count * 4) + al256(sig);
-    n.dev = n.host + al256(scratch_bytes(pset, 0, (uint32_t)count, ks->ck, tree_split(pset, (uint32_t)count),
-                                         ks->layers ? ks->first_layer : 0));
+    n.split = tree_split(pset, (uint32_t)count);
+    n.dev = n.host + al256(scratch_bytes(pset, 0, (uint32_t)count, ks->ck, n.split, ks->layers ? ks->first_layer : 0));
     return n;
 }
 
@@ -307,7 +308,7 @@ bool admit(ServerImpl& sv, Slot& slot, std::unique_lock<std::mutex>& lk) {
     b.count = (uint32_t)count;
     b.sigs = d + o_sigs;
     use_keyset(b, *ks);                           // resident keys, top layers from its cache
-    b.split = tree_split(p, (uint32_t)count);
+    b.split = need.split;
     b.msg_warp = alone && msg_warp(p, (uint32_t)count);
     b.crowded = !alone;
     b.status = device_status_word();

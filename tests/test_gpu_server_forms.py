@@ -35,3 +35,32 @@ def test_overlapping_batches(hs, sets, layers, max_batch):
             srv.wait(rid)
             assert out.tobytes() == work[ps][2][i].tobytes(), (ps, i)
         assert srv.stats()["max_inflight_batches"] >= 2      # batches ran beside each other
+
+
+def test_form_changed_while_serving(hs):
+    """Tuning knobs may change at any time: a batch's scratch and its
+    TREE_Sign form come from one look at them."""
+    import threading
+    from paper_2512_23969_gb300 import autotune
+    wl = inputs.make("128f", 64, num_keys=3, lengths=("uniform", 0, 100), seed=540, key_mode="random")
+    sk = hs.hs_keygen("128f", _dev(wl.seeds))[1]
+    ref = hs.hs_sign_batch("128f", sk, _dev(wl.msgs), _dev(wl.lens), key_idx=_dev(wl.key_idx)).cpu().numpy()
+    saved, stop = autotune.get("128f", "tree_split_below"), threading.Event()
+
+    def toggle():
+        while not stop.is_set():
+            for v in (0, 1 << 20):
+                autotune.set("128f", "tree_split_below", v)
+    t = threading.Thread(target=toggle)
+    t.start()
+    try:
+        with hs.Server({"128f": sk}, max_inflight=4, max_batch=16, mem_budget=64 << 20) as srv:
+            for _ in range(4):
+                reqs = [srv.submit("128f", int(wl.key_idx[i]), wl.message(i)) for i in range(64)]
+                for i, (rid, out) in enumerate(reqs):
+                    srv.wait(rid)
+                    assert out.tobytes() == ref[i].tobytes(), i
+    finally:
+        stop.set()
+        t.join()
+        autotune.set("128f", "tree_split_below", saved)
