@@ -21,6 +21,7 @@
 #include <cstring>
 #include <mutex>
 #include <vector>
+#include "graph_scratch.h"
 #include "hs_launch.h"
 #include "../../include/hs.h"
 
@@ -41,8 +42,7 @@ struct MixedDev {
     // whose batches and launch choices equal the last graph's relaunches it
     // as it is.  Every graph launch waits for the previous one (gdone):
     // they share the buffer.
-    void* gscratch = nullptr;
-    size_t gcap = 0;
+    GraphScratch gscratch;
     cudaEvent_t gdone = nullptr;
     cudaEvent_t gin = nullptr;          // the caller's stream up to the call
     cudaStream_t glaunch = nullptr;     // graph launches (idle between calls)
@@ -136,6 +136,27 @@ cudaError_t launch_graph(MixedDev& d, cudaStream_t origin) {
     return e;
 }
 
+// The device memory of the kept graph's scratch.
+struct DeviceMem {
+    MixedDev& d;
+    cudaError_t err = cudaSuccess;      // of the last allocation
+    bool alloc(void** p, size_t n) {
+        err = cudaMalloc(p, n);
+        if (err != cudaSuccess) cudaGetLastError();
+        return err == cudaSuccess;
+    }
+    void release(void* p) {
+        if (d.gdone_valid) cudaEventSynchronize(d.gdone);
+        cudaFree(p);
+        d.last_bs.clear();              // the old graph points into the old buffer
+    }
+    size_t avail() {
+        size_t f = 0, t = 0;
+        if (cudaMemGetInfo(&f, &t) != cudaSuccess) cudaGetLastError();
+        return f;
+    }
+};
+
 // Enqueue every job's stage DAG (fork from / join into 'origin').
 cudaError_t enqueue_jobs(MixedDev& d, std::vector<Batch>& bs, cudaStream_t origin) {
     cudaError_t e = cudaEventRecord(d.fork, origin);
@@ -213,33 +234,35 @@ HS_API hs_status hs_sign_mixed(const hs_sign_job* jobs, uint32_t njobs, int use_
     uint32_t* status = device_status_word();
     if (!status) return mx_fail(HS_ECUDA, "hs_sign_mixed: device state unavailable");
     std::lock_guard<std::mutex> lk(d->mu);
-    void* base = nullptr;
-    auto reserve = [&]() -> cudaError_t {
-        if (!use_graph) return pool_alloc(&base, total, s);
-        if (total <= d->gcap) return cudaSuccess;
-        if (d->gdone_valid) cudaEventSynchronize(d->gdone);   // grow the graph's fixed scratch
-        cudaFree(d->gscratch);
-        d->gscratch = nullptr;
-        d->gcap = 0;
-        d->last_bs.clear();                   // the old graph points into the old buffer
-        const cudaError_t ea = cudaMalloc(&d->gscratch, total);
-        if (ea == cudaSuccess) d->gcap = total;
-        return ea;
+    // without shared trees and chain ends, which are extra scratch
+    std::vector<Batch> lean = bs;
+    std::vector<size_t> lean_off;
+    size_t lean_total = 0;
+    for (Batch& b : lean) {
+        drop_dedup(b);
+        b.split = false;
+        lean_off.push_back(lean_total);
+        lean_total += scratch_bytes(b);
+    }
+    auto use_lean = [&] {
+        bs = lean;
+        off = lean_off;
+        total = lean_total;
     };
-    cudaError_t e = reserve();
-    if (e == cudaErrorMemoryAllocation) {     // shared trees and chain ends are extra scratch: without them
-        bool any = false;
-        total = 0;
-        for (size_t j = 0; j < bs.size(); j++) {
-            any = any || bs[j].max_uniq != 0 || bs[j].split;
-            drop_dedup(bs[j]);
-            bs[j].split = false;
-            off[j] = total;
-            total += scratch_bytes(bs[j]);
-        }
-        if (any) {
+    void* base = nullptr;
+    cudaError_t e = cudaSuccess;
+    if (use_graph) {
+        DeviceMem mem{*d};
+        const Layout l = reserve_graph_scratch(d->gscratch, total, lean_total, mem);
+        if (l == Layout::lean) use_lean();
+        e = l == Layout::none ? mem.err : cudaSuccess;
+        base = d->gscratch.p;
+    } else {
+        e = pool_alloc(&base, total, s);
+        if (e == cudaErrorMemoryAllocation && lean_total < total) {
             cudaGetLastError();
-            e = reserve();
+            use_lean();
+            e = pool_alloc(&base, total, s);
         }
     }
     if (e != cudaSuccess) {
@@ -248,7 +271,6 @@ HS_API hs_status hs_sign_mixed(const hs_sign_job* jobs, uint32_t njobs, int use_
         snprintf(buf, sizeof(buf), "hs_sign_mixed: scratch of %zu bytes: %s", total, cudaGetErrorString(e));
         return mx_fail(e == cudaErrorMemoryAllocation ? HS_ENOMEM : HS_ECUDA, buf);
     }
-    if (use_graph) base = d->gscratch;
     for (size_t j = 0; j < bs.size(); j++) {
         bs[j].status = status;
         carve_scratch(bs[j], static_cast<char*>(base) + off[j]);
