@@ -258,12 +258,13 @@ static cudaError_t tree_beside(const Batch& b, BesideFn beside, cudaStream_t s) 
     return e;
 }
 cudaError_t launch_tree(const Batch& b, cudaStream_t s) { return tree_beside(b, nullptr, s); }
-bool can_overlap(cudaStream_t s) {
+static bool capturing(cudaStream_t s) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) == cudaSuccess) return cap == cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
     cudaGetLastError();
-    return false;
+    return true;
 }
+bool can_overlap(cudaStream_t s) { return !capturing(s); }
 cudaError_t launch_prep(const Batch& b, bool verify, cudaStream_t s) {
     cudaError_t e = launch_keyprep(b, verify, s);
     if (needs_offsets(b) || !can_overlap(s)) {
@@ -297,7 +298,11 @@ cudaError_t launch_verify(const Batch& b, cudaStream_t s) {
 cudaError_t launch_keygen(int pset, const uint8_t* seeds, uint32_t count, uint8_t* pk, uint8_t* sk,
                           cudaStream_t s) {
     const SetOps* o = set_ops(pset);
-    return o ? o->keygen(seeds, count, pk, sk, keygen_split(pset, count), s) : cudaErrorInvalidValue;
+    // The chain-parallel form allocates.  In a captured graph that would be
+    // an allocation node, and such a graph cannot be instantiated twice, cloned
+    // or used as a child: there a thread per leaf (at the f sets one kernel and
+    // no allocation).
+    return o ? o->keygen(seeds, count, pk, sk, keygen_split(pset, count) && !capturing(s), s) : cudaErrorInvalidValue;
 }
 
 }  // namespace hs
