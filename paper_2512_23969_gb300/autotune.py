@@ -40,8 +40,12 @@ DEFAULT_COUNTS = {"128f": 16384, "192f": 8192, "256f": 8192, "toy": 4096, "128s"
 # (down to a few messages: the per-leaf form is latency-bound below one wave
 # of threads, so its time hardly falls with the batch while the chain-
 # parallel form's does)
-SPLIT_COUNTS = {"f": (8, 16, 32, 64, 128, 256, 1024, 2048, 4096, 8192), "s": (8, 16, 32, 64, 128, 256),
-                "shake-f": (8, 16, 32, 64, 128, 256, 1024, 2048, 4096, 8192), "shake-s": (4, 8, 16, 32, 64, 128)}
+SPLIT_COUNTS = {"f": (8, 16, 32, 64, 128, 192, 256, 384, 512, 768, 1024, 1536, 2048, 4096, 8192),
+                "s": (8, 16, 32, 64, 128, 256),
+                "shake-f": (8, 16, 32, 64, 128, 256, 512, 1024, 2048, 4096, 8192), "shake-s": (4, 8, 16, 32, 64, 128)}
+# device memory for the chain ends of the chain-parallel form: the line it is
+# tuned to keeps a call at or below this
+SPLIT_BYTES = 2.5e9
 
 
 def _family(ps):
@@ -132,6 +136,19 @@ def _shape(ps):
     return n[base]
 
 
+def form_line(counts, a, b):
+    """The batch size below which form a is taken, from its times and form b's
+    at the sizes measured: the one that gives away least, as the sum over the
+    sizes of how much slower the form taken is than the other (one past a
+    measured size; twice the last one if a is taken throughout, 0 if nowhere).
+    The forms' times are no smooth curves -- TREE_Sign's per-leaf time is a
+    staircase -- so a single late win does not carry the line over losses."""
+    def cost(i):
+        return sum(max(0.0, x / y - 1.0 if j < i else y / x - 1.0) for j, (x, y) in enumerate(zip(a, b)))
+    best = min(range(len(counts) + 1), key=lambda i: (cost(i), i))
+    return 0 if best == 0 else (2 * counts[-1] if best == len(counts) else counts[best - 1] + 1)
+
+
 def tune_tree_costs(ps, reps=3, verbose=True):
     """The per-leaf TREE_Sign time of one step (a warp per SM sub-partition:
     the per-leaf time grows in whole steps) and the chain-parallel time per
@@ -164,10 +181,13 @@ def tune_tree_costs(ps, reps=3, verbose=True):
 
 def tune_split(ps, counts=None, reps=3, verbose=True):
     """Batch size below which the chain-parallel TREE_Sign is faster: time
-    the TREE stage in both forms at growing batch sizes."""
-    counts = counts or SPLIT_COUNTS[_family(ps)]
+    the TREE stage in both forms at growing batch sizes whose chain ends stay
+    within SPLIT_BYTES."""
+    n = hs.N_BYTES[ps]
+    d, leaves = _shape(ps)
+    limit = int(SPLIT_BYTES // (d * leaves * (2 * n + 3) * n))
+    counts = [c for c in counts or SPLIT_COUNTS[_family(ps)] if c <= limit]
     rows = {}
-    below = 0
     set(ps, "tree_step_us", 0)                 # forms forced by the threshold alone while timing
     set(ps, "tree_split_ns", 0)
     for count in counts:
@@ -180,13 +200,12 @@ def tune_split(ps, counts=None, reps=3, verbose=True):
         if verbose:
             print("tune %s tree form at %d: split %.3f ms, per-leaf %.3f ms" % (ps, count, ms["split"], ms["leaf"]),
                   flush=True)
-        if ms["split"] < ms["leaf"]:
-            below = count * 2 if count == counts[-1] else counts[counts.index(count) + 1]
+    below = min(form_line(counts, [rows[str(c)]["split"] for c in counts], [rows[str(c)]["leaf"] for c in counts]), limit + 1)
     set(ps, "tree_split_below", below)
     return {"best": below, "ms": rows}
 
 
-MSG_COUNTS = (64, 128, 256, 512, 1024, 2048, 4096)
+MSG_COUNTS = (64, 128, 256, 512, 768, 1024, 1536, 2048, 3072, 4096)
 
 
 def tune_msg_warp(ps, counts=MSG_COUNTS, reps=3, verbose=True):
@@ -199,7 +218,6 @@ def tune_msg_warp(ps, counts=MSG_COUNTS, reps=3, verbose=True):
         set(ps, "msg_warp_below", 0)
         return {"best": 0}
     rows = {}
-    below = 0
     for count in counts:
         wl = inputs.make(ps, count, 16, ("loguniform", 16, 4096), 4343 + count)
         pk, sk = hs.hs_keygen(ps, torch.from_numpy(wl.seeds).cuda())
@@ -213,8 +231,7 @@ def tune_msg_warp(ps, counts=MSG_COUNTS, reps=3, verbose=True):
         if verbose:
             print("tune %s message form at %d: warp %.4f ms, thread %.4f ms" % (ps, count, ms["warp"], ms["thread"]),
                   flush=True)
-        if ms["warp"] < ms["thread"]:
-            below = count * 2 if count == counts[-1] else counts[counts.index(count) + 1]
+    below = form_line(counts, [rows[str(c)]["warp"] for c in counts], [rows[str(c)]["thread"] for c in counts])
     set(ps, "msg_warp_below", below)
     return {"best": below, "ms": rows, "lengths": "log-uniform 16 B - 4 KB, 16 keys"}
 
