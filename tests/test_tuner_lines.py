@@ -1,7 +1,7 @@
 """The tuner's lines between two forms, with made-up times in place of the
 GPU's: the line gives away least over the sizes measured, and lies just behind
 a size, not at the next one; the chain-parallel form's line keeps its chain
-ends within SPLIT_BYTES."""
+ends within SPLIT_BYTES; the batches timed share no trees."""
 import pytest
 
 from paper_2512_23969_gb300 import autotune, hs
@@ -39,3 +39,17 @@ def test_split_line_bounds_the_chain_ends(monkeypatch, ps):
     d, leaves = autotune._shape(ps)
     n = hs.N_BYTES[ps]
     assert 0 < (best - 1) * d * leaves * (2 * n + 3) * n <= autotune.SPLIT_BYTES
+
+
+@pytest.mark.parametrize("count", [1, 3, 110, 16384])
+def test_tuner_batches_share_no_trees(monkeypatch, count):
+    """Trees are shared from two messages per key on (plan_dedup)."""
+    class Made(Exception):
+        pass
+
+    def make(ps, n, num_keys, *a, **k):
+        assert n == count and 2 * num_keys > n
+        raise Made
+    monkeypatch.setattr(autotune.inputs, "make", make)
+    with pytest.raises(Made):
+        autotune._batch("128f", count)
