@@ -126,9 +126,33 @@ def _ctx_alu(nw):
     return 6 * 10 + 4 * 4 + (8 if nw == 4 else 0)
 
 
+def _keccak_hash_alu(n, payload):
+    """ALU ops of a SHAKE hash of one permutation (PRF, F, H) over PK.seed,
+    the address and payload bytes.  Its first round folds the zero lanes (a
+    column's zero lanes share theta's term), its last computes the n / 8
+    output lanes alone, from the lanes 2 further; 22 rounds run in full."""
+    data, out = (n + 32 + payload) // 8, n // 8
+    first = 10 + 48 + 50 + 1                       # rotations of the parities, rho, chi, iota (half a constant)
+    for pad in (data, 16):                         # the pad bits: one half of each of these lanes
+        for x in range(5):
+            t = sum(i < data or i == pad for i in range(x, 25, 5))
+            first += t // 2 + t + (t < 5)          # parity, theta's lanes, the zero lanes' shared term
+    need = min(out + 2, 5)
+    last = 20 + 2 * need + 2 * need + 2 * (need - 1) + 2 * out + 2
+    return first + 22 * (ALU_KECCAK // 24) + last
+
+
 def exec_alu_per_sig(ps, stage):
     """ALU-pipe ops per signature of a stage as the kernels execute them
-    (the roofline's work basis); the SHAKE sets execute the full basis."""
+    (the roofline's work basis)."""
+    if ps in KECCAK_WORK and stage in ("tree", "fors"):
+        n, d, hp, a, k, length = SET_SHAPE[ps[len("shake-"):]]
+        if stage == "tree":
+            f, h = d * (1 << hp) * length * 16, d * ((1 << hp) - 1)
+        else:
+            f, h = k * (2 << a), k * ((1 << a) - 1)
+        return f * _keccak_hash_alu(n, n) + h * _keccak_hash_alu(n, 2 * n) + \
+            (KECCAK_WORK[ps][stage] - f - h) * ALU_KECCAK
     if ps in KECCAK_WORK:
         return alu_ops_per_sig(ps, stage)
     n, d, hp, a, k, length = SET_SHAPE[ps]
