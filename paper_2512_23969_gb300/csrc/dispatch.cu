@@ -57,13 +57,17 @@ constexpr int kSplitNsDefault[kNumSets] = {5741, 9833, 22514, 0, 116992, 197938,
                                            425882, 626482, 473714, 11576, 17815, 54806};
 constexpr int kStrides[] = {0, 1, 2, 4, 8};
 // Default batch size below which the message stage runs a warp per message
-// (SHA-2 sets; the SHAKE sets always run a thread per message).  Measured on
-// GB300, thread / warp form with its prefix sum (us): 128f, 1024 messages of
-// 32 bytes 86 / 37, of 32 - 1024 bytes 171 / 90, 2048 89 / 56 and 169 / 160,
-// 4096 89 / 87 and 168 / 256; 256f 1024 133 / 68 and 244 / 132, 2048 134 /
-// 117 and 240 / 229.
-constexpr int kMsgWarpDefault[kNumSets] = {2048, 2048, 2048, 2048, 2048, 2048, 2048, 0, 0, 0, 0, 0, 0,
-                                           2048, 2048, 2048};
+// (SHA-2 sets; the SHAKE sets always run a thread per message): up to two warps
+// per SM sub-partition, 1216 messages.  The warp form is then ahead at every
+// length; with a third, long messages wait for issue slots (every lane runs
+// the rounds), while the thread form leaves most of them free.  Measured on GB300, whole calls of
+// messages of one length, thread / warp form (ms): 128f 32 bytes 1200 messages
+// 6.53 / 6.43, 2047 10.69 / 10.66; 64 KB 1200 10.86 / 10.24, 1500 12.46 /
+// 13.36, 2047 15.29 / 18.06 (verification 4.15 / 5.51); 192f 64 KB 1200 17.4 /
+// 16.7, 1500 20.3 / 21.6, 2047 25.7 / 29.3; 256f 64 KB 1200 31.0 / 30.3, 2047
+// 47.9 / 51.6.
+constexpr int kMsgWarpDefault[kNumSets] = {1217, 1217, 1217, 1217, 1217, 1217, 1217, 0, 0, 0, 0, 0, 0,
+                                           1217, 1217, 1217};
 bool is_shake(int pset) { return pset >= 7 && pset <= 12; }
 }
 
@@ -110,7 +114,7 @@ int tune_options(int pset, int knob, int32_t* values, int max) {
     case 5: for (int v : kStrides) buf[n++] = v; break;
     case 8:                             // suggestions: any value works (SHAKE sets: 0 only)
         if (is_shake(pset)) buf[n++] = 0;
-        else for (int v : {0, 64, 256, 512, 1024, 2048, 4096}) buf[n++] = v;
+        else for (int v : {0, 64, 256, 512, 1024, 1217, 2048, 4096}) buf[n++] = v;
         break;
     default:                            // 6, 7: measured coefficients, any value >= 0
         buf[n++] = 0;

@@ -2,9 +2,15 @@
 GPU's: the line gives away least over the sizes measured, and lies just behind
 a size, not at the next one; the chain-parallel form's line keeps its chain
 ends within SPLIT_BYTES; the batches timed share no trees."""
+import os
+import subprocess
+import sys
+
 import pytest
 
 from paper_2512_23969_gb300 import autotune, hs
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 def test_form_line():
@@ -53,3 +59,16 @@ def test_tuner_batches_share_no_trees(monkeypatch, count):
     monkeypatch.setattr(autotune.inputs, "make", make)
     with pytest.raises(Made):
         autotune._batch("128f", count)
+
+
+def test_default_message_line_is_two_warps_per_sub_partition():
+    """Beyond two warps per SM sub-partition (8 per SM, 152 SMs) the message
+    stage's warp form is behind at long messages: the default line stops
+    there.  (A process of its own: other tests set the knob.)"""
+    out = subprocess.run([sys.executable, "-c", "from paper_2512_23969_gb300 import autotune, hs\n"
+                          "for ps in hs.PARAMS: print(ps, autotune.get(ps, 'msg_warp_below'))"],
+                         cwd=ROOT, check=True, capture_output=True, text=True).stdout
+    lines = dict(row.split() for row in out.splitlines())
+    assert len(lines) == len(hs.PARAMS)
+    for ps, line in lines.items():
+        assert int(line) == 0 if ps.startswith("shake") else 0 < int(line) <= 8 * 152 + 1, ps
