@@ -47,7 +47,7 @@ std::atomic<int> g_ck_default{2};
 // the cost model's coefficients (split_faster below).  At the SHAKE and robust
 // f sets the chain-parallel form is ahead at every size measured (TREE_Sign,
 // ms: shake-256f 4096 226 / 232, 8192 437 / 442; robust-256f 4096 193 / 215),
-// so there the line bounds its scratch: the chain ends (98, 215 and 583 KB a
+// but for 0.3 - 2.5 % at robust-192f between 512 and 2048 messages, so there the line bounds its scratch: the chain ends (98, 215 and 583 KB a
 // message) stay at 2.4 GB or less.
 constexpr int kSplitDefault[kNumSets] = {1024, 256, 64, 0, 16, 16, 0, 16384, 8192, 4096, 256, 256, 256,
                                          16384, 8192, 4096};

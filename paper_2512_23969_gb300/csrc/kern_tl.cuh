@@ -16,14 +16,16 @@
 // Rows are [round][lane], so every shared-memory access of a warp is one
 // conflict-free row.  CH: the producers' time per block is below the rounds'
 // at both widths; two at SHA-256 halve the barriers (32 KB of shared memory),
-// one at SHA-512 keeps the two buffers at 40 KB, four groups to an SM.
+// one at SHA-512 keeps the two buffers at 40 KB, five groups to an SM.
 #pragma once
 #include <cuda_runtime.h>
 #include "hs_common.cuh"
 
 namespace hs {
 
-// Groups of 32 items an SM holds (40 KB of shared memory each at SHA-512).
+// Groups of 32 items per SM up to which a launch runs by groups: as many as an
+// SM holds at SHA-512 (40 KB of shared memory each); the same line at SHA-256
+// (32 KB, one more would fit).
 constexpr uint32_t kTlGroupsPerSm = 5;
 
 template <class P>
