@@ -182,8 +182,11 @@ int fors_lanes(int pset, uint32_t count);
 
 cudaError_t launch_keyprep(const Batch& b, bool from_pk, cudaStream_t s);
 // The message stage's warp form sums the lengths before its message itself
-// up to this many messages (1024 read 8 KB a warp at most; measured 7 us less
-// per call than the prefix sum's launch); above, and in the thread form, the
+// up to this many messages: the last warp reads all of them, 32 KB from L2, so
+// the sum grows with the count while the prefix sum's launch hardly does.
+// Verification on GB300 with the sum / with that launch, us: 128f 1024
+// messages 1324 / 1329, 4096 2568 / 2573; 192f 256 1801 / 1812, 2048 2865 /
+// 2877, 4096 3953 / 3956.  Above, and in the thread form, the
 // offsets come from a prefix sum.
 constexpr uint32_t kSumLens = 4096;
 inline bool needs_offsets(const Batch& b) { return !b.msg_warp || b.count > kSumLens; }
